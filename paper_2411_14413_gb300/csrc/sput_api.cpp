@@ -103,7 +103,9 @@ struct sput_scene {
     std::vector<DevPrim> dprims;
     std::vector<DevGeom> dgeoms;
     // cell masks of the surface test (empty: a geometry has more than 64 primitives)
-    std::vector<unsigned long long> cell_masks;
+    std::vector<uint32_t> cell_masks;
+    int cell_words = 1;
+    double mean_inv_lambda = 0.0;  // 1/mm, of 1 eV atoms, mean over the instances' particles
     double cell_lo[3] = {0, 0, 0}, cell_h = 0.0;
     int cell_n[3] = {0, 0, 0};
     std::vector<DevCathode> dcath;
@@ -306,71 +308,109 @@ static sput_status pack_instances(sput_scene* S)
         S->prefix[i + 1] = S->prefix[i] + I.n_particles;
     }
     S->n_tickets = S->prefix.back();
+    // mean inverse free path of 1 eV atoms, for the choice of the surface test (cell_masks_pay)
+    S->mean_inv_lambda = 0.0;
+    for (size_t i = 0; i < S->dinst.size(); ++i) {
+        const DevPair& pr = S->dpairs[S->dinst[i].pair];
+        const double v = 1.0 / std::sqrt((double)S->dcath[S->dinst[i].cathode].E_per_v2);
+        const double x = std::min(std::log(1.0 + v * pr.inv_s) * pr.w_inv_h, (double)pr.n_w);
+        const int j = std::min((int)x, pr.n_w - 1);
+        const float4 c = S->wtab[pr.K_off + j];
+        const double t = x - j, K = c.x + t * (c.y + t * (c.z + t * c.w));
+        const double inv_lambda = S->dinst[i].ng14 * (S->physics.gas_motion == SPUT_GAS_THERMAL ? K / v : K);
+        S->mean_inv_lambda += inv_lambda * ((double)S->dinst[i].n / (double)std::max(1ull, S->n_tickets));
+    }
     return SPUT_OK;
 }
 
-// Cell masks of the surface test.  A uniform grid of cubic cells (edge h, 32 along the
-// chamber's longest side) covers the chamber box.  For every geometry, cell c and
-// r = 1, 2, a 64-bit mask holds the local primitives that a flight of length at most
-// r h starting in c can reach: those whose bounding sphere meets the block of cells
-// within r of c (grown by a margin for FP32 rounding), and the chamber box when that
-// block touches a wall.  A flight that long cannot leave the block, so testing the
-// mask's primitives in ascending order finds the same nearest hit, with the same
-// tie-breaking, as testing every primitive.  Geometries of more than 64 primitives
-// leave the masks out (every flight tests every primitive).
+// Whether the surface test by cell masks is the faster one.  It replaces the loop over the
+// geometry's primitives by a mask lookup per piece of a flight and a round of (lane,
+// primitive) pairs, so it needs several primitives and flights that are short against the
+// chamber (edge / lambda, primitives).  Measured on a GB300, loop -> masks in ms:
+//   16 primitives, 4e6 atoms:   0 Pa 0.28 -> 0.34, 0.05 Pa 0.77 -> 0.82, 0.1 Pa (edge/lambda 6)
+//                               1.32 -> 1.31, 0.2 Pa 2.44 -> 2.18, 0.5 Pa 9.0 -> 7.8
+//   64 primitives, 4e6 atoms:   0 Pa 0.73 -> 0.78, 0.05 Pa (edge/lambda 3) 1.51 -> 1.13,
+//                               0.5 Pa 12.9 -> 5.9
+//   7 primitives, 4e6 atoms:    0.2 Pa 2.25 -> 2.43, 0.5 Pa 10.6 -> 10.9, 1 Pa 44.4 -> 44.4
+static bool cell_masks_pay(const sput_scene* S)
+{
+    double edge = 0.0;
+    for (int a = 0; a < 3; ++a) edge = std::max(edge, S->chamber.box_hi[a] - S->chamber.box_lo[a]);
+    return S->max_prims > 8 && S->max_prims * edge * S->mean_inv_lambda > 96.0;
+}
+
+// Distance from a point to a primitive's surface (not to a chamber box's).
+static double surface_distance(const DevPrim& Q, const double* x)
+{
+    const double w[3] = {x[0] - Q.cx, x[1] - Q.cy, x[2] - Q.cz};
+    const double a = w[0] * Q.ux + w[1] * Q.uy + w[2] * Q.uz;
+    if (Q.kind == SPUT_PRIM_CYLINDER) {
+        const double r = std::sqrt(std::max(0.0, dot3(w, w) - a * a));
+        const double da = std::max(0.0, std::fabs(a) - Q.p1), dr = r - Q.p0;
+        return std::sqrt(da * da + dr * dr);
+    }
+    const double z = w[0] * Q.nx + w[1] * Q.ny + w[2] * Q.nz;
+    const double b = w[0] * Q.vx + w[1] * Q.vy + w[2] * Q.vz;
+    if (Q.kind == SPUT_PRIM_RECT) {
+        const double da = std::max(0.0, std::fabs(a) - Q.p0), db = std::max(0.0, std::fabs(b) - Q.p1);
+        return std::sqrt(z * z + da * da + db * db);
+    }
+    const double r = std::sqrt(a * a + b * b);
+    const double dr = std::max(0.0, std::max(r - Q.p1, Q.p0 - r));
+    return std::sqrt(z * z + dr * dr);
+}
+
+// Cell masks of the surface test (nearest_hit_masks).  A uniform grid of cubic cells
+// covers the chamber box.  For every geometry, cell c and level k, a mask holds the local
+// primitives whose surface lies within r 2^k of a point of c: distance to the cell's centre
+// at most half its diagonal + r 2^k, grown by 0.1 mm, far above the FP32 rounding of
+// positions, midpoints and hit distances (1e-4 mm at these sizes).  Chamber boxes are left
+// out: the flight tests the walls by themselves.  A geometry of more than 64 primitives, or
+// without chamber walls, leaves the masks out (every flight tests every primitive).
 static void build_cell_masks(sput_scene* S)
 {
     S->cell_masks.clear();
     S->cell_h = 0.0;
-    for (const sput_geometry& g : S->geoms)
-        if (g.prim_count > 64) return;
+    S->cell_words = 1;
+    for (size_t g = 0; g < S->geoms.size(); ++g) {
+        if (S->geoms[g].prim_count > 64 || S->dgeoms[g].box() < 0) return;
+        if (S->geoms[g].prim_count > 32) S->cell_words = 2;
+    }
     double ext[3], emax = 0.0;
     for (int a = 0; a < 3; ++a) {
         S->cell_lo[a] = S->chamber.box_lo[a];
         ext[a] = S->chamber.box_hi[a] - S->chamber.box_lo[a];
         emax = std::max(emax, ext[a]);
     }
-    const double h = emax / 32.0;
-    for (int a = 0; a < 3; ++a) S->cell_n[a] = std::max(1, std::min(32, (int)std::ceil(ext[a] / h - 1e-9)));
-    S->cell_h = h;
-    const int nx = S->cell_n[0], ny = S->cell_n[1], nz = S->cell_n[2];
-    const size_t ncell = (size_t)nx * ny * nz;
-    const double margin = 1e-3 * h + 1e-3;
-    S->cell_masks.assign(S->geoms.size() * ncell * 2, 0ull);
+    // kCellGrid cells along the longest side (0.5 or 1 MB per geometry here), half as many when
+    // the geometries' masks would take more than 256 MB
+    size_t ncell = 0;
+    for (int n = kCellGrid; n >= kCellGrid / 2; n /= 2) {
+        S->cell_h = emax / n;
+        for (int a = 0; a < 3; ++a) S->cell_n[a] = std::max(1, std::min(n, (int)std::ceil(ext[a] / S->cell_h - 1e-9)));
+        ncell = (size_t)S->cell_n[0] * S->cell_n[1] * S->cell_n[2];
+        if (S->geoms.size() * ncell * kCellLevels * S->cell_words * sizeof(uint32_t) <= ((size_t)256 << 20)) break;
+    }
+    const double h = S->cell_h, half_diag = 0.5 * std::sqrt(3.0) * h;
+    double reach[kCellLevels];
+    for (int k = 0; k < kCellLevels; ++k) reach[k] = half_diag + std::ldexp(h / 8.0, k) + 0.1;
+    const size_t words = ncell * kCellLevels * S->cell_words;
+    S->cell_masks.assign(S->geoms.size() * words, 0u);
     for (size_t g = 0; g < S->geoms.size(); ++g) {
         const sput_geometry& G = S->geoms[g];
-        S->dgeoms[g].cell_base = (int)(g * ncell * 2);
-        for (int iz = 0; iz < nz; ++iz)
-            for (int iy = 0; iy < ny; ++iy)
-                for (int ix = 0; ix < nx; ++ix) {
-                    const int idx[3] = {ix, iy, iz};
-                    for (int r = 1; r <= 2; ++r) {
-                        double blo[3], bhi[3];
-                        bool wall = false;
-                        for (int a = 0; a < 3; ++a) {
-                            blo[a] = S->cell_lo[a] + (idx[a] - r) * h - margin;
-                            bhi[a] = S->cell_lo[a] + (idx[a] + 1 + r) * h + margin;
-                            if (idx[a] - r <= 0 || idx[a] + r >= S->cell_n[a] - 1) wall = true;
-                        }
-                        unsigned long long m = 0ull;
-                        for (int li = 0; li < G.prim_count; ++li) {
-                            const DevPrim& Q = S->dprims[G.prim_begin + li];
-                            bool in;
-                            if (Q.kind == SPUT_PRIM_BOX) {
-                                in = wall;
-                            } else {
-                                const double c[3] = {Q.bx, Q.by, Q.bz};
-                                double d2 = 0.0;
-                                for (int a = 0; a < 3; ++a) {
-                                    const double d = std::max(0.0, std::max(blo[a] - c[a], c[a] - bhi[a]));
-                                    d2 += d * d;
-                                }
-                                const double rr = (double)Q.br + margin;
-                                in = d2 <= rr * rr;
-                            }
-                            if (in) m |= 1ull << li;
-                        }
-                        S->cell_masks[(size_t)S->dgeoms[g].cell_base + 2 * (((size_t)iz * ny + iy) * nx + ix) + (r - 1)] = m;
+        S->dgeoms[g].cell_base = (int)(g * words);
+        uint32_t* m = &S->cell_masks[g * words];
+        for (int iz = 0; iz < S->cell_n[2]; ++iz)
+            for (int iy = 0; iy < S->cell_n[1]; ++iy)
+                for (int ix = 0; ix < S->cell_n[0]; ++ix, m += kCellLevels * S->cell_words) {
+                    const double x[3] = {S->cell_lo[0] + (ix + 0.5) * h, S->cell_lo[1] + (iy + 0.5) * h,
+                                         S->cell_lo[2] + (iz + 0.5) * h};
+                    for (int li = 0; li < G.prim_count; ++li) {
+                        const DevPrim& Q = S->dprims[G.prim_begin + li];
+                        if (Q.kind == SPUT_PRIM_BOX) continue;
+                        const double d = surface_distance(Q, x);
+                        for (int k = kCellLevels - 1; k >= 0 && d <= reach[k]; --k)
+                            m[k * S->cell_words + (li >> 5)] |= 1u << (li & 31);
                     }
                 }
     }
@@ -454,7 +494,12 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     S->dgeoms.resize(S->geoms.size());
     S->max_prims = 0;
     for (size_t g = 0; g < S->geoms.size(); ++g) {
-        S->dgeoms[g] = DevGeom{S->geoms[g].prim_begin, S->geoms[g].prim_count, S->geoms[g].substrate, -1};
+        const sput_geometry& G = S->geoms[g];
+        int box = 0;
+        for (int li = G.prim_count - 1; li >= 0; --li)
+            if (S->prims[G.prim_begin + li].kind == SPUT_PRIM_BOX) box = li + 1;
+        // (a block's shared memory holds fewer than 3000 primitives, so both indices fit 16 bits)
+        S->dgeoms[g] = DevGeom{G.prim_begin, G.prim_count, (G.substrate & 0xffff) | (box & 0x7fff) << 16, -1};
         S->max_prims = std::max(S->max_prims, S->geoms[g].prim_count);
     }
     build_cell_masks(S);
@@ -629,7 +674,7 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     S->off_lt = place(sizeof(float) * S->lt.size());
     const ChiTable* ct = hard ? nullptr : &chi_table(S->physics.chi_min);
     S->off_chi = place(ct ? sizeof(float4) * ct->cells.size() : 0);
-    S->off_cell = place(sizeof(unsigned long long) * S->cell_masks.size());
+    S->off_cell = place(sizeof(uint32_t) * S->cell_masks.size());
     S->blob_bytes = o;
     cudaError_t e = cudaMalloc(&S->d_blob, S->blob_bytes);
     if (e != cudaSuccess) {
@@ -652,7 +697,7 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     put(S->off_rt, S->rt.data(), sizeof(float4) * S->rt.size());
     put(S->off_lt, S->lt.data(), sizeof(float) * S->lt.size());
     if (ct) put(S->off_chi, ct->cells.data(), sizeof(float4) * ct->cells.size());
-    put(S->off_cell, S->cell_masks.data(), sizeof(unsigned long long) * S->cell_masks.size());
+    put(S->off_cell, S->cell_masks.data(), sizeof(uint32_t) * S->cell_masks.size());
     e = cudaMemcpy(S->d_blob, h.data(), S->blob_bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMallocHost(&S->h_scratch, 64);
     if (e == cudaSuccess) e = cudaEventCreate(&S->ev0);
@@ -677,14 +722,15 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     p.rt_tab = reinterpret_cast<const float4*>(S->d_blob + S->off_rt);
     p.lt_tab = reinterpret_cast<const float*>(S->d_blob + S->off_lt);
     p.chi_tab = ct ? reinterpret_cast<const float4*>(S->d_blob + S->off_chi) : nullptr;
-    p.cell_mask = S->cell_masks.empty() ? nullptr
-                                        : reinterpret_cast<const unsigned long long*>(S->d_blob + S->off_cell);
+    p.cell_mask = S->cell_masks.empty() ? nullptr : reinterpret_cast<const uint32_t*>(S->d_blob + S->off_cell);
+    p.cell_words = S->cell_words;
     for (int a = 0; a < 3; ++a) {
         p.cell_lo[a] = (float)S->cell_lo[a];
         p.cell_n[a] = S->cell_n[a];
     }
-    p.cell_h = (float)S->cell_h;
     p.cell_inv_h = S->cell_h > 0.0 ? (float)(1.0 / S->cell_h) : 0.0f;
+    p.cell_inv_r = 8.0f * p.cell_inv_h;
+    p.cell_inv_seg = 0.25f * p.cell_inv_h;
     p.n_prims = (int)S->dprims.size();
     p.n_geoms = (int)S->dgeoms.size();
     p.n_pairs = (int)S->dpairs.size();
@@ -734,6 +780,8 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     p.smem_counters = (size_t)p.n_inst * (p.max_prims + 1) <= 12288 ? 1 : 0;
     if (transport_smem_bytes(p) > S->smem_optin) {
         p.smem_counters = 0;
+        // the masks' pair lists give way to the scene's own tables
+        if (transport_smem_bytes(p) > S->smem_optin) p.cell_mask = nullptr;
         if (transport_smem_bytes(p) > S->smem_optin) {
             sput_scene_destroy(S);
             return fail(SPUT_ERR_UNSUPPORTED, "scene tables exceed the shared memory of one block");
@@ -865,9 +913,8 @@ sput_status run_impl(sput_scene* S, const sput_run_opts* opts, cudaStream_t stre
     p.smem_counters = (flags & SPUT_RUN_NO_SMEM_COUNTERS) ? 0 : S->smem_counters_fit;
     p.launch_at_cutoff = cutoff ? 1 : 0;
     p.inject_nonfinite = (opts->flags & SPUT_RUN_INJECT_NONFINITE) ? 1 : 0;
-    // the masked surface test pays where geometries have many primitives (see SPUT_RUN_CELL_MASKS)
-    const bool masks = (opts->flags & SPUT_RUN_CELL_MASKS) ||
-                       (!(opts->flags & SPUT_RUN_NO_CELL_MASKS) && S->max_prims > 32);
+    const bool masks =
+        (opts->flags & SPUT_RUN_CELL_MASKS) || (!(opts->flags & SPUT_RUN_NO_CELL_MASKS) && cell_masks_pay(S));
     if (!masks) p.cell_mask = nullptr;
 
     const TallySizes sz = tally_sizes(S);

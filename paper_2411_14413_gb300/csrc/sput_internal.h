@@ -70,8 +70,11 @@ struct alignas(16) DevPrim {
 };
 
 struct alignas(16) DevGeom {
-    int begin, count, substrate;
+    int begin, count;
+    int marks;      // substrate's local index | (local index + 1 of the first chamber box, 0: none) << 16
     int cell_base;  // offset of this geometry's cell masks in Params::cell_mask (-1: none)
+    __host__ __device__ int substrate() const { return marks & 0xffff; }
+    __host__ __device__ int box() const { return (marks >> 16) - 1; }
 };
 
 struct alignas(16) DevCathode {
@@ -140,11 +143,12 @@ struct Params {
     const float4* rt_tab;              // racetrack inverse-CDF pieces (2 rt_n per cathode)
     const float* lt_tab;               // joint launch-table CDFs (see DevCathode::lt_off)
     const float4* chi_tab;             // deflection table: kChiCells cells of 4 float4 (null: hard spheres)
-    // cell masks of the surface test (null: off): per geometry and cell of a uniform grid over
-    // the chamber, the local primitives a flight of length <= h (word 0) or <= 2 h (word 1)
-    // starting in the cell can reach
-    const unsigned long long* cell_mask;
-    float cell_lo[3], cell_h, cell_inv_h;
+    // cell masks of the surface test (null: off): per geometry, cell of a uniform grid over the
+    // chamber and level k, cell_words words with the local primitives (chamber boxes left out)
+    // that have a point within r 2^k of a point of the cell
+    const uint32_t* cell_mask;
+    int cell_words;
+    float cell_lo[3], cell_inv_h, cell_inv_r, cell_inv_seg;
     int cell_n[3];
     int n_prims, n_geoms, n_pairs, n_inst;
     int n_bm;
@@ -192,6 +196,13 @@ struct Params {
     float4 gm[kGMHalf];       // kGMNodes-point rule
     float4 gm_lo[kGMHalfLo];  // kGMNodesLo-point rule (ln eps < kGMLoLnEps)
 };
+
+// Cell masks: up to kCellGrid cells along the chamber's longest side (edge h), levels
+// r = h/8, h/4, ... 2 h; a flight is cut into pieces of at most 4 h (kCellMaxPieces of them:
+// enough for the diagonal of a cubic chamber).
+constexpr int kCellGrid = 32;
+constexpr int kCellLevels = 5;
+constexpr int kCellMaxPieces = 16;
 
 constexpr int kNumStats = 6;
 // rows of one SPUT_PROBE_TRACE record (launch state + 63 flights)

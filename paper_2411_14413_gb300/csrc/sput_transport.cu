@@ -405,19 +405,25 @@ __device__ void launch_state(const Params& P, const float4* rt_tab, uint32_t ins
 }
 
 // ------------------------------------------------------------- geometry
+// distance to the chamber walls from inside (0 behind a wall, infinite for a zero or NaN direction)
+__device__ __forceinline__ float hit_box(const Params& P, float px, float py, float pz, float dx, float dy, float dz)
+{
+    // approximate quotients (2 ulp): a hit distance needs no correctly rounded division
+    const float tx = dx > 0.0f ? __fdividef(P.box_hi[0] - px, dx)
+                               : (dx < 0.0f ? __fdividef(P.box_lo[0] - px, dx) : CUDART_INF_F);
+    const float ty = dy > 0.0f ? __fdividef(P.box_hi[1] - py, dy)
+                               : (dy < 0.0f ? __fdividef(P.box_lo[1] - py, dy) : CUDART_INF_F);
+    const float tz = dz > 0.0f ? __fdividef(P.box_hi[2] - pz, dz)
+                               : (dz < 0.0f ? __fdividef(P.box_lo[2] - pz, dz) : CUDART_INF_F);
+    return fmaxf(fminf(tx, fminf(ty, tz)), 0.0f);
+}
+
 __device__ __forceinline__ float hit_prim(const DevPrim& Q, const Params& P, float px, float py, float pz, float dx,
                                           float dy, float dz)
 {
     float t = CUDART_INF_F;
     if (Q.kind == SPUT_PRIM_BOX) {
-        // approximate quotients (2 ulp): a hit distance needs no correctly rounded division
-        const float tx = dx > 0.0f ? __fdividef(P.box_hi[0] - px, dx)
-                                   : (dx < 0.0f ? __fdividef(P.box_lo[0] - px, dx) : CUDART_INF_F);
-        const float ty = dy > 0.0f ? __fdividef(P.box_hi[1] - py, dy)
-                                   : (dy < 0.0f ? __fdividef(P.box_lo[1] - py, dy) : CUDART_INF_F);
-        const float tz = dz > 0.0f ? __fdividef(P.box_hi[2] - pz, dz)
-                                   : (dz < 0.0f ? __fdividef(P.box_lo[2] - pz, dz) : CUDART_INF_F);
-        t = fmaxf(fminf(tx, fminf(ty, tz)), 0.0f);
+        t = hit_box(P, px, py, pz, dx, dy, dz);
     } else if (Q.kind == SPUT_PRIM_CYLINDER) {
         const float wx = px - Q.cx, wy = py - Q.cy, wz = pz - Q.cz;
         const float wa = wx * Q.ux + wy * Q.uy + wz * Q.uz;
@@ -523,97 +529,187 @@ struct StepOut {
     float Gv;       // d ln K / d ln s at the flight's speed (temperature score only)
 };
 
-// Free flight k+1 of the atom in S and the surface test.  Landing: S keeps the
-// pre-flight position and out.t is the hit distance.  Otherwise the atom moves
-// to the collision point; w is the flight's Philox block (words 1 and 2, the
-// impact parameter and azimuth, are used by the collision; word 3 is unused).
-template <int kMode, bool kMasks>
-__device__ int flight_move(Lane& S, const Params& P, const TableView& T, const DevPrim* prims, const DevPair* pairs,
-                           StepOut& out, uint4& w)
+// Free flight k+1 of the atom in S: its Philox block w (word 0 the free path; words 1 and 2,
+// the impact parameter and azimuth, are used by the collision; word 3 is unused), the
+// inverse mean free path and the flight length.
+template <int kMode>
+__device__ void flight_begin(Lane& S, const Params& P, const TableView& T, const DevPair* pairs, StepOut& out,
+                             uint4& w, float& inv_lam, float& ell)
 {
     S.k += 1u;
-    out.attempts = 0;
-    out.nonfinite = 0;
-    out.prim = -1;
     w = philox(P, S.pid, stream_of(T, P, S.inst), S.k, 0u);
     const DevPair pr = pairs[S.pair];
     // inverse mean free path n_g <sigma g>/v (thermal) or n_g sigma(v) (gas at rest)
     const float Kv = wtab_eval(T, pr, pr.K_off, S.speed);
-    float inv_lam = P.gas_thermal ? S.ng14 * Kv / S.speed : S.ng14 * Kv;
+    inv_lam = P.gas_thermal ? S.ng14 * Kv / S.speed : S.ng14 * Kv;
     // diffusion shortcut: exponential steps of mean lambda_D, 1/lambda_D = n sigma_D
     if (kMode == kModeWalk && S.diff) inv_lam = S.ng14 * pr.sigma_D;
-    constexpr bool kScoreT = kMode == kModeScoreT;
-    const float ell = S.ng14 > 0.0f ? __fdividef(neg_log_fast(rn(w.x)), inv_lam) : CUDART_INF_F;
-    // temperature score: d ln(n_g K(v)/v)/dT = (-1 + G/2)/T with n_g = p/(k_B T), G = d ln K/d ln s
-    float aT = 0.0f;
-    if (kScoreT) {
+    ell = S.ng14 > 0.0f ? __fdividef(neg_log_fast(rn(w.x)), inv_lam) : CUDART_INF_F;
+    if (kMode == kModeScoreT) {
         // (this table stays in global memory: w_tab + G_off, read through L1)
         out.Gv = idx_ok(P.status, (long long)pr.G_off + pr.n_w - 1, P.n_w_all)
                      ? cubic_eval(P.w_tab + pr.G_off, pr.n_w, w_of(pr, S.speed) * pr.w_inv_h)
                      : 0.0f;
-        aT = (0.5f * out.Gv - 1.0f) * P.inv_T;
     }
+}
 
-    // surface test: nearest hit, ties to the lowest index; the emitting target
-    // is skipped on the first flight.  Every primitive whose bounding sphere lies
-    // within min(ell, best t) is tested (margin covers FP32 rounding): no hit
-    // beyond that can be the landing.
-    float tb = CUDART_INF_F;
-    int hb = -1;
-    // the emitting target is skipped on the first flight (read only then)
+// The emitting target's local index on the first flight (it is skipped then: the atom
+// leaves its plane; read only then), else -1.
+__device__ __forceinline__ int excluded_prim(const Lane& S, const Params& P)
+{
+    return S.k == 1u ? P.cath[P.inst[S.inst].cathode].target : -1;
+}
+
+// Nearest hit by a loop over the geometry's primitives, ties to the lowest index.  Every
+// primitive whose bounding sphere lies within min(ell, best t) is tested (margin covers
+// FP32 rounding): no hit beyond that can be the landing.
+__device__ __forceinline__ void nearest_hit_loop(const Lane& S, const Params& P, const TableView& T,
+                                                 const DevPrim* prims, float ell, float& tb, int& hb)
+{
     const DevGeom G = T.geoms[S.geom];
-    const int excl = S.k == 1u ? P.cath[P.inst[S.inst].cathode].target : -1;
-    if (!kMasks) {
-        for (int li = 0; li < G.count; ++li) {
-            if (li == excl) continue;
-            if (!idx_ok(P.status, G.begin + li, P.n_prims)) break;
-            const DevPrim& Q = prims[G.begin + li];
-            if (Q.kind != SPUT_PRIM_BOX) {
-                const float ex = Q.bx - S.px, ey = Q.by - S.py, ez = Q.bz - S.pz;
-                const float reach = fminf(ell, tb) * 1.0001f + Q.br + 1e-3f;
-                if (ex * ex + ey * ey + ez * ez > reach * reach) continue;
+    const int excl = excluded_prim(S, P);
+    for (int li = 0; li < G.count; ++li) {
+        if (li == excl) continue;
+        if (!idx_ok(P.status, G.begin + li, P.n_prims)) break;
+        const DevPrim& Q = prims[G.begin + li];
+        if (Q.kind != SPUT_PRIM_BOX) {
+            const float ex = Q.bx - S.px, ey = Q.by - S.py, ez = Q.bz - S.pz;
+            const float reach = fminf(ell, tb) * 1.0001f + Q.br + 1e-3f;
+            if (ex * ex + ey * ey + ez * ez > reach * reach) continue;
+        }
+        const float t = hit_prim(Q, P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
+        if (t < tb) {
+            tb = t;
+            hb = li;
+        }
+    }
+}
+
+// Nearest hit of every active lane by the cell masks, the whole warp together.
+//   * The chamber walls are tested first, so the flight is a segment of length
+//     L = min(ell, wall) inside the box.
+//   * It is cut into pieces of at most 4 cell edges (most flights are one piece).  All of a
+//     piece lies within R, half its length, of its centre: the mask of the centre's cell at
+//     the smallest level r 2^k >= R holds every primitive it can reach (usually none: most
+//     flights pass far from any surface).
+//   * The (lane, primitive) pairs of all lanes are tested 32 at a time, one per lane,
+//     whichever atom they belong to: a loop per lane would run as long as the busiest
+//     lane's, and a loop over the geometry runs each test for the few lanes near it.
+// A primitive outside the mask has no hit at t <= L, so the nearest hit and its tie-break
+// (lowest index) are those of the loop above.  kWords: 32-bit words of a mask.
+// The transport is bound by instruction issue, and the loop took 43 % (16 primitives, 0.5 Pa)
+// to 67 % (64 primitives, 3 Pa) of the kernel: a warp ran 9.2 of 16 primitives' tests per
+// step although 0.12 per atom cross the primitive at all.  Masks of the midpoint leave 13
+// pairs per warp and step (0.5 Pa), so one round does.  Measured loop -> masks (GB300):
+// quaternary 4e7 atoms 67.2 -> 58.8 ms, 64 primitives at 3 Pa 1e6 atoms 118 -> 59 ms, with the
+// diffusion shortcut 4e6 atoms 61.3 -> 24.7 ms.
+template <int kWords>
+__device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, const Params& P, const TableView& T,
+                                                  const DevPrim* prims, uint2* list, float ell, float& tb, int& hb)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned lo = 0u, hi = 0u;  // candidates 0..31 and 32..63
+    int begin = 0;
+    if (active) {
+        const DevGeom G = T.geoms[S.geom];
+        begin = G.begin;
+        const int box = G.box();  // a geometry with masks has one
+        tb = hit_box(P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
+        hb = tb < CUDART_INF_F ? box : -1;
+        const float L = fminf(ell, tb);
+        int pieces = min((int)(L * P.cell_inv_seg), kCellMaxPieces - 1) + 1;
+        const float R = 0.5f * __fdividef(L, (float)pieces);
+        // the smallest level: max(0, ceil(log2(R / r))) from the exponent bits
+        const int k = max(0, (int)((__float_as_uint(R * P.cell_inv_r) + 0x7fffffu) >> 23) - 127);
+        for (float c = R; pieces > 0; --pieces, c += 2.0f * R) {
+            const float mx = (fmaf(c, S.dx, S.px) - P.cell_lo[0]) * P.cell_inv_h;
+            const float my = (fmaf(c, S.dy, S.py) - P.cell_lo[1]) * P.cell_inv_h;
+            const float mz = (fmaf(c, S.dz, S.pz) - P.cell_lo[2]) * P.cell_inv_h;
+            if (k < kCellLevels && fminf(fminf(mx, my), mz) >= 0.0f && mx < (float)P.cell_n[0] &&
+                my < (float)P.cell_n[1] && mz < (float)P.cell_n[2]) {
+                const int cell = ((int)mz * P.cell_n[1] + (int)my) * P.cell_n[0] + (int)mx;
+                const uint32_t* m = P.cell_mask + G.cell_base + (cell * kCellLevels + k) * kWords;
+                if (kWords == 1) {
+                    lo |= __ldg(m);
+                } else {
+                    const uint2 m2 = __ldg(reinterpret_cast<const uint2*>(m));
+                    lo |= m2.x;
+                    hi |= m2.y;
+                }
+            } else {
+                // a centre outside the grid (FP32 rounding at a wall), or a flight that starts outside
+                lo = G.count >= 32 ? ~0u : (1u << G.count) - 1u;
+                if (kWords == 2) hi = G.count >= 64 ? ~0u : G.count > 32 ? (1u << (G.count - 32)) - 1u : 0u;
+                if (box < 32) lo &= ~(1u << box);
+                if (kWords == 2 && box >= 32) hi &= ~(1u << (box - 32));
             }
-            const float t = hit_prim(Q, P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
-            if (t < tb) {
+        }
+        const int excl = excluded_prim(S, P);
+        if (excl >= 0 && excl < 32) lo &= ~(1u << excl);
+        if (kWords == 2 && excl >= 32) hi &= ~(1u << (excl - 32));
+    }
+    const int n = __popc(lo) + (kWords == 2 ? __popc(hi) : 0);
+    if (!__any_sync(kFull, n != 0)) return;
+    // pos: exclusive prefix of n over the lanes, from the ballots of its bits
+    const unsigned lt = (1u << lane) - 1u;
+    int pos = 0, total = 0, bit = 0;
+    do {
+        const unsigned m = __ballot_sync(kFull, (n >> bit) & 1);
+        pos += __popc(m & lt) << bit;
+        total += __popc(m) << bit;
+        ++bit;
+    } while (__any_sync(kFull, n >> bit));
+    for (; total > 0; total -= 32, pos -= 32) {
+        // the lanes list their pairs of this round (positions 0..31)
+        const int first = pos;
+        while (pos < 32 && (kWords == 2 ? (lo | hi) : lo)) {
+            int li;
+            if (kWords == 1 || lo) {
+                li = __ffs(lo) - 1;
+                lo &= lo - 1u;
+            } else {
+                li = 31 + __ffs(hi);
+                hi &= hi - 1u;
+            }
+            list[pos++].x = (uint32_t)(begin + li) << 5 | (uint32_t)lane;
+        }
+        __syncwarp();
+        const bool mine = lane < total;
+        const uint32_t pr = mine ? list[lane].x : (uint32_t)lane;
+        const int src = (int)(pr & 31u);
+        const float px = __shfl_sync(kFull, S.px, src), py = __shfl_sync(kFull, S.py, src),
+                    pz = __shfl_sync(kFull, S.pz, src);
+        const float dx = __shfl_sync(kFull, S.dx, src), dy = __shfl_sync(kFull, S.dy, src),
+                    dz = __shfl_sync(kFull, S.dz, src);
+        if (mine)
+            list[lane].y = __float_as_uint(idx_ok(P.status, pr >> 5, P.n_prims)
+                                               ? hit_prim(prims[pr >> 5], P, px, py, pz, dx, dy, dz)
+                                               : CUDART_INF_F);
+        __syncwarp();
+        // and take their hits
+        for (int i = first; i < pos; ++i) {
+            const uint2 e = list[i];
+            const float t = __uint_as_float(e.y);
+            const int li = (int)(e.x >> 5) - begin;
+            if (t < tb || (t == tb && li < hb)) {
                 tb = t;
                 hb = li;
             }
         }
-    } else {
-        // candidates as 32-bit masks of local indices, visited in ascending order; a
-        // flight of length <= h (2 h) takes its cell's mask of the primitives it can
-        // reach, which leaves the result unchanged
-        unsigned long long near = ~0ull;
-        if (ell <= 2.0f * P.cell_h) {
-            const int ix = min(max((int)floorf((S.px - P.cell_lo[0]) * P.cell_inv_h), 0), P.cell_n[0] - 1);
-            const int iy = min(max((int)floorf((S.py - P.cell_lo[1]) * P.cell_inv_h), 0), P.cell_n[1] - 1);
-            const int iz = min(max((int)floorf((S.pz - P.cell_lo[2]) * P.cell_inv_h), 0), P.cell_n[2] - 1);
-            const int c = (iz * P.cell_n[1] + iy) * P.cell_n[0] + ix;
-            near = __ldg(P.cell_mask + G.cell_base + 2 * c + (ell <= P.cell_h ? 0 : 1));
-        }
-        for (int base = 0; base < G.count; base += 32) {
-            const int left = G.count - base;
-            unsigned mask = left >= 32 ? 0xffffffffu : ((1u << left) - 1u);
-            if (base < 64) mask &= (unsigned)(near >> base);
-            if (excl >= base && excl < base + 32) mask &= ~(1u << (excl - base));
-            while (mask) {
-                const int li = base + __ffs(mask) - 1;
-                mask &= mask - 1u;
-                if (!idx_ok(P.status, G.begin + li, P.n_prims)) break;
-                const DevPrim& Q = prims[G.begin + li];
-                if (Q.kind != SPUT_PRIM_BOX) {
-                    const float ex = Q.bx - S.px, ey = Q.by - S.py, ez = Q.bz - S.pz;
-                    const float reach = fminf(ell, tb) * 1.0001f + Q.br + 1e-3f;
-                    if (ex * ex + ey * ey + ez * ez > reach * reach) continue;
-                }
-                const float t = hit_prim(Q, P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
-                if (t < tb) {
-                    tb = t;
-                    hb = li;
-                }
-            }
-        }
+        __syncwarp();
     }
+}
+
+// The flight's end.  Landing: S keeps the pre-flight position and out.t is the hit
+// distance.  Otherwise the atom moves to the collision point.
+template <int kMode>
+__device__ int flight_end(Lane& S, const Params& P, StepOut& out, float inv_lam, float ell, float tb, int hb)
+{
+    constexpr bool kScoreT = kMode == kModeScoreT;
+    out.nonfinite = 0;
+    out.prim = -1;
+    // temperature score: d ln(n_g K(v)/v)/dT = (-1 + G/2)/T with n_g = p/(k_B T), G = d ln K/d ln s
+    const float aT = kScoreT ? (0.5f * out.Gv - 1.0f) * P.inv_T : 0.0f;
     if (hb >= 0 && tb <= ell) {
         S.score -= tb * inv_lam;
         if (kScoreT) S.scoreT -= aT * tb * inv_lam;
@@ -824,16 +920,23 @@ __device__ void scatter(Lane& S, const Params& P, const TableView& T, const DevP
 // One flight of every active lane of the warp (flight, surface test, then for
 // the lanes that collide: warp-wide partner sampling and the scattering).
 // Must be called by all 32 lanes together; inactive lanes return kStepNone.
-template <int kMode, bool kMasks>
+// kMasks: words of the surface test's cell masks (0: the counted loop); list: the warp's
+// 32 entries of shared memory for them.
+template <int kMode, int kMasks>
 __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const TableView& T, const DevPrim* prims,
-                                const DevPair* pairs, StepOut& out)
+                                const DevPair* pairs, uint2* list, StepOut& out)
 {
     uint4 w = make_uint4(0u, 0u, 0u, 0u);
     int res = kStepNone;
     out.attempts = 0;
     constexpr bool kScoreT = kMode == kModeScoreT;
     if (kScoreT) out.Gv = 0.0f;
-    if (active) res = flight_move<kMode, kMasks>(S, P, T, prims, pairs, out, w);
+    float inv_lam = 0.0f, ell = 0.0f, tb = CUDART_INF_F;
+    int hb = -1;
+    if (active) flight_begin<kMode>(S, P, T, pairs, out, w, inv_lam, ell);
+    if (kMasks) nearest_hit_masks<kMasks ? kMasks : 1>(active, S, P, T, prims, list, ell, tb, hb);
+    else if (active) nearest_hit_loop(S, P, T, prims, ell, tb, hb);
+    if (active) res = flight_end<kMode>(S, P, out, inv_lam, ell, tb, hb);
     // a thermalised atom (diffusion shortcut) turns isotropically at the end of its step
     const bool walk = kMode == kModeWalk && res == kStepCollided && S.diff;
     const bool coll = res == kStepCollided && !walk;
@@ -873,7 +976,7 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
 
 // ------------------------------------------------------------- kernel
 struct SmemLayout {
-    size_t prims, geoms, pairs, bm, prefix, xh, gm, stream, pool, queue, counters, total;
+    size_t prims, geoms, pairs, bm, prefix, xh, gm, stream, pool, queue, list, counters, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -902,6 +1005,8 @@ __host__ __device__ inline SmemLayout smem_layout(const Params& p)
     o = align16(o + sizeof(unsigned long long) * 4 * 8);
     L.queue = o;
     o = align16(o + sizeof(uint32_t) * kLaunchWords * 32 * 8);
+    L.list = o;
+    o = align16(o + (p.cell_mask ? sizeof(uint2) * 32 * 8 : 0));
     L.counters = o;
     o = align16(o + (p.smem_counters ? sizeof(unsigned int) * (size_t)p.n_inst * (p.max_prims + 1) : 0));
     L.total = o;
@@ -923,7 +1028,7 @@ __device__ __forceinline__ void copy16(void* dst, const void* src, size_t bytes)
 // few spills at 64 registers; the lane state is kept small for it (a geometry index
 // instead of the geometry's fields, the ticket recomputed from (instance, id), the
 // warp's ticket pool in shared memory).
-template <bool kCount64, int kMode, bool kMasks>
+template <bool kCount64, int kMode, int kMasks>
 __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -985,6 +1090,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     // and its queue of prepared launches: s_wpool[2] entries of kLaunchWords words
     unsigned long long* s_wpool = s_pool + 4 * (threadIdx.x >> 5);
     uint32_t* s_wqueue = s_queue + kLaunchWords * 32 * (threadIdx.x >> 5);
+    uint2* s_wlist = reinterpret_cast<uint2*>(smem + L.list) + 32 * (threadIdx.x >> 5);
     if (lane == 0) s_wpool[0] = s_wpool[1] = s_wpool[2] = 0ull;
     __syncwarp();
 
@@ -1074,7 +1180,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 
         // ---------------------------------------------------- one flight (all lanes together)
         StepOut so;
-        const int res = flight_step_warp<kMode, kMasks>(alive, S, P, T, s_prims, s_pairs, so);
+        const int res = flight_step_warp<kMode, kMasks>(alive, S, P, T, s_prims, s_pairs, s_wlist, so);
         c_att += so.attempts;
         if (res == kStepLanded) {
             // ------------------------------------------------ landing tally
@@ -1084,7 +1190,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
             int cell = -1;
             float cosang = 0.0f;
             const DevGeom G = s_geoms[S.geom];
-            if (hb == G.substrate) {
+            if (hb == G.substrate()) {
                 const DevPrim& Q = s_prims[G.begin + hb];
                 const float dn = S.dx * Q.nx + S.dy * Q.ny + S.dz * Q.nz;
                 if (dn < 0.0f) {
@@ -1227,11 +1333,10 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
         for (int r = 1; r < kTraceRows; ++r) {
             if (!__any_sync(kFull, running)) break;
             StepOut so;
+            // (the oracle's trace tests the counted loop; both surface tests give the same flights)
             const int status = P.E_switch > 0.0f
-                                   ? (P.cell_mask ? flight_step_warp<kModeWalk, true>(running, S, P, T, P.prims, P.pairs, so)
-                                                  : flight_step_warp<kModeWalk, false>(running, S, P, T, P.prims, P.pairs, so))
-                                   : (P.cell_mask ? flight_step_warp<kModePlain, true>(running, S, P, T, P.prims, P.pairs, so)
-                                                  : flight_step_warp<kModePlain, false>(running, S, P, T, P.prims, P.pairs, so));
+                                   ? flight_step_warp<kModeWalk, 0>(running, S, P, T, P.prims, P.pairs, nullptr, so)
+                                   : flight_step_warp<kModePlain, 0>(running, S, P, T, P.prims, P.pairs, nullptr, so);
             if (running) {
                 double* q = o + (size_t)r * 10;
                 float px = S.px, py = S.py, pz = S.pz;
@@ -1299,18 +1404,17 @@ namespace {
 
 using KernelFn = void (*)(const Params);
 
-// the instances [count type][mode][surface-test loop]
-KernelFn kernel_for(int count64, int mode, int masks)
+// the instances [count type][mode][words of the cell masks, 0 = the counted loop]
+#define SPUT_KERNELS(c64, mode) \
+    {transport_kernel<c64, mode, 0>, transport_kernel<c64, mode, 1>, transport_kernel<c64, mode, 2>}
+KernelFn kernel_for(int count64, int mode, int words)
 {
-    static const KernelFn tab[2][3][2] = {
-        {{transport_kernel<false, kModePlain, false>, transport_kernel<false, kModePlain, true>},
-         {transport_kernel<false, kModeScoreT, false>, transport_kernel<false, kModeScoreT, true>},
-         {transport_kernel<false, kModeWalk, false>, transport_kernel<false, kModeWalk, true>}},
-        {{transport_kernel<true, kModePlain, false>, transport_kernel<true, kModePlain, true>},
-         {transport_kernel<true, kModeScoreT, false>, transport_kernel<true, kModeScoreT, true>},
-         {transport_kernel<true, kModeWalk, false>, transport_kernel<true, kModeWalk, true>}}};
-    return tab[count64 ? 1 : 0][mode][masks ? 1 : 0];
+    static const KernelFn tab[2][3][3] = {
+        {SPUT_KERNELS(false, kModePlain), SPUT_KERNELS(false, kModeScoreT), SPUT_KERNELS(false, kModeWalk)},
+        {SPUT_KERNELS(true, kModePlain), SPUT_KERNELS(true, kModeScoreT), SPUT_KERNELS(true, kModeWalk)}};
+    return tab[count64 ? 1 : 0][mode][words];
 }
+#undef SPUT_KERNELS
 
 }  // namespace
 
@@ -1319,9 +1423,9 @@ int transport_max_blocks_per_sm(int count64, int threads, size_t smem)
     // the smallest occupancy of the instances of this count type
     int m = 1 << 30;
     for (int mode = 0; mode < 3; ++mode)
-        for (int masks = 0; masks < 2; ++masks) {
+        for (int words = 0; words < 3; ++words) {
             int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel_for(count64, mode, masks), threads, smem) !=
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel_for(count64, mode, words), threads, smem) !=
                 cudaSuccess)
                 return 0;
             m = nb < m ? nb : m;
@@ -1334,8 +1438,8 @@ int transport_configure(int max_dynamic_smem)
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     for (int c64 = 0; c64 < 2; ++c64)
         for (int mode = 0; mode < 3; ++mode)
-            for (int masks = 0; masks < 2; ++masks) {
-                const cudaError_t e = cudaFuncSetAttribute(kernel_for(c64, mode, masks), a, max_dynamic_smem);
+            for (int words = 0; words < 3; ++words) {
+                const cudaError_t e = cudaFuncSetAttribute(kernel_for(c64, mode, words), a, max_dynamic_smem);
                 if (e != cudaSuccess) return (int)e;
             }
     return 0;
@@ -1344,7 +1448,7 @@ int transport_configure(int max_dynamic_smem)
 int transport_launch(const Params& p, int count64, int blocks, int threads, size_t smem, void* stream)
 {
     const int mode = p.score_T ? kModeScoreT : (p.E_switch > 0.0f ? kModeWalk : kModePlain);
-    kernel_for(count64, mode, p.cell_mask != nullptr)<<<blocks, threads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(p);
+    kernel_for(count64, mode, p.cell_mask ? p.cell_words : 0)<<<blocks, threads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(p);
     return (int)cudaGetLastError();
 }
 
