@@ -293,7 +293,8 @@ const char* sput_last_error(void);
  * b_max(eps) and the head-on apsis in reduced Moliere units, <sigma g>(v) and
  * the partner rejection envelope per cathode/gas pair, the deflection table,
  * racetrack guesses, the surface test's cell masks) and copy
- * scene and tables to `device`.  On success *out owns device memory until
+ * scene and tables to `device`, beside a pool for the last atoms of a run (64 bytes per
+ * lane of the GPU, 10 MB).  On success *out owns device memory until
  * sput_scene_destroy.  Errors: INVALID_ARG, INVALID_SCENE (found on the host
  * before any CUDA call, e.g. an instance whose Thompson cut-off
  * E_max = k Lambda E_i - U_s is not positive), CUDA, NO_MEMORY, and UNSUPPORTED
@@ -331,7 +332,7 @@ sput_status sput_run_host(sput_scene* scene, const sput_run_opts* opts, const sp
  * is owned by another allocator that has reserved it, or latency-critical
  * loops that keep the driver allocator (which may synchronise the device) off
  * their path.  sput_run allocates its run scratch (ticket counter, statistics,
- * status word: 64 bytes) on its first call for a scene; this variant instead
+ * status word, pool counters: 128 bytes) on its first call for a scene; this variant instead
  * uses a static array of 256 bytes in the library's module memory, which every
  * GPU that loads the library holds until the process exits.  It never calls
  * cudaMalloc, cudaFree or any other allocating routine; the scene (inputs) and
@@ -350,6 +351,8 @@ sput_status sput_run_host(sput_scene* scene, const sput_run_opts* opts, const sp
  *     applies) and also reuses the scene's pinned statistics buffer and its two
  *     timing events for kernel_ms; a run of the same scene that overlaps this
  *     one overwrites them, which is one more reason to serialise such calls.
+ * It runs without the drain of the last atoms, whose pool (64 bytes per lane of the GPU)
+ * belongs to the scene and is serialised with its scratch: same results, a longer tail.
  * The paper has no counterpart of this entry point. */
 sput_status sput_run_noalloc(sput_scene* scene, const sput_run_opts* opts, void* stream, const sput_tallies* tallies,
                              sput_run_stats* stats);

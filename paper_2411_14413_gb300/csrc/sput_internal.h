@@ -113,7 +113,7 @@ struct alignas(16) DevPair {
     float inv_s;        // 1 / s_gas, w = ln(1 + v / s_gas)
     int G_off;          // float4 offset of the d ln K / d ln s table (zero for a gas at rest)
     float sigma_D;      // diffusion cross section (A^2) of the thermalised-atom shortcut: 1/lambda_D = n sigma_D
-    float pad_d[2];
+    float w_n, w_top;   // n_w, and 2^23 + n_w - 1 (see table_cell)
 };
 
 struct alignas(16) DevInstance {
@@ -153,7 +153,7 @@ struct Params {
     int n_prims, n_geoms, n_pairs, n_inst;
     int n_bm;
     int n_w_all, n_rt_all, n_lt_all;   // entries of w_tab, rt_tab and lt_tab (bounds of the checked build)
-    float bm_lo, bm_inv_h;
+    float bm_lo, bm_inv_h, bm_n;       // (bm_n = n_bm)
     float box_lo[3], box_hi[3];
     float s_gas;
     float inv_T, inv_s2;               // 1/T (1/K), 1/s_gas^2
@@ -169,6 +169,7 @@ struct Params {
     float ebin_per_eV;
     // tallies (caller-owned device memory, may be null)
     void* counts;
+    int count64;                       // counts are 64-bit
     double* energy;
     double* score;
     double* score_T;                   // temperature score tally (null = off)
@@ -192,6 +193,11 @@ struct Params {
     unsigned long long* ticket_counter;
     unsigned long long* stats;         // [particles, landed, timed_out, flights, collisions, attempts]
     unsigned int* status;
+    // atoms handed over from transport_kernel to drain_kernel (null: none), 4 float4 each
+    float4* pool;
+    unsigned int* pool_count;          // atoms in the pool (zeroed before the run)
+    unsigned int* pool_next;           // next atom to take (zeroed before the run)
+    int drain_live;                    // a warp without tickets hands its atoms over from this many on (32: at once)
     // Gauss-Mehler node constants per evaluation j: (u_j, 1/(1+u_j), u_j/(1-u_j^2), 1/u_j - 1)
     float4 gm[kGMHalf];       // kGMNodes-point rule
     float4 gm_lo[kGMHalfLo];  // kGMNodesLo-point rule (ln eps < kGMLoLnEps)
@@ -210,10 +216,15 @@ constexpr int kTraceRows = 64;
 
 // Launchers implemented in sput_transport.cu.
 int transport_configure(int max_dynamic_smem);
-int transport_launch(const Params& p, int count64, int blocks, int threads, size_t smem, void* stream);
+int transport_launch(const Params& p, int blocks, int threads, size_t smem, void* stream);
 // (the launch picks the kernel instance with the temperature score when p.score_T is set)
 size_t transport_smem_bytes(const Params& p);
-int transport_max_blocks_per_sm(int count64, int threads, size_t smem);
+// the drain of the atoms that transport_kernel hands over (Params::pool)
+constexpr int kDrainThreads = 256;
+int drain_launch(const Params& p, int blocks, size_t smem, void* stream);
+size_t drain_smem_bytes(const Params& p);
+int drain_max_blocks_per_sm(size_t smem);
+int transport_max_blocks_per_sm(int threads, size_t smem);
 int probe_launch(const Params& p, int what, int idx, int n, const double* x_dev, double* y_dev, void* stream);
 
 // Device copy of the scene's instance table (for the adjoint kernels).
@@ -232,7 +243,7 @@ struct NvtxRange {
 void set_last_error(const char* msg);
 
 // Static run scratch of sput_run_noalloc (module memory, no allocation).
-constexpr size_t kRunScratchBytes = 64;      // ticket counter + kNumStats statistics + status word
+constexpr size_t kRunScratchBytes = 128;     // ticket counter, kNumStats statistics, status word, pool counters
 constexpr size_t kStaticScratchBytes = 256;  // capacity of the static array
 // Device address of the static scratch for `device` (must be current); looked
 // up with cudaGetSymbolAddress on the first call in each CUDA context of the

@@ -77,15 +77,18 @@ __device__ __forceinline__ bool idx_ok(unsigned int* status, long long i, long l
 }
 
 // ------------------------------------------------------------- tables
-__device__ __forceinline__ float cubic_eval(const float4* tab, int n, float x)
+// Cell and position of a table coordinate x in [0, n], top = 2^23 + n - 1: i = min(floor(x), n - 1),
+// t = x - i.  The sum with 2^23, rounded down, holds floor(x) in its mantissa; a conversion to
+// integer and back would go through the XU pipe, at a quarter of the rate and five times the
+// latency.
+__device__ __forceinline__ void table_cell(float x, float top, int& i, float& t)
 {
-    // x in piece units; clamped to [0, n]
-    x = fminf(fmaxf(x, 0.0f), (float)n);
-    int i = min((int)x, n - 1);
-    float t = x - (float)i;
-    float4 c = tab[i];
-    return fmaf(t, fmaf(t, fmaf(t, c.w, c.z), c.y), c.x);
+    const float r = fminf(__fadd_rd(x, 8388608.0f), top);
+    i = __float_as_int(r) & 0x7fffff;
+    t = x - (r - 8388608.0f);
 }
+
+__device__ __forceinline__ float cubic(const float4& c, float t) { return fmaf(t, fmaf(t, fmaf(t, c.w, c.z), c.y), c.x); }
 
 struct TableView {
     const float4* bm;
@@ -94,8 +97,8 @@ struct TableView {
     const float4* gm;  // Gauss-Mehler nodes: kGMHalf of the kGMNodes rule, then kGMHalfLo of the kGMNodesLo rule
     const DevPair* pairs;
     const DevGeom* geoms;
-    int n_bm;
     int n_w;           // entries of w (bounds of the checked build)
+    float bm_n, bm_top;  // pieces of bm, and 2^23 + pieces - 1
     float bm_lo, bm_inv_h;
     unsigned int* status;
     const uint32_t* stream;  // Philox stream word per instance (shared memory), or null: read P.inst
@@ -109,14 +112,17 @@ __device__ __forceinline__ uint32_t stream_of(const TableView& T, const Params& 
 
 __device__ __forceinline__ float bmax_eval(const TableView& T, float ln_eps)
 {
-    return cubic_eval(T.bm, T.n_bm, (ln_eps - T.bm_lo) * T.bm_inv_h);
+    int i;
+    float t;
+    table_cell(fminf(fmaxf((ln_eps - T.bm_lo) * T.bm_inv_h, 0.0f), T.bm_n), T.bm_top, i, t);
+    return cubic(T.bm[i], t);
 }
 
 __device__ __forceinline__ float xh_eval(const TableView& T, float ln_eps)
 {
-    float x = fminf(fmaxf((ln_eps - T.bm_lo) * T.bm_inv_h, 0.0f), (float)T.n_bm);
-    int i = min((int)x, T.n_bm - 1);
-    float t = x - (float)i;
+    int i;
+    float t;
+    table_cell(fminf(fmaxf((ln_eps - T.bm_lo) * T.bm_inv_h, 0.0f), T.bm_n), T.bm_top, i, t);
     return fmaf(t, T.xh[i + 1] - T.xh[i], T.xh[i]);
 }
 
@@ -124,17 +130,16 @@ __device__ __forceinline__ float xh_eval(const TableView& T, float ln_eps)
 // (about 4e-7 absolute) moves K, A and B far less than their interpolation error.
 __device__ __forceinline__ float w_of(const DevPair& pr, float v) { return __logf(1.0f + v * pr.inv_s); }
 
-// K(v), A(v) or B(v) of a pair: cubic pieces in w = ln(1 + v/s), at a given w.  The
+// K(v), A(v), B(v) or G(v) of a pair: cubic pieces in w = ln(1 + v/s), at a given w.  The
 // tables are read through L1 from global memory (a few KB per pair, L1-resident), which
 // keeps them out of shared memory so that four blocks fit on an SM.
 __device__ __forceinline__ float wtab_at(const TableView& T, const DevPair& pr, int off, float w)
 {
     if (!idx_ok(T.status, (long long)off + pr.n_w - 1, T.n_w) || !idx_ok(T.status, off, T.n_w)) return 0.0f;
-    const float x = fminf(fmaxf(w * pr.w_inv_h, 0.0f), (float)pr.n_w);
-    const int i = min((int)x, pr.n_w - 1);
-    const float t = x - (float)i;
-    const float4 c = __ldg(T.w + off + i);
-    return fmaf(t, fmaf(t, fmaf(t, c.w, c.z), c.y), c.x);
+    int i;
+    float t;
+    table_cell(fminf(fmaxf(w * pr.w_inv_h, 0.0f), pr.w_n), pr.w_top, i, t);
+    return cubic(__ldg(T.w + off + i), t);
 }
 
 __device__ __forceinline__ float wtab_eval(const TableView& T, const DevPair& pr, int off, float v)
@@ -145,9 +150,8 @@ __device__ __forceinline__ float wtab_eval(const TableView& T, const DevPair& pr
 // sigma(g) g in A^2 km/s
 __device__ __forceinline__ float h_of_g(const TableView& T, const DevPair& pr, float g, float g2)
 {
-    if (pr.hard_sphere) return pr.sigma_scale * g;
-    float b = bmax_eval(T, __logf(pr.kappa * g2));
-    return pr.sigma_scale * b * b * g;
+    const float b = bmax_eval(T, __logf(pr.kappa * g2));
+    return pr.hard_sphere ? pr.sigma_scale * g : pr.sigma_scale * b * b * g;
 }
 
 // 1 - exp(-y) without cancellation for small y
@@ -172,7 +176,7 @@ __device__ __forceinline__ float one_minus_exp_neg(float y)
 // units of pi: apsis by Newton from the head-on lower bound max(beta, x_h),
 // then the Gauss-Mehler sum chi / pi = (2 / N) sum_j D_j / (S_j (S_j + beta/x0))
 // with N = kGMNodesLo below ln eps = kGMLoLnEps, else kGMNodes (2/N is a power
-// of two, so the scaling is exact).
+// of two, so the scaling is exact).  Roundings spelled out, as in the collision (sumsq_xyz).
 __device__ float chi_over_pi_moliere(float eps, float ln_eps, float beta, float xh, const float4* gm)
 {
     const float ie = 1.0f / eps;
@@ -186,20 +190,20 @@ __device__ float chi_over_pi_moliere(float eps, float ln_eps, float beta, float 
     // loops are not unrolled: a compact kernel misses the instruction cache less
 #pragma unroll 1
     for (int it = 0; it < kApsisIters; ++it) {
-        float e0 = kMolC0 * expf(-kMolD0 * x);
+        float e0 = __fmul_rn(kMolC0, expf(-kMolD0 * x));
         float e1 = t1 ? kMolC1 * expf(-kMolD1 * x) : 0.0f;
         float e2 = t2 ? kMolC2 * expf(-kMolD2 * x) : 0.0f;
-        float ph = e0 + e1 + e2;
-        float dph = -(kMolD0 * e0 + kMolD1 * e1 + kMolD2 * e2);
+        float ph = __fadd_rn(__fadd_rn(e0, e1), e2);
+        float dph = -fmaf(kMolD2, e2, fmaf(kMolD1, e1, __fmul_rn(kMolD0, e0)));
         float ix = __frcp_rn(x);
         float ix2 = ix * ix;
-        float g = 1.0f - b2 * ix2 - ph * ix * ie;
-        float gp = 2.0f * b2 * ix2 * ix - (dph * x - ph) * ix2 * ie;
+        float g = fmaf(-__fmul_rn(ph, ix), ie, fmaf(-b2, ix2, 1.0f));  // 1 - b2/x^2 - ph/(x eps)
+        // 2 b2/x^3 - (dph x - ph)/(x^2 eps)
+        float gp = fmaf(__fmul_rn(2.0f * b2, ix2), ix, -__fmul_rn(__fmul_rn(fmaf(dph, x, -ph), ix2), ie));
         x -= __fdividef(g, gp);
     }
     const float x0 = x;
     const float bt = beta / x0;
-    const float bt2 = bt * bt;
     const float iex = ie / x0;
     const bool u1 = x0 < 23.0f, u2 = x0 < 4.0f;
     const float p0 = kMolC0 * expf(-kMolD0 * x0) * iex;
@@ -218,43 +222,41 @@ __device__ float chi_over_pi_moliere(float eps, float ln_eps, float beta, float 
         if (u2) D = fmaf(p2, fmaf(nd.z, one_minus_exp_neg(y2 * nd.w), nd.y), D);
         // S = sqrt(q), q = (beta/x0)^2 + D > 0; approximate reciprocal square root
         // and division (2 ulp) are well inside the quadrature error
-        const float q = bt2 + D;
-        const float S = q * rsqrtf(q);
-        s += __fdividef(D, S * (S + bt));
+        const float q = fmaf(bt, bt, D);
+        const float S = __fmul_rn(q, rsqrtf(q));
+        s += __fdividef(D, __fmul_rn(S, __fadd_rn(S, bt)));
     }
     return s * (lo ? 2.0f / (float)kGMNodesLo : 2.0f / (float)kGMNodes);
 }
 
-// Deflection from the table: q = ln tan(chi/2) at x = ln eps, y = ln(b/b_max) (y <= 0),
-// bicubic in the cell; false outside the table (the caller integrates instead).
-__device__ __forceinline__ bool chi_table_q(const float4* tab, unsigned int* status, float x, float y, float& q)
+// Column and position of y = ln(b/b_max) <= 0 in the deflection table; false below it.
+__device__ __forceinline__ bool chi_table_column(float y, int& j, float& ty)
+{
+    const bool coarse = y < kChiY1;
+    const float fy = (y - (coarse ? kChiY0 : kChiY1)) * (coarse ? 1.0f / kChiHyC : 1.0f / kChiHyF);
+    table_cell(fmaxf(fy, 0.0f), 8388608.0f + (float)((coarse ? kChiNyC : kChiNyF) - 1), j, ty);
+    ty = fminf(ty, 1.0f);
+    j += coarse ? 0 : kChiNyC;
+    return y >= kChiY0;
+}
+
+// Deflection from the table: q = ln tan(chi/2) at x = ln eps in column j at ty, bicubic in the
+// cell; false outside the table (then q is that of the nearest row: the caller integrates
+// instead).  No branch, so that it overlaps with what the caller does beside it.
+__device__ __forceinline__ bool chi_table_q(const float4* tab, unsigned int* status, float x, int j, float ty, float& q)
 {
     const float fx = (x - kChiX0) * (1.0f / kChiHx);
-    if (!(fx >= 0.0f && fx < (float)kChiNx && y >= kChiY0)) return false;
-    const int i = min((int)fx, kChiNx - 1);
-    const float tx = fx - (float)i;
-    int j;
-    float ty;
-    if (y < kChiY1) {
-        const float fy = (y - kChiY0) * (1.0f / kChiHyC);
-        j = min((int)fy, kChiNyC - 1);
-        ty = fy - (float)j;
-    } else {
-        const float fy = (y - kChiY1) * (1.0f / kChiHyF);
-        j = min((int)fy, kChiNyF - 1);
-        ty = fminf(fy - (float)j, 1.0f);
-        j += kChiNyC;
-    }
+    const bool in = fx >= 0.0f && fx < (float)kChiNx;
+    int i;
+    float tx;
+    table_cell(fminf(fmaxf(fx, 0.0f), (float)kChiNx), 8388608.0f + (float)(kChiNx - 1), i, tx);
     const int cell = i * kChiNy + j;
     if (!idx_ok(status, cell, kChiCells)) return false;
     const float4* c = tab + 4 * cell;
     const float4 r0 = __ldg(c), r1 = __ldg(c + 1), r2 = __ldg(c + 2), r3 = __ldg(c + 3);
-    const float c0 = fmaf(ty, fmaf(ty, fmaf(ty, r0.w, r0.z), r0.y), r0.x);
-    const float c1 = fmaf(ty, fmaf(ty, fmaf(ty, r1.w, r1.z), r1.y), r1.x);
-    const float c2 = fmaf(ty, fmaf(ty, fmaf(ty, r2.w, r2.z), r2.y), r2.x);
-    const float c3 = fmaf(ty, fmaf(ty, fmaf(ty, r3.w, r3.z), r3.y), r3.x);
+    const float c0 = cubic(r0, ty), c1 = cubic(r1, ty), c2 = cubic(r2, ty), c3 = cubic(r3, ty);
     q = fmaf(tx, fmaf(tx, fmaf(tx, c3, c2), c1), c0);
-    return true;
+    return in;
 }
 
 // cos and sin of the deflection from q = ln tan(chi/2): with T = e^q,
@@ -271,12 +273,16 @@ __device__ __forceinline__ void chi_cos_sin(float q, float& cc, float& sc)
 // (sin 2 pi u, cos 2 pi u) for u in (0, 1] from the MUFU sine and cosine, whose
 // absolute error bound (about 2^-21.4) holds on [-pi, pi]: 2 pi u = 2 pi (u - 1/2) + pi,
 // and u - 1/2 is exact for u = m 2^-24
+__device__ __forceinline__ void neg_sincos_2pi_fast(float u, float* ns, float* nc)
+{
+    __sincosf(6.283185307179586f * (u - 0.5f), ns, nc);
+}
 __device__ __forceinline__ void sincos_2pi_fast(float u, float* s, float* c)
 {
-    float ss, cc;
-    __sincosf(6.283185307179586f * (u - 0.5f), &ss, &cc);
-    *s = -ss;
-    *c = -cc;
+    float ns, nc;
+    neg_sincos_2pi_fast(u, &ns, &nc);
+    *s = -ns;
+    *c = -nc;
 }
 
 // -ln u for u in (0, 1] from the MUFU logarithm (absolute error about 2^-21.4 near 1,
@@ -296,14 +302,28 @@ __device__ __forceinline__ void onb(float nx, float ny, float nz, float3& b1, fl
     b2 = make_float3(b, sgn + ny * ny * a, -ny);
 }
 
+// Sums of products with their roundings spelled out.  An atom's collisions are computed in more
+// than one kernel, and its path has to be the same in each of them: what is fused to an FMA is
+// therefore not left to the compiler, which decides it by the surrounding code.
+__device__ __forceinline__ float sumsq_xyz(float x, float y, float z)
+{
+    return fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)));
+}
+__device__ __forceinline__ float sumsq_yxz(float x, float y, float z)
+{
+    return fmaf(z, z, fmaf(x, x, __fmul_rn(y, y)));
+}
+// a b + c d, the second product rounded first
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return fmaf(a, b, __fmul_rn(c, d)); }
+
 // ------------------------------------------------------------- launch
 struct Lane {
     float px, py, pz, dx, dy, dz, speed, score;
     float scoreT;  // d ln p(path)/dT (kernel instance with the temperature score only)
     bool diff;     // thermalised: random walk of the diffusion shortcut
-    uint32_t pid, inst, k, ncoll;
+    uint32_t pid, inst, k;  // k flights begun: k - 1 collisions while the k-th lasts
     int geom, pair;  // geometry index (its record is read from TableView::geoms), gas pair
-    float ng14, E_per_v2;
+    float ng14;
 };
 
 __device__ __forceinline__ float racetrack_r(const DevCathode& C, const float4* rt_tab, int rt_n, int n_rt_all,
@@ -495,7 +515,6 @@ __device__ void start_from(Lane& S, const Params& P, const Launch& L)
     S.geom = idx_ok(P.status, I.geometry, P.n_geoms) ? I.geometry : 0;
     S.pair = idx_ok(P.status, I.pair, P.n_pairs) ? I.pair : 0;
     S.ng14 = I.ng14;
-    S.E_per_v2 = P.cath[I.cathode].E_per_v2;
     S.px = L.px;
     S.py = L.py;
     S.pz = L.pz;
@@ -507,7 +526,6 @@ __device__ void start_from(Lane& S, const Params& P, const Launch& L)
     // flight step retires with the non-finite status bit
     if (P.inject_nonfinite && L.pid == 0u) S.speed = CUDART_NAN_F;
     S.k = 0u;
-    S.ncoll = 0u;
     S.score = 0.0f;
     S.scoreT = 0.0f;
     S.diff = false;
@@ -529,6 +547,38 @@ struct StepOut {
     float Gv;       // d ln K / d ln s at the flight's speed (temperature score only)
 };
 
+// Inverse mean free path at the atom's speed and the flight length, nl = -ln u; Gv =
+// d ln K / d ln s at its speed (temperature score only).
+template <int kMode>
+__device__ __forceinline__ void flight_length(const Lane& S, const Params& P, const TableView& T, const DevPair& pr,
+                                              float nl, float& inv_lam, float& ell, float& Gv)
+{
+    // n_g <sigma g>/v (thermal) or n_g sigma(v) (gas at rest)
+    const float Kv = wtab_eval(T, pr, pr.K_off, S.speed);
+    inv_lam = P.gas_thermal ? S.ng14 * Kv / S.speed : S.ng14 * Kv;
+    // diffusion shortcut: exponential steps of mean lambda_D, 1/lambda_D = n sigma_D
+    if (kMode == kModeWalk && S.diff) inv_lam = S.ng14 * pr.sigma_D;
+    ell = S.ng14 > 0.0f ? __fdividef(nl, inv_lam) : CUDART_INF_F;
+    if (kMode == kModeScoreT) {
+        // (this table stays in global memory: w_tab + G_off, read through L1)
+        Gv = idx_ok(P.status, (long long)pr.G_off + pr.n_w - 1, P.n_w_all)
+                 ? wtab_eval(T, pr, pr.G_off, S.speed)
+                 : 0.0f;
+    }
+}
+
+// Terms of the path scores.  Pressure: a flight of length l that ends in a collision adds
+// 1 - l/lambda, a landing takes t/lambda.  Temperature: the same times d ln(n_g K(v)/v)/dT =
+// (-1 + G/2)/T (n_g = p/(k_B T), G = d ln K/d ln s), and per collision the partner density
+// f_T(V) sigma(g) g / K(v): d ln/dT = (|V|^2/(2 s^2) - 3/2 - G/2)/T, here without its 1/T.
+// Rounded as written wherever they are used.
+__device__ __forceinline__ float score_gain(float ell, float inv_lam) { return fmaf(-ell, inv_lam, 1.0f); }
+__device__ __forceinline__ float score_T_rate(const Params& P, float Gv) { return fmaf(0.5f, Gv, -1.0f) * P.inv_T; }
+__device__ __forceinline__ float score_T_partner(const Params& P, float V2, float Gv)
+{
+    return fmaf(-0.5f, Gv, fmaf(0.5f * V2, P.inv_s2, -1.5f));
+}
+
 // Free flight k+1 of the atom in S: its Philox block w (word 0 the free path; words 1 and 2,
 // the impact parameter and azimuth, are used by the collision; word 3 is unused), the
 // inverse mean free path and the flight length.
@@ -538,19 +588,7 @@ __device__ void flight_begin(Lane& S, const Params& P, const TableView& T, const
 {
     S.k += 1u;
     w = philox(P, S.pid, stream_of(T, P, S.inst), S.k, 0u);
-    const DevPair pr = pairs[S.pair];
-    // inverse mean free path n_g <sigma g>/v (thermal) or n_g sigma(v) (gas at rest)
-    const float Kv = wtab_eval(T, pr, pr.K_off, S.speed);
-    inv_lam = P.gas_thermal ? S.ng14 * Kv / S.speed : S.ng14 * Kv;
-    // diffusion shortcut: exponential steps of mean lambda_D, 1/lambda_D = n sigma_D
-    if (kMode == kModeWalk && S.diff) inv_lam = S.ng14 * pr.sigma_D;
-    ell = S.ng14 > 0.0f ? __fdividef(neg_log_fast(rn(w.x)), inv_lam) : CUDART_INF_F;
-    if (kMode == kModeScoreT) {
-        // (this table stays in global memory: w_tab + G_off, read through L1)
-        out.Gv = idx_ok(P.status, (long long)pr.G_off + pr.n_w - 1, P.n_w_all)
-                     ? cubic_eval(P.w_tab + pr.G_off, pr.n_w, w_of(pr, S.speed) * pr.w_inv_h)
-                     : 0.0f;
-    }
+    flight_length<kMode>(S, P, T, pairs[S.pair], neg_log_fast(rn(w.x)), inv_lam, ell, out.Gv);
 }
 
 // The emitting target's local index on the first flight (it is skipped then: the atom
@@ -708,11 +746,10 @@ __device__ int flight_end(Lane& S, const Params& P, StepOut& out, float inv_lam,
     constexpr bool kScoreT = kMode == kModeScoreT;
     out.nonfinite = 0;
     out.prim = -1;
-    // temperature score: d ln(n_g K(v)/v)/dT = (-1 + G/2)/T with n_g = p/(k_B T), G = d ln K/d ln s
-    const float aT = kScoreT ? (0.5f * out.Gv - 1.0f) * P.inv_T : 0.0f;
+    const float aT = kScoreT ? score_T_rate(P, out.Gv) : 0.0f;
     if (hb >= 0 && tb <= ell) {
-        S.score -= tb * inv_lam;
-        if (kScoreT) S.scoreT -= aT * tb * inv_lam;
+        S.score = fmaf(-tb, inv_lam, S.score);
+        if (kScoreT) S.scoreT = fmaf(-(aT * tb), inv_lam, S.scoreT);
         out.t = tb;
         out.prim = hb;
         return kStepLanded;
@@ -721,8 +758,9 @@ __device__ int flight_end(Lane& S, const Params& P, StepOut& out, float inv_lam,
     S.px = fmaf(ell, S.dx, S.px);
     S.py = fmaf(ell, S.dy, S.py);
     S.pz = fmaf(ell, S.dz, S.pz);
-    S.score += 1.0f - ell * inv_lam;
-    if (kScoreT) S.scoreT += aT * (1.0f - ell * inv_lam);
+    const float gain = score_gain(ell, inv_lam);
+    S.score += gain;
+    if (kScoreT) S.scoreT = fmaf(aT, gain, S.scoreT);
     if (!isfinite(S.px + S.py + S.pz + S.speed)) {
         out.nonfinite = 1;
         return kStepTimedOut;
@@ -742,6 +780,74 @@ __device__ __forceinline__ int nth_set_bit(unsigned mask, int n)
     for (int w = 16; w >= 1; w >>= 1)
         if (__popc(mask & ((1u << (pos + w)) - 1u)) <= n) pos += w;
     return pos;
+}
+
+// One attempt of the partner rejection below: the proposal's normals and their norms, and
+// the uniform of its test.  Independent of the atom's velocity.
+struct Attempt {
+    float z1, z2, z3;
+    float r3;     // |(z1, z2, z3)|: rho of the Maxwellian branch
+    float rho_w;  // |(z1, z2, z3, z4)|: rho of the weighted branch
+    float sc_w;   // scale of (z1, z2, z3) in the weighted branch
+    float u;
+};
+
+__device__ __forceinline__ Attempt attempt_draw(const Params& P, uint32_t pid, uint32_t strm, uint32_t k, uint32_t a)
+{
+    const uint4 wn = philox(P, pid, strm, k, 1u + a);
+    const float R0 = sqrt_fast(2.0f * neg_log_fast(rn(wn.x)));
+    const float R1 = sqrt_fast(2.0f * neg_log_fast(rn(wn.z)));
+    float s1, c1, s3, c3;
+    sincos_2pi_fast(rn(wn.y), &s1, &c1);
+    sincos_2pi_fast(rn(wn.w), &s3, &c3);
+    Attempt d;
+    d.z1 = R0 * c1;
+    d.z2 = R0 * s1;
+    d.z3 = R1 * c3;
+    const float z4 = R1 * s3;
+    // low bytes of words 0, 1, 2 as one more 24-bit uniform
+    const uint32_t lowb = ((wn.x & 0xffu) << 24) | ((wn.y & 0xffu) << 16) | ((wn.z & 0xffu) << 8);
+    d.u = rn(lowb);
+    const float r32 = sumsq_xyz(d.z1, d.z2, d.z3);
+    const float ir3 = r32 > 0.0f ? rsqrtf(r32) : 0.0f;
+    d.r3 = r32 * ir3;
+    d.rho_w = sqrt_fast(r32 + z4 * z4);
+    d.sc_w = P.s_gas * (d.rho_w * ir3);
+    return d;
+}
+
+// Whether the attempt takes the rho-weighted branch when the pair's envelope is EA + EB rho.
+__device__ __forceinline__ bool attempt_weighted(const Attempt& d, float EA, float EB, float& ut, float& Bm)
+{
+    Bm = __fmul_rn(EB, (float)kEnvM);
+    ut = __fmul_rn(d.u, __fadd_rn(EA, Bm));
+    return ut <= Bm;
+}
+
+// The attempt's gas velocity in a branch.
+__device__ __forceinline__ void attempt_velocity(const Params& P, const Attempt& d, bool weighted, float& cx, float& cy,
+                                                 float& cz)
+{
+    const float sc = weighted ? d.sc_w : P.s_gas;
+    cx = __fmul_rn(sc, d.z1);
+    cy = __fmul_rn(sc, d.z2);
+    cz = __fmul_rn(sc, d.z3);
+}
+
+// h(g) = sigma(g) g between the atom's velocity v and the gas velocity c
+__device__ __forceinline__ float attempt_h(const TableView& T, const DevPair& pr, float vx, float vy, float vz, float cx,
+                                           float cy, float cz)
+{
+    const float g2 = sumsq_yxz(__fsub_rn(vx, cx), __fsub_rn(vy, cy), __fsub_rn(vz, cz));
+    return h_of_g(T, pr, sqrt_fast(g2), g2);
+}
+
+// Acceptance: the branch's own uniform, rescaled to (0, 1], times the envelope against h.
+__device__ __forceinline__ bool attempt_accept(const Attempt& d, bool weighted, float ut, float Bm, float EA, float EB,
+                                               float hg)
+{
+    const float env = fmaf(EB, weighted ? d.rho_w : d.r3, EA);
+    return weighted ? ut * env <= Bm * hg : __fsub_rn(ut, Bm) * env <= EA * hg;
 }
 
 // Gas partners of every lane with `need`, drawn by the whole warp: the
@@ -805,33 +911,13 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
         bool acc = false;
         float cx = 0.0f, cy = 0.0f, cz = 0.0f;
         if (a < A) {
-            const uint4 wn = philox(P, o_pid, o_strm, o_k, 1u + (uint32_t)a);
-            const float R0 = sqrt_fast(2.0f * neg_log_fast(rn(wn.x)));
-            const float R1 = sqrt_fast(2.0f * neg_log_fast(rn(wn.z)));
-            float s1, c1, s3, c3;
-            sincos_2pi_fast(rn(wn.y), &s1, &c1);
-            sincos_2pi_fast(rn(wn.w), &s3, &c3);
-            const float z1 = R0 * c1, z2 = R0 * s1, z3 = R1 * c3, z4 = R1 * s3;
-            // low bytes of words 0, 1, 2 as one more 24-bit uniform
-            const uint32_t lowb = ((wn.x & 0xffu) << 24) | ((wn.y & 0xffu) << 16) | ((wn.z & 0xffu) << 8);
-            const float Bm = o_B * (float)kEnvM;
-            const float ut = rn(lowb) * (o_A + Bm);
-            const bool weighted = ut <= Bm;
-            const float r32 = z1 * z1 + z2 * z2 + z3 * z3;
-            const float ir3 = r32 > 0.0f ? rsqrtf(r32) : 0.0f;
-            const float r3 = r32 * ir3;
-            const float rho = weighted ? sqrt_fast(r32 + z4 * z4) : r3;
-            const float sc = P.s_gas * (weighted ? rho * ir3 : 1.0f);
-            cx = sc * z1;
-            cy = sc * z2;
-            cz = sc * z3;
-            const float gx = o_vx - cx, gy = o_vy - cy, gz = o_vz - cz;
-            const float g2 = gx * gx + gy * gy + gz * gz;
             const int op = idx_ok(T.status, o_pair, P.n_pairs) ? o_pair : 0;
-            const float hg = h_of_g(T, pairs[op], sqrt_fast(g2), g2);
-            const float env = fmaf(o_B, rho, o_A);
-            // the branch's own uniform, rescaled to (0, 1], times the envelope against h
-            acc = (weighted ? ut * env <= Bm * hg : (ut - Bm) * env <= o_A * hg) || a == A - 1;
+            const Attempt d = attempt_draw(P, o_pid, o_strm, o_k, (uint32_t)a);
+            float ut, Bm;
+            const bool weighted = attempt_weighted(d, o_A, o_B, ut, Bm);
+            attempt_velocity(P, d, weighted, cx, cy, cz);
+            const float hg = attempt_h(T, pairs[op], o_vx, o_vy, o_vz, cx, cy, cz);
+            acc = attempt_accept(d, weighted, ut, Bm, o_A, o_B, hg) || a == A - 1;
         }
         const unsigned accm = __ballot_sync(kFull, acc);
         const bool is_owner = (pending >> lane) & 1u;
@@ -864,57 +950,101 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
     }
 }
 
-// Binary collision in the CM frame: rotate g = v - V by (chi, psi), |g| kept.
-__device__ void scatter(Lane& S, const Params& P, const TableView& T, const DevPair& pr, float vx, float vy, float vz,
-                        float Vx, float Vy, float Vz, const uint4& w)
+// The draws of a collision, from its flight's Philox block.
+struct Impact {
+    float ub;        // uniform of the impact parameter b = b_max sqrt(ub)
+    int j;           // column of ln(ub)/2 in the deflection table, -1 below it
+    float ty;
+    float nsp, ncp;  // negated sine and cosine of the azimuth
+};
+
+__device__ __forceinline__ Impact impact_draw(const uint4& w)
 {
-    const float gx = vx - Vx, gy = vy - Vy, gz = vz - Vz;
-    const float g2 = gx * gx + gy * gy + gz * gz;
+    Impact I;
+    I.ub = rn(w.y);
+    if (!chi_table_column(0.5f * logf(I.ub), I.j, I.ty)) I.j = -1;
+    neg_sincos_2pi_fast(rn(w.z), &I.nsp, &I.ncp);
+    return I;
+}
+
+// Cosine and sine of the CM deflection off the table: hard spheres, or the scattering integral.
+__device__ __forceinline__ void deflect_off_table(const TableView& T, const DevPair& pr, float eps, float le, float ub,
+                                                  float& cc, float& sc)
+{
+    if (pr.hard_sphere) {
+        sincospif(acosf(sqrtf(ub)) * (2.0f / 3.14159265358979f), &sc, &cc);
+    } else {
+        const float beta = bmax_eval(T, le) * sqrtf(ub);
+        sincospif(chi_over_pi_moliere(eps, le, beta, xh_eval(T, le), T.gm), &sc, &cc);
+    }
+}
+
+// Binary collision in the CM frame: rotate g = v - V by (chi, psi), |g| kept; the atom's speed and
+// direction (of velocity v) become those after it.  One rare branch (off the deflection
+// table); the rest is straight-line code.
+template <int kMode>
+__device__ __forceinline__ void scatter(float& speed, float& dx, float& dy, float& dz, const Params& P,
+                                        const TableView& T, const DevPair& pr, float vx, float vy, float vz, float Vx,
+                                        float Vy, float Vz, const Impact& I)
+{
+    const float gx = __fsub_rn(vx, Vx), gy = __fsub_rn(vy, Vy), gz = __fsub_rn(vz, Vz);
+    // (the temperature-score instance rounds this sum in the other order, as its results always were)
+    const float g2 = kMode == kModeScoreT ? sumsq_yxz(gx, gy, gz) : sumsq_xyz(gx, gy, gz);
+    const float ig = rsqrtf(g2);
+    const float g = g2 * ig;
+    const float hx = gx * ig, hy = gy * ig, hz = gz * ig;
+    const float eps = pr.kappa * g2;
+    const float le = logf(eps);
+    float sc, cc, q = 0.0f;
+    bool on_table = false;
+    if (P.chi_tab) {
+        on_table = chi_table_q(P.chi_tab, P.status, le, max(I.j, 0), I.ty, q) && I.j >= 0;
+        chi_cos_sin(q, cc, sc);
+    }
+    if (!on_table && g2 > 0.0f) deflect_off_table(T, pr, eps, le, I.ub, cc, sc);
+    const float sp = -I.nsp, cp = -I.ncp;
+    float3 b1, b2;
+    onb(hx, hy, hz, b1, b2);
+    const float gpx = __fmul_rn(g, dot2(cc, hx, sc, dot2(sp, b2.x, cp, b1.x)));
+    const float gpy = __fmul_rn(g, dot2(cc, hy, sc, dot2(sp, b2.y, cp, b1.y)));
+    const float gpz = __fmul_rn(g, dot2(cc, hz, sc, dot2(sp, b2.z, cp, b1.z)));
+    const float nvx = fmaf(pr.m2M, gpx, dot2(pr.m1M, vx, pr.m2M, Vx));
+    const float nvy = fmaf(pr.m2M, gpy, dot2(pr.m1M, vy, pr.m2M, Vy));
+    const float nvz = fmaf(pr.m2M, gpz, dot2(pr.m1M, vz, pr.m2M, Vz));
+    // an atom slowed to ~1e-15 km/s or below (gas at rest) would underflow the
+    // squares: scale by the exact power of two 2^60 first
+    const float up = sumsq_xyz(nvx, nvy, nvz) < 1e-30f ? 0x1p60f : 1.0f;
+    const float ux = nvx * up, uy = nvy * up, uz = nvz * up;
+    const float sp2 = sumsq_yxz(ux, uy, uz);
+    const float is = rsqrtf(sp2);
+    const float sn = sp2 * is;
+    const bool moves = sp2 > 0.0f;
     if (g2 > 0.0f) {
-        const float ig = rsqrtf(g2);
-        const float g = g2 * ig;
-        const float hx = gx * ig, hy = gy * ig, hz = gz * ig;
-        float sc, cc, sp, cp;
-        const float ub = rn(w.y);  // impact parameter b = b_max sqrt(ub)
-        float q;
-        if (pr.hard_sphere) {
-            sincospif(acosf(sqrtf(ub)) * (2.0f / 3.14159265358979f), &sc, &cc);
-        } else {
-            const float eps = pr.kappa * g2;
-            const float le = logf(eps);
-            if (chi_table_q(P.chi_tab, P.status, le, 0.5f * logf(ub), q)) {
-                chi_cos_sin(q, cc, sc);
-            } else {
-                const float beta = bmax_eval(T, le) * sqrtf(ub);
-                sincospif(chi_over_pi_moliere(eps, le, beta, xh_eval(T, le), T.gm), &sc, &cc);
-            }
-        }
-        sincos_2pi_fast(rn(w.z), &sp, &cp);
-        float3 b1, b2;
-        onb(hx, hy, hz, b1, b2);
-        const float gpx = g * (cc * hx + sc * (cp * b1.x + sp * b2.x));
-        const float gpy = g * (cc * hy + sc * (cp * b1.y + sp * b2.y));
-        const float gpz = g * (cc * hz + sc * (cp * b1.z + sp * b2.z));
-        const float nvx = pr.m1M * vx + pr.m2M * Vx + pr.m2M * gpx;
-        const float nvy = pr.m1M * vy + pr.m2M * Vy + pr.m2M * gpy;
-        const float nvz = pr.m1M * vz + pr.m2M * Vz + pr.m2M * gpz;
-        // an atom slowed to ~1e-15 km/s or below (gas at rest) would underflow the
-        // squares: scale by the exact power of two 2^60 first
-        const float up = nvx * nvx + nvy * nvy + nvz * nvz < 1e-30f ? 0x1p60f : 1.0f;
-        const float ux = nvx * up, uy = nvy * up, uz = nvz * up;
-        const float sp2 = ux * ux + uy * uy + uz * uz;
-        if (sp2 > 0.0f) {
-            const float is = rsqrtf(sp2);
-            const float sn = sp2 * is;
-            S.speed = up == 1.0f ? sn : sn * 0x1p-60f;
-            S.dx = ux * is;
-            S.dy = uy * is;
-            S.dz = uz * is;
-        } else {
-            S.speed = 0.0f;  // at rest: the direction is kept
+        speed = !moves ? 0.0f : up == 1.0f ? sn : sn * 0x1p-60f;
+        if (moves) {  // at rest: the direction is kept
+            dx = ux * is;
+            dy = uy * is;
+            dz = uz * is;
         }
     }
-    ++S.ncoll;
+}
+
+// Isotropic direction of the diffusion shortcut's walk from the flight block's words 1 and 2.
+__device__ __forceinline__ void walk_direction(const uint4& w, float& dx, float& dy, float& dz)
+{
+    const float mu = 2.0f * rn(w.y) - 1.0f;
+    const float st = sqrtf(fmaxf(0.0f, (1.0f - mu) * (1.0f + mu)));
+    float sp, cp;
+    sincospif(2.0f * rn(w.z), &sp, &cp);
+    dx = st * cp;
+    dy = st * sp;
+    dz = mu;
+}
+
+// E (eV) of an atom of instance inst at this speed
+__device__ __forceinline__ float energy_of(const Params& P, uint32_t inst, float speed)
+{
+    return P.cath[P.inst[inst].cathode].E_per_v2 * speed * speed;
 }
 
 // One flight of every active lane of the warp (flight, surface test, then for
@@ -941,7 +1071,7 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
     const bool walk = kMode == kModeWalk && res == kStepCollided && S.diff;
     const bool coll = res == kStepCollided && !walk;
     const DevPair pr = pairs[S.pair];
-    const float vx = S.speed * S.dx, vy = S.speed * S.dy, vz = S.speed * S.dz;
+    const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
     float Vx = 0.0f, Vy = 0.0f, Vz = 0.0f;
     if (P.gas_thermal) {
         float EA = 0.0f, EB = 0.0f;
@@ -953,25 +1083,127 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
         // the owner's Philox stream word travels with it (one shuffle instead of a lookup per attempt)
         partner_sample_warp(coll, P, T, pairs, S.pid, stream_of(T, P, S.inst), S.k, S.pair, vx, vy, vz, EA, EB, Vx,
                             Vy, Vz, out.attempts);
-        // partner density f_T(V) sigma(g) g / K(v): d ln/dT = (|V|^2/(2 s^2) - 3/2 - G/2)/T
         if (kScoreT && coll)
-            S.scoreT += (0.5f * (Vx * Vx + Vy * Vy + Vz * Vz) * P.inv_s2 - 1.5f - 0.5f * out.Gv) * P.inv_T;
+            S.scoreT = fmaf(score_T_partner(P, sumsq_xyz(Vx, Vy, Vz), out.Gv), P.inv_T, S.scoreT);
     }
     if (coll) {
-        scatter(S, P, T, pr, vx, vy, vz, Vx, Vy, Vz, w);
-        if (kMode == kModeWalk && S.E_per_v2 * S.speed * S.speed < P.E_switch) S.diff = true;
+        scatter<kMode>(S.speed, S.dx, S.dy, S.dz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, impact_draw(w));
+        if (kMode == kModeWalk && energy_of(P, S.inst, S.speed) < P.E_switch) S.diff = true;
     } else if (walk) {
-        // isotropic direction from the flight block's words 1 and 2
-        const float mu = 2.0f * rn(w.y) - 1.0f;
-        const float st = sqrtf(fmaxf(0.0f, (1.0f - mu) * (1.0f + mu)));
-        float sp, cp;
-        sincospif(2.0f * rn(w.z), &sp, &cp);
-        S.dx = st * cp;
-        S.dy = st * sp;
-        S.dz = mu;
-        ++S.ncoll;
+        walk_direction(w, S.dx, S.dy, S.dz);
     }
     return res;
+}
+
+// Adds the lanes' statistics to the run's; particles = landed + timed out, flights = landed +
+// timed out + collisions.  Called by whole warps.
+__device__ __forceinline__ void add_stats(const Params& P, uint32_t landed, uint32_t timed, unsigned long long coll,
+                                          uint32_t att)
+{
+    unsigned long long v[kNumStats] = {landed + timed, landed, timed, landed + timed + coll, coll, att};
+#pragma unroll
+    for (int i = 0; i < kNumStats; ++i) {
+        unsigned long long x = v[i];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
+        if ((threadIdx.x & 31) == 0 && x) atomicAdd(P.stats + i, x);
+    }
+}
+
+// ------------------------------------------------------------- hand-over
+// Atoms between two flights, in Params::pool.
+__device__ __forceinline__ void pool_store(const Params& P, bool have, const Lane& S)
+{
+    const unsigned m = __ballot_sync(kFull, have);
+    const int lane = threadIdx.x & 31;
+    unsigned base = 0u;
+    if (lane == 0 && m) base = atomicAdd(P.pool_count, (unsigned)__popc(m));
+    base = __shfl_sync(kFull, base, 0);
+    if (!have) return;
+    const unsigned i = base + __popc(m & ((1u << lane) - 1u));
+    float4* q = P.pool + 4 * (size_t)i;
+    q[0] = make_float4(S.px, S.py, S.pz, S.speed);
+    q[1] = make_float4(S.dx, S.dy, S.dz, S.score);
+    q[2] = make_float4(__uint_as_float(S.pid), __uint_as_float(S.inst), __uint_as_float(S.k),
+                       __uint_as_float(S.diff ? 1u : 0u));
+    q[3] = make_float4(S.scoreT, 0.0f, 0.0f, 0.0f);
+}
+
+// ------------------------------------------------------------- tallies
+__device__ __forceinline__ void write_record(const Params& P, const Lane& S, int prim, int cell, float E, float cosang)
+{
+    const unsigned long long t = P.prefix[S.inst] + S.pid - P.ticket_begin;
+    if (!idx_ok(P.status, (long long)t, (long long)(P.ticket_end - P.ticket_begin))) return;
+    sput_record rec;
+    rec.prim = prim;
+    rec.cell = cell;
+    rec.energy = E;
+    rec.cos_angle = cosang;
+    rec.n_collisions = S.k - 1u;
+    rec.score = S.score;
+    P.records[t] = rec;
+}
+
+// Landing of the atom in S (pre-flight position) on primitive hb at distance tb; s_cnt: the
+// block's counters when they are privatised (P.smem_counters).
+template <int kMode>
+__device__ __forceinline__ void tally_landed(const Params& P, const Lane& S, const DevGeom* geoms, const DevPrim* prims,
+                                             unsigned int* s_cnt, float tb, int hb)
+{
+    const float E = energy_of(P, S.inst, S.speed);
+    int cell = -1;
+    float cosang = 0.0f;
+    const DevGeom G = geoms[S.geom];
+    if (hb == G.substrate()) {
+        const DevPrim& Q = prims[G.begin + hb];
+        const float dn = S.dx * Q.nx + S.dy * Q.ny + S.dz * Q.nz;
+        if (dn < 0.0f) {
+            const float qx = fmaf(tb, S.dx, S.px) - Q.cx, qy = fmaf(tb, S.dy, S.py) - Q.cy,
+                        qz = fmaf(tb, S.dz, S.pz) - Q.cz;
+            const float a1 = qx * Q.ux + qy * Q.uy + qz * Q.uz;
+            const float a2 = qx * Q.vx + qy * Q.vy + qz * Q.vz;
+            const float fx = (a1 + P.half_u) * P.cells_per_mm_u;
+            const float fy = (a2 + P.half_v) * P.cells_per_mm_v;
+            if (fx >= 0.0f && fy >= 0.0f && fx <= (float)P.nx && fy <= (float)P.ny) {
+                const int ix = min((int)fx, P.nx - 1), iy = min((int)fy, P.ny - 1);
+                cell = iy * P.nx + ix;
+            }
+            cosang = -dn;
+        }
+    }
+    const int ncell = P.nx * P.ny;
+    if (cell >= 0 && idx_ok(P.status, (long long)S.inst * ncell + cell, (long long)P.n_inst * ncell)) {
+        const size_t ci = (size_t)S.inst * ncell + cell;
+        if (P.counts) {
+            if (P.count64) atomicAdd(reinterpret_cast<unsigned long long*>(P.counts) + ci, 1ull);
+            else atomicAdd(reinterpret_cast<unsigned int*>(P.counts) + ci, 1u);
+        }
+        if (P.energy) atomicAdd(P.energy + ci, (double)E);
+        if (P.score) atomicAdd(P.score + ci, (double)S.score);
+        if (kMode == kModeScoreT) atomicAdd(P.score_T + ci, (double)S.scoreT);
+        if (P.hist_E) {
+            int b = min(max((int)(E * P.ebin_per_eV), 0), P.n_ebins - 1);
+            atomicAdd(reinterpret_cast<unsigned long long*>(P.hist_E) + (size_t)S.inst * P.n_ebins + b, 1ull);
+        }
+        if (P.hist_A) {
+            const float th = acosf(fminf(cosang, 1.0f)) * (57.29577951308232f / 90.0f);
+            int b = min(max((int)(th * (float)P.n_abins), 0), P.n_abins - 1);
+            atomicAdd(reinterpret_cast<unsigned long long*>(P.hist_A) + (size_t)S.inst * P.n_abins + b, 1ull);
+        }
+    }
+    if (!idx_ok(P.status, hb, P.max_prims)) {
+        // dropped: the checked build reports it
+    } else if (s_cnt) atomicAdd(&s_cnt[S.inst * (P.max_prims + 1) + hb], 1u);
+    else if (P.prim_counts)
+        atomicAdd(reinterpret_cast<unsigned long long*>(P.prim_counts) + (size_t)S.inst * P.max_prims + hb, 1ull);
+    if (P.records) write_record(P, S, hb, cell, E, cosang);
+}
+
+__device__ __forceinline__ void tally_timed_out(const Params& P, const Lane& S, unsigned int* s_cnt, int nonfinite)
+{
+    if (nonfinite) atomicOr(P.status, kStatusNonFinite);
+    if (s_cnt) atomicAdd(&s_cnt[S.inst * (P.max_prims + 1) + P.max_prims], 1u);
+    else if (P.timed_out) atomicAdd(reinterpret_cast<unsigned long long*>(P.timed_out) + S.inst, 1ull);
+    if (P.records) write_record(P, S, -1, -1, energy_of(P, S.inst, S.speed), 0.0f);
 }
 
 // ------------------------------------------------------------- kernel
@@ -1028,7 +1260,7 @@ __device__ __forceinline__ void copy16(void* dst, const void* src, size_t bytes)
 // few spills at 64 registers; the lane state is kept small for it (a geometry index
 // instead of the geometry's fields, the ticket recomputed from (instance, id), the
 // warp's ticket pool in shared memory).
-template <bool kCount64, int kMode, int kMasks>
+template <int kMode, int kMasks>
 __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1043,7 +1275,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     uint32_t* s_stream = reinterpret_cast<uint32_t*>(smem + L.stream);
     unsigned long long* s_pool = reinterpret_cast<unsigned long long*>(smem + L.pool);
     uint32_t* s_queue = reinterpret_cast<uint32_t*>(smem + L.queue);
-    unsigned int* s_cnt = reinterpret_cast<unsigned int*>(smem + L.counters);
+    unsigned int* s_cnt = P.smem_counters ? reinterpret_cast<unsigned int*>(smem + L.counters) : nullptr;
 
     copy16(s_prims, P.prims, sizeof(DevPrim) * P.n_prims);
     copy16(s_geoms, P.geoms, sizeof(DevGeom) * P.n_geoms);
@@ -1065,7 +1297,8 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     T.gm = s_gm;
     T.pairs = s_pairs;
     T.geoms = s_geoms;
-    T.n_bm = P.n_bm;
+    T.bm_n = P.bm_n;
+    T.bm_top = 8388608.0f + (P.bm_n - 1.0f);
     T.n_w = P.n_w_all;
     T.bm_lo = P.bm_lo;
     T.bm_inv_h = P.bm_inv_h;
@@ -1074,13 +1307,11 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 
     const int lane = threadIdx.x & 31;
     const unsigned lane_lt = (1u << lane) - 1u;
-    const int ncell = P.nx * P.ny;
-
     Lane S;
     S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
-    S.pid = S.inst = S.k = S.ncoll = 0u;
+    S.pid = S.inst = S.k = 0u;
     S.geom = S.pair = 0;
-    S.ng14 = S.E_per_v2 = 0.0f;
+    S.ng14 = 0.0f;
     bool alive = false;
 
     // per-lane statistics; particles = landed + timed out, flights = landed + timed out + collided
@@ -1175,6 +1406,13 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
             __syncwarp();
             if (lane == 0) s_wpool[2] = qn - (n < qn ? n : qn);
             __syncwarp();
+            // no tickets left and few atoms alive (or every atom, when the run is small):
+            // hand them over to drain_kernel, which follows
+            if (P.pool && (P.drain_live >= 32 || (qn < n && 32 - (int)(n - qn) <= P.drain_live))) {
+                pool_store(P, alive, S);
+                alive = false;
+                if (qn >= n) continue;  // every lane got an atom: there may be more tickets
+            }
         }
         if (!__any_sync(kFull, alive)) break;
 
@@ -1183,97 +1421,20 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
         const int res = flight_step_warp<kMode, kMasks>(alive, S, P, T, s_prims, s_pairs, s_wlist, so);
         c_att += so.attempts;
         if (res == kStepLanded) {
-            // ------------------------------------------------ landing tally
-            const float tb = so.t;
-            const int hb = so.prim;
-            const float E = S.E_per_v2 * S.speed * S.speed;
-            int cell = -1;
-            float cosang = 0.0f;
-            const DevGeom G = s_geoms[S.geom];
-            if (hb == G.substrate()) {
-                const DevPrim& Q = s_prims[G.begin + hb];
-                const float dn = S.dx * Q.nx + S.dy * Q.ny + S.dz * Q.nz;
-                if (dn < 0.0f) {
-                    const float qx = fmaf(tb, S.dx, S.px) - Q.cx, qy = fmaf(tb, S.dy, S.py) - Q.cy,
-                                qz = fmaf(tb, S.dz, S.pz) - Q.cz;
-                    const float a1 = qx * Q.ux + qy * Q.uy + qz * Q.uz;
-                    const float a2 = qx * Q.vx + qy * Q.vy + qz * Q.vz;
-                    const float fx = (a1 + P.half_u) * P.cells_per_mm_u;
-                    const float fy = (a2 + P.half_v) * P.cells_per_mm_v;
-                    if (fx >= 0.0f && fy >= 0.0f && fx <= (float)P.nx && fy <= (float)P.ny) {
-                        const int ix = min((int)fx, P.nx - 1), iy = min((int)fy, P.ny - 1);
-                        cell = iy * P.nx + ix;
-                    }
-                    cosang = -dn;
-                }
-            }
-            if (cell >= 0 && idx_ok(P.status, (long long)S.inst * ncell + cell, (long long)P.n_inst * ncell)) {
-                const size_t ci = (size_t)S.inst * ncell + cell;
-                if (P.counts) {
-                    if (kCount64) atomicAdd(reinterpret_cast<unsigned long long*>(P.counts) + ci, 1ull);
-                    else atomicAdd(reinterpret_cast<unsigned int*>(P.counts) + ci, 1u);
-                }
-                if (P.energy) atomicAdd(P.energy + ci, (double)E);
-                if (P.score) atomicAdd(P.score + ci, (double)S.score);
-                if (kMode == kModeScoreT) atomicAdd(P.score_T + ci, (double)S.scoreT);
-                if (P.hist_E) {
-                    int b = min(max((int)(E * P.ebin_per_eV), 0), P.n_ebins - 1);
-                    atomicAdd(reinterpret_cast<unsigned long long*>(P.hist_E) + (size_t)S.inst * P.n_ebins + b, 1ull);
-                }
-                if (P.hist_A) {
-                    const float th = acosf(fminf(cosang, 1.0f)) * (57.29577951308232f / 90.0f);
-                    int b = min(max((int)(th * (float)P.n_abins), 0), P.n_abins - 1);
-                    atomicAdd(reinterpret_cast<unsigned long long*>(P.hist_A) + (size_t)S.inst * P.n_abins + b, 1ull);
-                }
-            }
-            if (!idx_ok(P.status, hb, P.max_prims)) {
-                // dropped: the checked build reports it
-            } else if (P.smem_counters) atomicAdd(&s_cnt[S.inst * (P.max_prims + 1) + hb], 1u);
-            else if (P.prim_counts)
-                atomicAdd(reinterpret_cast<unsigned long long*>(P.prim_counts) + (size_t)S.inst * P.max_prims + hb, 1ull);
-            if (P.records && idx_ok(P.status, (long long)(s_prefix[S.inst] + S.pid - P.ticket_begin),
-                                    (long long)(P.ticket_end - P.ticket_begin))) {
-                sput_record rec;
-                rec.prim = hb;
-                rec.cell = cell;
-                rec.energy = E;
-                rec.cos_angle = cosang;
-                rec.n_collisions = S.ncoll;
-                rec.score = S.score;
-                P.records[s_prefix[S.inst] + S.pid - P.ticket_begin] = rec;
-            }
+            tally_landed<kMode>(P, S, s_geoms, s_prims, s_cnt, so.t, so.prim);
             ++c_landed;
+            c_coll += S.k - 1u;
             alive = false;
         } else if (res == kStepTimedOut) {
-            if (so.nonfinite) atomicOr(P.status, kStatusNonFinite);
-            if (P.smem_counters) atomicAdd(&s_cnt[S.inst * (P.max_prims + 1) + P.max_prims], 1u);
-            else if (P.timed_out) atomicAdd(reinterpret_cast<unsigned long long*>(P.timed_out) + S.inst, 1ull);
-            if (P.records && idx_ok(P.status, (long long)(s_prefix[S.inst] + S.pid - P.ticket_begin),
-                                    (long long)(P.ticket_end - P.ticket_begin))) {
-                sput_record rec;
-                rec.prim = -1;
-                rec.cell = -1;
-                rec.energy = S.E_per_v2 * S.speed * S.speed;
-                rec.cos_angle = 0.0f;
-                rec.n_collisions = S.ncoll;
-                rec.score = S.score;
-                P.records[s_prefix[S.inst] + S.pid - P.ticket_begin] = rec;
-            }
+            tally_timed_out(P, S, s_cnt, so.nonfinite);
             ++c_timed;
+            c_coll += S.k - 1u;
             alive = false;
-        } else if (res == kStepCollided) {
-            ++c_coll;
         }
     }
 
     // ---------------------------------------------------- flush counters
-    unsigned long long v[kNumStats] = {c_landed + c_timed, c_landed, c_timed, c_landed + c_timed + c_coll, c_coll, c_att};
-#pragma unroll
-    for (int i = 0; i < kNumStats; ++i) {
-        unsigned long long x = v[i];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-        if (lane == 0 && x) atomicAdd(P.stats + i, x);
-    }
+    add_stats(P, c_landed, c_timed, c_coll, c_att);
     if (P.smem_counters) {
         __syncthreads();
         for (int i = threadIdx.x; i < n_cnt; i += blockDim.x) {
@@ -1291,6 +1452,369 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     }
 }
 
+// ------------------------------------------------------------- the last atoms
+// Atoms handed over by transport_kernel: the whole of a small run, and the last ones of a large
+// one.  Trajectories are long-tailed (0.5 Pa: median 12 collisions, longest of 1e5 atoms 734;
+// 3 Pa: 270 and 9652 of 1e6), so a run's end, or all of a small one, lasts as long as the
+// longest trajectory takes, one dependent step after the other: 3.3 us per step in a sparse warp
+// of transport_kernel.  Here G = 8, 16 or 32 lanes carry one atom, G flights at a time, so that
+// what does not depend on the trajectory is done in parallel and little is left on the chain:
+//   1. the lanes draw the batch's random numbers (flight l and its first four partner
+//      attempts in lane l) into shared memory;
+//   2. the collisions, one after the other.  The gas is homogeneous, so velocities follow from
+//      the collisions alone: where the atom is does not enter.  Eight lanes compute the
+//      collision with each of four attempts in either branch of its proposal while the envelope
+//      is looked up and tested, and the accepted lane's velocity is taken (0.1 % of the
+//      collisions need more attempts); lane f keeps the velocity before flight f;
+//   3. lane f works out flight f: the free path, the position (a running sum over the
+//      flights), the surface test.  The first flight that lands ends the atom; the
+//      collisions drawn beyond it are dropped.
+// A warp starts with as many lanes per atom as the pool's size allows, and once the pool is
+// empty the lanes of finished atoms join the others'.  Every number is computed as in the
+// single-lane step, so the results are bit-identical.
+// Bound by the latency of the chain (320 instructions and 1650 cycles per step, 0.82 us, of which
+// 370 wait for the deflection table in L1 or L2).  Measured on a GB300 without and with the
+// drain: single Ni 3e3 atoms 1.8 -> 0.53 ms, 1e5 2.4 -> 1.26 ms, quaternary 4e5 3.0 -> 1.8 ms,
+// 64 primitives at 3 Pa 1e5 atoms 31 -> 14.5 ms, 1e6 59 -> 47 ms.  Runs of 3e4 single-Ni atoms
+// take 0.74 ms when they go to it at once, 0.95 ms when only the last atoms of each warp do;
+// from 1.5e5 atoms on (one per lane of the GPU) the two meet.
+constexpr int kDrawn = 4;
+constexpr int kMinGroupLog2 = 3;
+
+struct DrainWarp {                // by the flight's lane
+    float4 z[32][kDrawn];         // z1, z2, z3, u of an attempt
+    float4 rho[32][kDrawn];       // r3, rho_w, sc_w
+    Impact hit[32];               // the collision after the flight
+    float4 walk[32];              // direction after the flight (diffusion shortcut)
+    uint2 list[32];               // of nearest_hit_masks
+};
+
+struct DrainLayout {
+    size_t prims, geoms, pairs, bm, xh, gm, warps, total;
+};
+
+__host__ __device__ inline DrainLayout drain_layout(const Params& p)
+{
+    DrainLayout L;
+    size_t o = 0;
+    L.warps = o;
+    o = align16(o + sizeof(DrainWarp) * (kDrainThreads / 32));
+    L.prims = o;
+    o = align16(o + sizeof(DevPrim) * p.n_prims);
+    L.geoms = o;
+    o = align16(o + sizeof(DevGeom) * p.n_geoms);
+    L.pairs = o;
+    o = align16(o + sizeof(DevPair) * p.n_pairs);
+    L.bm = o;
+    o = align16(o + sizeof(float4) * p.n_bm);
+    L.xh = o;
+    o = align16(o + sizeof(float) * (p.n_bm + 1));
+    L.gm = o;
+    o = align16(o + sizeof(float4) * (kGMHalf + kGMHalfLo));
+    L.total = o;
+    return L;
+}
+
+template <int kMode, int kMasks>
+__global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr bool kScoreT = kMode == kModeScoreT;
+    const unsigned n_pool = *P.pool_count;
+    const unsigned n_warps = gridDim.x * (kDrainThreads / 32);
+    const unsigned per_warp = (n_pool + n_warps - 1u) / n_warps;
+    int lg = per_warp <= 1u ? 5 : per_warp <= 2u ? 4 : kMinGroupLog2;  // log2 of the lanes per atom
+    if ((unsigned long long)blockIdx.x * (kDrainThreads / 32) * (32u >> lg) >= n_pool) return;
+
+    const DrainLayout L = drain_layout(P);
+    DevPrim* s_prims = reinterpret_cast<DevPrim*>(smem + L.prims);
+    DevGeom* s_geoms = reinterpret_cast<DevGeom*>(smem + L.geoms);
+    DevPair* s_pairs = reinterpret_cast<DevPair*>(smem + L.pairs);
+    float4* s_bm = reinterpret_cast<float4*>(smem + L.bm);
+    float* s_xh = reinterpret_cast<float*>(smem + L.xh);
+    float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
+    DrainWarp& W = reinterpret_cast<DrainWarp*>(smem + L.warps)[threadIdx.x >> 5];
+    copy16(s_prims, P.prims, sizeof(DevPrim) * P.n_prims);
+    copy16(s_geoms, P.geoms, sizeof(DevGeom) * P.n_geoms);
+    copy16(s_pairs, P.pairs, sizeof(DevPair) * P.n_pairs);
+    copy16(s_bm, P.bm_tab, sizeof(float4) * P.n_bm);
+    copy16(s_xh, P.xh_tab, sizeof(float) * (P.n_bm + 1));
+    if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
+    else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
+    __syncthreads();
+
+    TableView T;
+    T.bm = s_bm;
+    T.xh = s_xh;
+    T.w = P.w_tab;
+    T.gm = s_gm;
+    T.pairs = s_pairs;
+    T.geoms = s_geoms;
+    T.bm_n = P.bm_n;
+    T.bm_top = 8388608.0f + (P.bm_n - 1.0f);
+    T.n_w = P.n_w_all;
+    T.bm_lo = P.bm_lo;
+    T.bm_inv_h = P.bm_inv_h;
+    T.status = P.status;
+    T.stream = nullptr;
+
+    const int lane = threadIdx.x & 31;
+    const int A = P.max_attempts;
+    Lane S;  // the group's atom, the same in its lanes
+    S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
+    S.pid = S.inst = S.k = 0u;
+    S.geom = S.pair = 0;
+    S.ng14 = 0.0f;
+    S.diff = false;
+    uint32_t strm = 0u;
+    bool have = false, more = true;  // more: the pool may hold further atoms (warp-uniform)
+    uint32_t c_landed = 0, c_timed = 0, c_coll = 0, c_att = 0;
+
+    for (;;) {
+        int head = lane >> lg << lg, l = lane - head;  // the group's first lane, lane in the group
+        // ---------------------------------------------------- next atoms
+        if (more && __any_sync(kFull, !have)) {
+            unsigned i = 0u;
+            if (!have && l == 0) i = atomicAdd(P.pool_next, 1u);
+            i = __shfl_sync(kFull, i, head);
+            if (!have && i < n_pool) {
+                const float4* q = P.pool + 4 * (size_t)i;
+                const float4 a = q[0], b = q[1], c = q[2];
+                S.px = a.x;
+                S.py = a.y;
+                S.pz = a.z;
+                S.speed = a.w;
+                S.dx = b.x;
+                S.dy = b.y;
+                S.dz = b.z;
+                S.score = b.w;
+                S.pid = __float_as_uint(c.x);
+                S.inst = __float_as_uint(c.y);
+                S.k = __float_as_uint(c.z);
+                S.diff = __float_as_uint(c.w) != 0u;
+                if (kScoreT) S.scoreT = q[3].x;
+                const DevInstance& I = P.inst[S.inst];
+                S.geom = idx_ok(P.status, I.geometry, P.n_geoms) ? I.geometry : 0;
+                S.pair = idx_ok(P.status, I.pair, P.n_pairs) ? I.pair : 0;
+                S.ng14 = I.ng14;
+                strm = I.stream;
+                have = true;
+            }
+            more = !__any_sync(kFull, !have);
+        }
+        if (!more) {
+            // half as many atoms as groups or fewer: twice as many lanes each
+            const unsigned heads = __ballot_sync(kFull, have && l == 0);
+            const int live = __popc(heads);
+            if (live == 0) break;
+            if (lg < 5 && 2 * live <= 32 >> lg) {
+                do ++lg;
+                while (lg < 5 && 2 * live <= 32 >> lg);
+                const int to = lane >> lg;
+                have = to < live;
+                const int src = nth_set_bit(heads, have ? to : 0);
+                S.px = __shfl_sync(kFull, S.px, src);
+                S.py = __shfl_sync(kFull, S.py, src);
+                S.pz = __shfl_sync(kFull, S.pz, src);
+                S.dx = __shfl_sync(kFull, S.dx, src);
+                S.dy = __shfl_sync(kFull, S.dy, src);
+                S.dz = __shfl_sync(kFull, S.dz, src);
+                S.speed = __shfl_sync(kFull, S.speed, src);
+                S.score = __shfl_sync(kFull, S.score, src);
+                if (kScoreT) S.scoreT = __shfl_sync(kFull, S.scoreT, src);
+                if (kMode == kModeWalk) S.diff = __shfl_sync(kFull, (int)S.diff, src) != 0;
+                S.pid = __shfl_sync(kFull, S.pid, src);
+                S.inst = __shfl_sync(kFull, S.inst, src);
+                S.k = __shfl_sync(kFull, S.k, src);
+                S.geom = __shfl_sync(kFull, S.geom, src);
+                S.pair = __shfl_sync(kFull, S.pair, src);
+                S.ng14 = __shfl_sync(kFull, S.ng14, src);
+                strm = __shfl_sync(kFull, strm, src);
+                head = lane >> lg << lg;
+                l = lane - head;
+            }
+        }
+        const int G = 1 << lg;
+
+        // ---------------------------------------------------- 1. random numbers
+        float nl = 0.0f;  // -ln u of the free path of flight l
+        if (have) {
+            const uint32_t k = S.k + 1u + l;
+            const uint4 w = philox(P, S.pid, strm, k, 0u);
+            nl = neg_log_fast(rn(w.x));
+            W.hit[lane] = impact_draw(w);
+            if (kMode == kModeWalk) {
+                float4 d = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                walk_direction(w, d.x, d.y, d.z);
+                W.walk[lane] = d;
+            }
+            if (P.gas_thermal) {
+#pragma unroll 2
+                for (int a = 0; a < kDrawn; ++a) {
+                    const Attempt d = attempt_draw(P, S.pid, strm, k, (uint32_t)a);
+                    W.z[lane][a] = make_float4(d.z1, d.z2, d.z3, d.u);
+                    W.rho[lane][a] = make_float4(d.r3, d.rho_w, d.sc_w, 0.0f);
+                }
+            }
+        }
+        __syncwarp();
+
+        // ---------------------------------------------------- 2. collisions
+        Lane F;  // flight l: the velocity before it, later its position and scores
+        F.pid = S.pid;
+        F.inst = S.inst;
+        F.geom = S.geom;
+        F.pair = S.pair;
+        F.ng14 = S.ng14;
+        F.k = S.k + 1u + l;
+        F.speed = F.dx = F.dy = F.dz = 0.0f;
+        F.diff = false;
+        uint32_t att = 0u;
+        float V2 = 0.0f;
+        const DevPair& pr = s_pairs[S.pair];
+        const int my_a = l & (kDrawn - 1);
+        const bool my_branch = (l & kDrawn) != 0;
+#pragma unroll 1
+        for (int f = 0; f < G; ++f) {
+            if (l == f) {
+                F.speed = S.speed;
+                F.dx = S.dx;
+                F.dy = S.dy;
+                F.dz = S.dz;
+                F.diff = S.diff;
+            }
+            const bool walk = kMode == kModeWalk && S.diff;
+            bool pend = have && !walk;
+            if (kMode == kModeWalk && walk) {
+                const float4 d = W.walk[head + f];
+                S.dx = d.x;
+                S.dy = d.y;
+                S.dz = d.z;
+            }
+            if (kMode == kModeWalk && !__any_sync(kFull, pend)) continue;
+            const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
+            float EA = 0.0f, EB = 0.0f;
+            if (P.gas_thermal) {
+                const float w = w_of(pr, S.speed);
+                EA = wtab_at(T, pr, pr.A_off, w);
+                EB = wtab_at(T, pr, pr.B_off, w);
+            }
+            const Impact h = W.hit[head + f];
+            const float4 z = W.z[head + f][my_a], r = W.rho[head + f][my_a];
+            Attempt d;
+            d.z1 = z.x;
+            d.z2 = z.y;
+            d.z3 = z.z;
+            d.u = z.w;
+            d.r3 = r.x;
+            d.rho_w = r.y;
+            d.sc_w = r.z;
+            for (int a = my_a;;) {
+                // the collision with this lane's attempt in its branch, and whether it is the one
+                float cx = 0.0f, cy = 0.0f, cz = 0.0f;
+                bool acc = true;
+                if (P.gas_thermal) {
+                    float ut, Bm;
+                    const bool weighted = attempt_weighted(d, EA, EB, ut, Bm);
+                    attempt_velocity(P, d, my_branch, cx, cy, cz);
+                    const float hg = attempt_h(T, pr, vx, vy, vz, cx, cy, cz);
+                    acc = a < A && weighted == my_branch &&
+                          (attempt_accept(d, my_branch, ut, Bm, EA, EB, hg) || a == A - 1);
+                }
+                float ns = S.speed, nx = S.dx, ny = S.dy, nz = S.dz;
+                scatter<kMode>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, cx, cy, cz, h);
+                // the first accepted attempt, in either branch
+                const unsigned m = __ballot_sync(kFull, acc) >> head;
+                const unsigned first = (m | m >> kDrawn) & ((1u << kDrawn) - 1u);
+                int src = first ? __ffs(first) - 1 : 0;
+                const uint32_t n_att = (uint32_t)(a - my_a + src) + 1u;
+                if (!((m >> src) & 1u)) src += kDrawn;
+                ns = __shfl_sync(kFull, ns, head + src);
+                nx = __shfl_sync(kFull, nx, head + src);
+                ny = __shfl_sync(kFull, ny, head + src);
+                nz = __shfl_sync(kFull, nz, head + src);
+                const float c2 = kScoreT ? __shfl_sync(kFull, sumsq_xyz(cx, cy, cz), head + src) : 0.0f;
+                if (pend && first) {
+                    S.speed = ns;
+                    S.dx = nx;
+                    S.dy = ny;
+                    S.dz = nz;
+                    if (l == f) {
+                        att = P.gas_thermal ? n_att : 0u;
+                        V2 = c2;
+                    }
+                    if (kMode == kModeWalk && energy_of(P, S.inst, S.speed) < P.E_switch) S.diff = true;
+                    pend = false;
+                }
+                if (!__any_sync(kFull, pend)) break;
+                // rare: none of the drawn attempts; the group draws four more
+                a += kDrawn;
+                d = attempt_draw(P, S.pid, strm, S.k + 1u + f, (uint32_t)a);
+            }
+        }
+
+        // ---------------------------------------------------- 3. flights
+        float inv_lam = 0.0f, ell = 0.0f, Gv = 0.0f;
+        if (have) flight_length<kMode>(F, P, T, pr, nl, inv_lam, ell, Gv);
+        // positions and scores before each flight: running sums over the batch, in order
+        const float gain = score_gain(ell, inv_lam);
+        const float aT = kScoreT ? score_T_rate(P, Gv) : 0.0f;
+        const float cT = kScoreT ? score_T_partner(P, V2, Gv) : 0.0f;
+        F.px = S.px;
+        F.py = S.py;
+        F.pz = S.pz;
+        F.score = S.score;
+        F.scoreT = S.scoreT;
+#pragma unroll 8
+        for (int f = 0; f < G; ++f) {
+            const int src = head + f;
+            const float e = __shfl_sync(kFull, ell, src);
+            S.px = fmaf(e, __shfl_sync(kFull, F.dx, src), S.px);
+            S.py = fmaf(e, __shfl_sync(kFull, F.dy, src), S.py);
+            S.pz = fmaf(e, __shfl_sync(kFull, F.dz, src), S.pz);
+            const float gn = __shfl_sync(kFull, gain, src);
+            S.score += gn;
+            if (kScoreT) {
+                S.scoreT = fmaf(__shfl_sync(kFull, aT, src), gn, S.scoreT);
+                if (P.gas_thermal) S.scoreT = fmaf(__shfl_sync(kFull, cT, src), P.inv_T, S.scoreT);
+            }
+            if (l > f) {
+                F.px = S.px;
+                F.py = S.py;
+                F.pz = S.pz;
+                F.score = S.score;
+                F.scoreT = S.scoreT;
+            }
+        }
+        float tb = CUDART_INF_F;
+        int hb = -1;
+        if (kMasks) nearest_hit_masks<kMasks ? kMasks : 1>(have, F, P, T, s_prims, W.list, ell, tb, hb);
+        else if (have) nearest_hit_loop(F, P, T, s_prims, ell, tb, hb);
+        StepOut out;
+        out.Gv = Gv;
+        int res = kStepNone;
+        if (have) res = flight_end<kMode>(F, P, out, inv_lam, ell, tb, hb);
+        const unsigned ends = (__ballot_sync(kFull, res == kStepLanded || res == kStepTimedOut) >> head) &
+                              (0xffffffffu >> (32 - G));
+        const int last = ends ? __ffs(ends) - 1 : G;
+        if (have && l < last) c_att += att;
+        if (have && l == last) {
+            if (res == kStepLanded) {
+                tally_landed<kMode>(P, F, s_geoms, s_prims, nullptr, out.t, out.prim);
+                ++c_landed;
+            } else {
+                tally_timed_out(P, F, nullptr, out.nonfinite);
+                ++c_timed;
+            }
+            c_coll += F.k - 1u;
+        }
+        S.k += G;
+        if (ends) have = false;
+        __syncwarp();
+    }
+    add_stats(P, c_landed, c_timed, c_coll, c_att);
+}
+
 // ------------------------------------------------------------- probes
 __global__ void probe_kernel(const Params P, int what, int idx, int n, const double* x, double* y)
 {
@@ -1306,7 +1830,8 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
     T.gm = s_gm;
     T.pairs = P.pairs;
     T.geoms = P.geoms;
-    T.n_bm = P.n_bm;
+    T.bm_n = P.bm_n;
+    T.bm_top = 8388608.0f + (P.bm_n - 1.0f);
     T.n_w = P.n_w_all;
     T.bm_lo = P.bm_lo;
     T.bm_inv_h = P.bm_inv_h;
@@ -1318,9 +1843,9 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
         const bool valid = i < n;
         Lane S;
         S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
-        S.pid = S.inst = S.k = S.ncoll = 0u;
+        S.pid = S.inst = S.k = 0u;
         S.geom = S.pair = 0;
-        S.ng14 = S.E_per_v2 = 0.0f;
+        S.ng14 = 0.0f;
         double* o = valid ? y + (size_t)i * kTraceRows * 10 : nullptr;
         if (valid) {
             start_particle(S, P, (uint32_t)idx, (uint32_t)x[i]);
@@ -1361,8 +1886,10 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
         // the collision's path: table inside its range, direct integration outside
         const float eps = (float)x[2 * i], ub = (float)x[2 * i + 1];
         const float le = logf(eps);
-        float q;
-        if (chi_table_q(P.chi_tab, P.status, le, 0.5f * logf(ub), q)) {
+        float q, ty;
+        int j;
+        const bool column = chi_table_column(0.5f * logf(ub), j, ty);
+        if (chi_table_q(P.chi_tab, P.status, le, j, ty, q) && column) {
             y[i] = 2.0 * atan(exp((double)q));
         } else {
             const float beta = bmax_eval(T, le) * sqrtf(ub);
@@ -1404,51 +1931,61 @@ namespace {
 
 using KernelFn = void (*)(const Params);
 
-// the instances [count type][mode][words of the cell masks, 0 = the counted loop]
-#define SPUT_KERNELS(c64, mode) \
-    {transport_kernel<c64, mode, 0>, transport_kernel<c64, mode, 1>, transport_kernel<c64, mode, 2>}
-KernelFn kernel_for(int count64, int mode, int words)
-{
-    static const KernelFn tab[2][3][3] = {
-        {SPUT_KERNELS(false, kModePlain), SPUT_KERNELS(false, kModeScoreT), SPUT_KERNELS(false, kModeWalk)},
-        {SPUT_KERNELS(true, kModePlain), SPUT_KERNELS(true, kModeScoreT), SPUT_KERNELS(true, kModeWalk)}};
-    return tab[count64 ? 1 : 0][mode][words];
-}
+// the instances [mode][words of the cell masks, 0 = the counted loop]
+#define SPUT_KERNELS(k, mode) {k<mode, 0>, k<mode, 1>, k<mode, 2>}
+#define SPUT_KERNEL_TABLE(k) {SPUT_KERNELS(k, kModePlain), SPUT_KERNELS(k, kModeScoreT), SPUT_KERNELS(k, kModeWalk)}
+const KernelFn kTransport[3][3] = SPUT_KERNEL_TABLE(transport_kernel);
+const KernelFn kDrain[3][3] = SPUT_KERNEL_TABLE(drain_kernel);
+#undef SPUT_KERNEL_TABLE
 #undef SPUT_KERNELS
 
-}  // namespace
-
-int transport_max_blocks_per_sm(int count64, int threads, size_t smem)
+// the smallest occupancy of a kernel's instances
+int min_blocks_per_sm(const KernelFn (&k)[3][3], int threads, size_t smem)
 {
-    // the smallest occupancy of the instances of this count type
     int m = 1 << 30;
     for (int mode = 0; mode < 3; ++mode)
         for (int words = 0; words < 3; ++words) {
             int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel_for(count64, mode, words), threads, smem) !=
-                cudaSuccess)
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k[mode][words], threads, smem) != cudaSuccess)
                 return 0;
             m = nb < m ? nb : m;
         }
     return m;
 }
 
+int instance_mode(const Params& p) { return p.score_T ? kModeScoreT : (p.E_switch > 0.0f ? kModeWalk : kModePlain); }
+
+}  // namespace
+
+size_t drain_smem_bytes(const Params& p) { return drain_layout(p).total; }
+
+int transport_max_blocks_per_sm(int threads, size_t smem) { return min_blocks_per_sm(kTransport, threads, smem); }
+
+int drain_max_blocks_per_sm(size_t smem) { return min_blocks_per_sm(kDrain, kDrainThreads, smem); }
+
 int transport_configure(int max_dynamic_smem)
 {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    for (int c64 = 0; c64 < 2; ++c64)
-        for (int mode = 0; mode < 3; ++mode)
-            for (int words = 0; words < 3; ++words) {
-                const cudaError_t e = cudaFuncSetAttribute(kernel_for(c64, mode, words), a, max_dynamic_smem);
-                if (e != cudaSuccess) return (int)e;
-            }
+    for (int mode = 0; mode < 3; ++mode)
+        for (int words = 0; words < 3; ++words) {
+            cudaError_t e = cudaFuncSetAttribute(kTransport[mode][words], a, max_dynamic_smem);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kDrain[mode][words], a, max_dynamic_smem);
+            if (e != cudaSuccess) return (int)e;
+        }
     return 0;
 }
 
-int transport_launch(const Params& p, int count64, int blocks, int threads, size_t smem, void* stream)
+int transport_launch(const Params& p, int blocks, int threads, size_t smem, void* stream)
 {
-    const int mode = p.score_T ? kModeScoreT : (p.E_switch > 0.0f ? kModeWalk : kModePlain);
-    kernel_for(count64, mode, p.cell_mask ? p.cell_words : 0)<<<blocks, threads, smem, reinterpret_cast<cudaStream_t>(stream)>>>(p);
+    kTransport[instance_mode(p)][p.cell_mask ? p.cell_words : 0]<<<blocks, threads, smem,
+                                                                   reinterpret_cast<cudaStream_t>(stream)>>>(p);
+    return (int)cudaGetLastError();
+}
+
+int drain_launch(const Params& p, int blocks, size_t smem, void* stream)
+{
+    kDrain[instance_mode(p)][p.cell_mask ? p.cell_words : 0]<<<blocks, kDrainThreads, smem,
+                                                               reinterpret_cast<cudaStream_t>(stream)>>>(p);
     return (int)cudaGetLastError();
 }
 
