@@ -769,8 +769,10 @@ __device__ int flight_end(Lane& S, const Params& P, StepOut& out, float inv_lam,
     return kStepCollided;
 }
 
-// correctly rounded 1/d for d = 1..33 (the values __frcp_rn gives), indexed by warp-uniform d
-__constant__ float kRcpSmall[34] = {0.0f, 1.0f / 1.0f, 1.0f / 2.0f, 1.0f / 3.0f, 1.0f / 4.0f, 1.0f / 5.0f, 1.0f / 6.0f, 1.0f / 7.0f, 1.0f / 8.0f, 1.0f / 9.0f, 1.0f / 10.0f, 1.0f / 11.0f, 1.0f / 12.0f, 1.0f / 13.0f, 1.0f / 14.0f, 1.0f / 15.0f, 1.0f / 16.0f, 1.0f / 17.0f, 1.0f / 18.0f, 1.0f / 19.0f, 1.0f / 20.0f, 1.0f / 21.0f, 1.0f / 22.0f, 1.0f / 23.0f, 1.0f / 24.0f, 1.0f / 25.0f, 1.0f / 26.0f, 1.0f / 27.0f, 1.0f / 28.0f, 1.0f / 29.0f, 1.0f / 30.0f, 1.0f / 31.0f, 1.0f / 32.0f, 1.0f / 33.0f};
+// ceil(2^11 / d) for d = 1..33: floor(l / d) = (l kInv11[d]) >> 11 for l <= 32 (the excess, below
+// l / 2^11 <= 1/64, stays under the 1/33 that separates a quotient from the next integer)
+__constant__ int kInv11[34] = {0,   2048, 1024, 683, 512, 410, 342, 293, 256, 228, 205, 187, 171, 158, 147, 137, 128,
+                               121, 114,  108,  103, 98,  94,  90,  86,  82,  79,  76,  74,  71,  69,  67,  64,  63};
 
 // position of the n-th (0-based) set bit of mask; mask has more than n set bits
 __device__ __forceinline__ int nth_set_bit(unsigned mask, int n)
@@ -878,35 +880,35 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
     int next_a = 0;
     Vx = Vy = Vz = 0.0f;
     attempts = 0;
+    // Most lanes pending: each tries its first attempt itself, without the hand-out below.
+    bool own = __popc(pending) > 16;
     while (pending) {
-        // np pending particles share 32 lanes: the first `extra` get m + 1 lanes, the rest m
-        // (small-integer quotients through a correctly rounded reciprocal from a
-        // table, d = 1..33: 32/np is exact as np <= 32 divides 32 only as a power of
-        // two, and (l + 1/2)/d stays at least 1/66 away from an integer for l < 32)
-        const int np = __popc(pending);
-        const int m = (int)(32.0f * kRcpSmall[np]);
-        const int extra = 32 - m * np;
-        const int cut = extra * (m + 1);
-        int slot, j;
-        if (lane < cut) {
-            slot = (int)(((float)lane + 0.5f) * kRcpSmall[m + 1]);
-            j = lane - slot * (m + 1);
-        } else {
-            const int r = (int)(((float)(lane - cut) + 0.5f) * kRcpSmall[m]);
-            slot = extra + r;
-            j = lane - cut - r * m;
+        uint32_t o_pid = pid, o_strm = strm, o_k = k;
+        int o_pair = pair, o_next = next_a, j = need ? 0 : A, m = 1, extra = 32, cut = 64;
+        float o_vx = vx, o_vy = vy, o_vz = vz, o_A = EA, o_B = EB;
+        if (!own) {
+            // np pending particles share 32 lanes: the first `extra` get m + 1 lanes, the rest m
+            const int np = __popc(pending);
+            m = (32 * kInv11[np]) >> 11;
+            extra = 32 - m * np;
+            cut = extra * (m + 1);
+            const bool more = lane < cut;
+            const int d = more ? m + 1 : m, at = more ? lane : lane - cut;
+            const int q = (at * kInv11[d]) >> 11;
+            j = at - q * d;
+            const int slot = more ? q : extra + q;
+            const int owner = nth_set_bit(pending, slot);
+            o_pid = __shfl_sync(kFull, pid, owner);
+            o_strm = __shfl_sync(kFull, strm, owner);
+            o_k = __shfl_sync(kFull, k, owner);
+            o_pair = __shfl_sync(kFull, pair, owner);
+            o_vx = __shfl_sync(kFull, vx, owner);
+            o_vy = __shfl_sync(kFull, vy, owner);
+            o_vz = __shfl_sync(kFull, vz, owner);
+            o_A = __shfl_sync(kFull, EA, owner);
+            o_B = __shfl_sync(kFull, EB, owner);
+            o_next = __shfl_sync(kFull, next_a, owner);
         }
-        const int owner = nth_set_bit(pending, slot);
-        const uint32_t o_pid = __shfl_sync(kFull, pid, owner);
-        const uint32_t o_strm = __shfl_sync(kFull, strm, owner);
-        const uint32_t o_k = __shfl_sync(kFull, k, owner);
-        const int o_pair = __shfl_sync(kFull, pair, owner);
-        const float o_vx = __shfl_sync(kFull, vx, owner);
-        const float o_vy = __shfl_sync(kFull, vy, owner);
-        const float o_vz = __shfl_sync(kFull, vz, owner);
-        const float o_A = __shfl_sync(kFull, EA, owner);
-        const float o_B = __shfl_sync(kFull, EB, owner);
-        const int o_next = __shfl_sync(kFull, next_a, owner);
         const int a = o_next + j;
         bool acc = false;
         float cx = 0.0f, cy = 0.0f, cz = 0.0f;
@@ -920,6 +922,18 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
             acc = attempt_accept(d, weighted, ut, Bm, o_A, o_B, hg) || a == A - 1;
         }
         const unsigned accm = __ballot_sync(kFull, acc);
+        if (own) {
+            if (acc) {
+                Vx = cx;
+                Vy = cy;
+                Vz = cz;
+                attempts = 1;
+            }
+            next_a = 1;
+            pending &= ~accm;
+            own = false;
+            continue;
+        }
         const bool is_owner = (pending >> lane) & 1u;
         int src = lane, first = 0;
         bool done = false;
