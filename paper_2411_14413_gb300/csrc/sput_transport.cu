@@ -1163,11 +1163,19 @@ template <int kMode>
 __device__ __forceinline__ void tally_landed(const Params& P, const Lane& S, const DevGeom* geoms, const DevPrim* prims,
                                              unsigned int* s_cnt, float tb, int hb)
 {
+    // every landing counts on its primitive; few (a tenth) reach the substrate
+    if (!idx_ok(P.status, hb, P.max_prims)) {
+        // dropped: the checked build reports it
+    } else if (s_cnt) atomicAdd(&s_cnt[S.inst * (P.max_prims + 1) + hb], 1u);
+    else if (P.prim_counts)
+        atomicAdd(reinterpret_cast<unsigned long long*>(P.prim_counts) + (size_t)S.inst * P.max_prims + hb, 1ull);
+    const DevGeom G = geoms[S.geom];
+    const bool substrate = hb == G.substrate();
+    if (!substrate && !P.records) return;
     const float E = energy_of(P, S.inst, S.speed);
     int cell = -1;
     float cosang = 0.0f;
-    const DevGeom G = geoms[S.geom];
-    if (hb == G.substrate()) {
+    if (substrate) {
         const DevPrim& Q = prims[G.begin + hb];
         const float dn = S.dx * Q.nx + S.dy * Q.ny + S.dz * Q.nz;
         if (dn < 0.0f) {
@@ -1204,11 +1212,6 @@ __device__ __forceinline__ void tally_landed(const Params& P, const Lane& S, con
             atomicAdd(reinterpret_cast<unsigned long long*>(P.hist_A) + (size_t)S.inst * P.n_abins + b, 1ull);
         }
     }
-    if (!idx_ok(P.status, hb, P.max_prims)) {
-        // dropped: the checked build reports it
-    } else if (s_cnt) atomicAdd(&s_cnt[S.inst * (P.max_prims + 1) + hb], 1u);
-    else if (P.prim_counts)
-        atomicAdd(reinterpret_cast<unsigned long long*>(P.prim_counts) + (size_t)S.inst * P.max_prims + hb, 1ull);
     if (P.records) write_record(P, S, hb, cell, E, cosang);
 }
 
