@@ -117,15 +117,17 @@ struct alignas(16) DevPair {
 };
 
 struct alignas(16) DevInstance {
-    int geometry, cathode, pair;
-    uint32_t n;           // particles
+    // read together at every flight (load_conditions)
     float ng14;           // n_gas (mm^-3) * 1e-14: inverse mean free path = ng14 * K / v
+    uint32_t stream;      // word 1 of every Philox counter of this instance's particles
+    int geometry, pair;
+    int cathode;
+    uint32_t n;           // particles
     float thompson_q;     // E_max / (E_max + U_s)
     float U_s;
     float kLambda;        // d E_max / d E_i = k Lambda
+    uint32_t pad;
     unsigned long long ticket_begin;
-    uint32_t stream;      // word 1 of every Philox counter of this instance's particles
-    uint32_t pad2;
 };
 
 // Everything the transport kernel needs; passed by value (kernel parameter).

@@ -101,14 +101,7 @@ struct TableView {
     float bm_n, bm_top;  // pieces of bm, and 2^23 + pieces - 1
     float bm_lo, bm_inv_h;
     unsigned int* status;
-    const uint32_t* stream;  // Philox stream word per instance (shared memory), or null: read P.inst
 };
-
-// word 1 of the Philox counters of instance `inst`'s particles
-__device__ __forceinline__ uint32_t stream_of(const TableView& T, const Params& P, uint32_t inst)
-{
-    return T.stream ? T.stream[inst] : P.inst[inst].stream;
-}
 
 __device__ __forceinline__ float bmax_eval(const TableView& T, float ln_eps)
 {
@@ -322,9 +315,22 @@ struct Lane {
     float scoreT;  // d ln p(path)/dT (kernel instance with the temperature score only)
     bool diff;     // thermalised: random walk of the diffusion shortcut
     uint32_t pid, inst, k;  // k flights begun: k - 1 collisions while the k-th lasts
-    int geom, pair;  // geometry index (its record is read from TableView::geoms), gas pair
+    // of the instance (load_conditions)
     float ng14;
+    uint32_t strm;
+    int geom, pair;  // geometry index (its record is read from TableView::geoms), gas pair
 };
+
+// The instance's conditions that a flight needs, 16 bytes through L1.  The transport reads them
+// anew for every flight instead of carrying them in registers from one to the next.
+__device__ __forceinline__ void load_conditions(Lane& S, const Params& P)
+{
+    const uint4 c = __ldg(reinterpret_cast<const uint4*>(P.inst + S.inst));
+    S.ng14 = __uint_as_float(c.x);
+    S.strm = c.y;
+    S.geom = idx_ok(P.status, (int)c.z, P.n_geoms) ? (int)c.z : 0;
+    S.pair = idx_ok(P.status, (int)c.w, P.n_pairs) ? (int)c.w : 0;
+}
 
 __device__ __forceinline__ float racetrack_r(const DevCathode& C, const float4* rt_tab, int rt_n, int n_rt_all,
                                             unsigned int* status, float u)
@@ -508,13 +514,8 @@ __device__ Launch prepare_launch(const Params& P, uint32_t inst, uint32_t pid)
 // The lane takes up the prepared particle.
 __device__ void start_from(Lane& S, const Params& P, const Launch& L)
 {
-    const uint32_t inst = L.inst;
-    const DevInstance& I = P.inst[inst];
-    S.inst = inst;
+    S.inst = L.inst;
     S.pid = L.pid;
-    S.geom = idx_ok(P.status, I.geometry, P.n_geoms) ? I.geometry : 0;
-    S.pair = idx_ok(P.status, I.pair, P.n_pairs) ? I.pair : 0;
-    S.ng14 = I.ng14;
     S.px = L.px;
     S.py = L.py;
     S.pz = L.pz;
@@ -587,7 +588,7 @@ __device__ void flight_begin(Lane& S, const Params& P, const TableView& T, const
                              uint4& w, float& inv_lam, float& ell)
 {
     S.k += 1u;
-    w = philox(P, S.pid, stream_of(T, P, S.inst), S.k, 0u);
+    w = philox(P, S.pid, S.strm, S.k, 0u);
     flight_length<kMode>(S, P, T, pairs[S.pair], neg_log_fast(rn(w.x)), inv_lam, ell, out.Gv);
 }
 
@@ -1070,6 +1071,7 @@ template <int kMode, int kMasks>
 __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const TableView& T, const DevPrim* prims,
                                 const DevPair* pairs, uint2* list, StepOut& out)
 {
+    load_conditions(S, P);
     uint4 w = make_uint4(0u, 0u, 0u, 0u);
     int res = kStepNone;
     out.attempts = 0;
@@ -1094,8 +1096,7 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
             EA = wtab_at(T, pr, pr.A_off, w);
             EB = wtab_at(T, pr, pr.B_off, w);
         }
-        // the owner's Philox stream word travels with it (one shuffle instead of a lookup per attempt)
-        partner_sample_warp(coll, P, T, pairs, S.pid, stream_of(T, P, S.inst), S.k, S.pair, vx, vy, vz, EA, EB, Vx,
+        partner_sample_warp(coll, P, T, pairs, S.pid, S.strm, S.k, S.pair, vx, vy, vz, EA, EB, Vx,
                             Vy, Vz, out.attempts);
         if (kScoreT && coll)
             S.scoreT = fmaf(score_T_partner(P, sumsq_xyz(Vx, Vy, Vz), out.Gv), P.inv_T, S.scoreT);
@@ -1225,7 +1226,7 @@ __device__ __forceinline__ void tally_timed_out(const Params& P, const Lane& S, 
 
 // ------------------------------------------------------------- kernel
 struct SmemLayout {
-    size_t prims, geoms, pairs, bm, prefix, xh, gm, stream, pool, queue, list, counters, total;
+    size_t prims, geoms, pairs, bm, prefix, xh, gm, pool, queue, list, counters, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -1248,8 +1249,6 @@ __host__ __device__ inline SmemLayout smem_layout(const Params& p)
     o = align16(o + sizeof(float) * (p.n_bm + 1));
     L.gm = o;
     o = align16(o + sizeof(float4) * (kGMHalf + kGMHalfLo));
-    L.stream = o;
-    o = align16(o + sizeof(uint32_t) * p.n_inst);
     L.pool = o;
     o = align16(o + sizeof(unsigned long long) * 4 * 8);
     L.queue = o;
@@ -1289,7 +1288,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     unsigned long long* s_prefix = reinterpret_cast<unsigned long long*>(smem + L.prefix);
     float* s_xh = reinterpret_cast<float*>(smem + L.xh);
     float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
-    uint32_t* s_stream = reinterpret_cast<uint32_t*>(smem + L.stream);
     unsigned long long* s_pool = reinterpret_cast<unsigned long long*>(smem + L.pool);
     uint32_t* s_queue = reinterpret_cast<uint32_t*>(smem + L.queue);
     unsigned int* s_cnt = P.smem_counters ? reinterpret_cast<unsigned int*>(smem + L.counters) : nullptr;
@@ -1302,7 +1300,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     copy16(s_xh, P.xh_tab, sizeof(float) * (P.n_bm + 1));
     if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
     else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
-    for (int i = threadIdx.x; i < P.n_inst; i += blockDim.x) s_stream[i] = P.inst[i].stream;
     const int n_cnt = P.smem_counters ? P.n_inst * (P.max_prims + 1) : 0;
     for (int i = threadIdx.x; i < n_cnt; i += blockDim.x) s_cnt[i] = 0u;
     __syncthreads();
@@ -1320,7 +1317,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     T.bm_lo = P.bm_lo;
     T.bm_inv_h = P.bm_inv_h;
     T.status = P.status;
-    T.stream = s_stream;
 
     const int lane = threadIdx.x & 31;
     const unsigned lane_lt = (1u << lane) - 1u;
@@ -1328,6 +1324,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
     S.pid = S.inst = S.k = 0u;
     S.geom = S.pair = 0;
+    S.strm = 0u;
     S.ng14 = 0.0f;
     bool alive = false;
 
@@ -1573,7 +1570,6 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     T.bm_lo = P.bm_lo;
     T.bm_inv_h = P.bm_inv_h;
     T.status = P.status;
-    T.stream = nullptr;
 
     const int lane = threadIdx.x & 31;
     const int A = P.max_attempts;
@@ -1581,9 +1577,9 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
     S.pid = S.inst = S.k = 0u;
     S.geom = S.pair = 0;
+    S.strm = 0u;
     S.ng14 = 0.0f;
     S.diff = false;
-    uint32_t strm = 0u;
     bool have = false, more = true;  // more: the pool may hold further atoms (warp-uniform)
     uint32_t c_landed = 0, c_timed = 0, c_coll = 0, c_att = 0;
 
@@ -1610,11 +1606,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
                 S.k = __float_as_uint(c.z);
                 S.diff = __float_as_uint(c.w) != 0u;
                 if (kScoreT) S.scoreT = q[3].x;
-                const DevInstance& I = P.inst[S.inst];
-                S.geom = idx_ok(P.status, I.geometry, P.n_geoms) ? I.geometry : 0;
-                S.pair = idx_ok(P.status, I.pair, P.n_pairs) ? I.pair : 0;
-                S.ng14 = I.ng14;
-                strm = I.stream;
+                load_conditions(S, P);
                 have = true;
             }
             more = !__any_sync(kFull, !have);
@@ -1646,7 +1638,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
                 S.geom = __shfl_sync(kFull, S.geom, src);
                 S.pair = __shfl_sync(kFull, S.pair, src);
                 S.ng14 = __shfl_sync(kFull, S.ng14, src);
-                strm = __shfl_sync(kFull, strm, src);
+                S.strm = __shfl_sync(kFull, S.strm, src);
                 head = lane >> lg << lg;
                 l = lane - head;
             }
@@ -1657,7 +1649,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
         float nl = 0.0f;  // -ln u of the free path of flight l
         if (have) {
             const uint32_t k = S.k + 1u + l;
-            const uint4 w = philox(P, S.pid, strm, k, 0u);
+            const uint4 w = philox(P, S.pid, S.strm, k, 0u);
             nl = neg_log_fast(rn(w.x));
             W.hit[lane] = impact_draw(w);
             if (kMode == kModeWalk) {
@@ -1668,7 +1660,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
             if (P.gas_thermal) {
 #pragma unroll 2
                 for (int a = 0; a < kDrawn; ++a) {
-                    const Attempt d = attempt_draw(P, S.pid, strm, k, (uint32_t)a);
+                    const Attempt d = attempt_draw(P, S.pid, S.strm, k, (uint32_t)a);
                     W.z[lane][a] = make_float4(d.z1, d.z2, d.z3, d.u);
                     W.rho[lane][a] = make_float4(d.r3, d.rho_w, d.sc_w, 0.0f);
                 }
@@ -1766,7 +1758,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
                 if (!__any_sync(kFull, pend)) break;
                 // rare: none of the drawn attempts; the group draws four more
                 a += kDrawn;
-                d = attempt_draw(P, S.pid, strm, S.k + 1u + f, (uint32_t)a);
+                d = attempt_draw(P, S.pid, S.strm, S.k + 1u + f, (uint32_t)a);
             }
         }
 
@@ -1853,7 +1845,6 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
     T.bm_lo = P.bm_lo;
     T.bm_inv_h = P.bm_inv_h;
     T.status = P.status;
-    T.stream = nullptr;
     if (what == SPUT_PROBE_TRACE) {
         // state after each flight of particle x[i] of instance idx, kTraceRows rows of 10;
         // the flight step is warp-collective, so lanes past n take part without a particle
@@ -1862,6 +1853,7 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
         S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
         S.pid = S.inst = S.k = 0u;
         S.geom = S.pair = 0;
+        S.strm = 0u;
         S.ng14 = 0.0f;
         double* o = valid ? y + (size_t)i * kTraceRows * 10 : nullptr;
         if (valid) {
