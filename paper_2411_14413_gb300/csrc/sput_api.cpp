@@ -318,7 +318,7 @@ static sput_status pack_instances(sput_scene* S)
         const double v = 1.0 / std::sqrt((double)S->dcath[S->dinst[i].cathode].E_per_v2);
         const double x = std::min(std::log(1.0 + v * pr.inv_s) * pr.w_inv_h, (double)pr.n_w);
         const int j = std::min((int)x, pr.n_w - 1);
-        const float4 c = S->wtab[pr.K_off + j];
+        const float4 c = S->wtab[pr.K_off + 3 * j];
         const double t = x - j, K = c.x + t * (c.y + t * (c.z + t * c.w));
         const double inv_lambda = S->dinst[i].ng14 * (S->physics.gas_motion == SPUT_GAS_THERMAL ? K / v : K);
         S->mean_inv_lambda += inv_lambda * ((double)S->dinst[i].n / (double)std::max(1ull, S->n_tickets));
@@ -552,11 +552,12 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
         D.m2M = (float)(pp.m2 / (pp.m1 + pp.m2));
         D.hard_sphere = hard ? 1 : 0;
         D.K_off = (int)S->wtab.size();
-        S->wtab.insert(S->wtab.end(), K.begin(), K.end());
-        D.A_off = (int)S->wtab.size();
-        S->wtab.insert(S->wtab.end(), EA.begin(), EA.end());
-        D.B_off = (int)S->wtab.size();
-        S->wtab.insert(S->wtab.end(), EB.begin(), EB.end());
+        for (size_t i = 0; i < K.size(); ++i) {
+            S->wtab.push_back(K[i]);
+            S->wtab.push_back(EA[i]);
+            S->wtab.push_back(EB[i]);
+        }
+        D.pad_i[0] = D.pad_i[1] = 0;
         g_tabs[p] = std::move(Gt);
         D.sigma_D = S->physics.thermal_switch_eV > 0.0 ? (float)sigma_D64(pp, S->bt, S->chamber.gas_T) : 0.0f;
         D.n_w = n_w;

@@ -106,8 +106,9 @@ struct alignas(16) DevPair {
     float m1M;          // m1 / (m1 + m2)
     float m2M;          // m2 / (m1 + m2)
     int hard_sphere;
-    int K_off;          // float4 offset of the <sigma g>(w) table
-    int A_off, B_off;   // float4 offsets of the rejection-envelope coefficient tables A(w), B(w)
+    int K_off;          // float4 offset of the pieces of <sigma g>(w) and of the rejection-envelope
+                        // coefficients A(w), B(w): three float4 per interval
+    int pad_i[2];
     int n_w;            // intervals of the w tables
     float w_inv_h;      // 1 / Delta w
     float inv_s;        // 1 / s_gas, w = ln(1 + v / s_gas)

@@ -123,21 +123,27 @@ __device__ __forceinline__ float xh_eval(const TableView& T, float ln_eps)
 // (about 4e-7 absolute) moves K, A and B far less than their interpolation error.
 __device__ __forceinline__ float w_of(const DevPair& pr, float v) { return __logf(1.0f + v * pr.inv_s); }
 
-// K(v), A(v), B(v) or G(v) of a pair: cubic pieces in w = ln(1 + v/s), at a given w.  The
-// tables are read through L1 from global memory (a few KB per pair, L1-resident), which
-// keeps them out of shared memory so that four blocks fit on an SM.
-__device__ __forceinline__ float wtab_at(const TableView& T, const DevPair& pr, int off, float w)
+// K(v), A(v), B(v) and G(v) of a pair: cubic pieces in w = ln(1 + v/s).  K, A and B lie beside one
+// another (three float4 per piece), so one cell lookup serves all three.  The tables are read
+// through L1 from global memory (a few KB per pair, L1-resident), which keeps them out of
+// shared memory so that four blocks fit on an SM.
+enum { kTabK = 0, kTabA = 1, kTabB = 2 };
+
+__device__ __forceinline__ void wtab_cell(const DevPair& pr, float v, int& i, float& t)
 {
-    if (!idx_ok(T.status, (long long)off + pr.n_w - 1, T.n_w) || !idx_ok(T.status, off, T.n_w)) return 0.0f;
-    int i;
-    float t;
-    table_cell(fminf(fmaxf(w * pr.w_inv_h, 0.0f), pr.w_n), pr.w_top, i, t);
-    return cubic(__ldg(T.w + off + i), t);
+    table_cell(fminf(fmaxf(w_of(pr, v) * pr.w_inv_h, 0.0f), pr.w_n), pr.w_top, i, t);
 }
 
-__device__ __forceinline__ float wtab_eval(const TableView& T, const DevPair& pr, int off, float v)
+__device__ __forceinline__ float wtab_at(const TableView& T, const DevPair& pr, int which, int i, float t)
 {
-    return wtab_at(T, pr, off, w_of(pr, v));
+    if (!idx_ok(T.status, (long long)pr.K_off + 3 * i + which, T.n_w)) return 0.0f;
+    return cubic(__ldg(T.w + pr.K_off + 3 * i + which), t);
+}
+
+__device__ __forceinline__ float wtab_G(const TableView& T, const DevPair& pr, int i, float t)
+{
+    if (!idx_ok(T.status, (long long)pr.G_off + i, T.n_w)) return 0.0f;
+    return cubic(__ldg(T.w + pr.G_off + i), t);
 }
 
 // sigma(g) g in A^2 km/s
@@ -548,24 +554,19 @@ struct StepOut {
     float Gv;       // d ln K / d ln s at the flight's speed (temperature score only)
 };
 
-// Inverse mean free path at the atom's speed and the flight length, nl = -ln u; Gv =
-// d ln K / d ln s at its speed (temperature score only).
+// Inverse mean free path at the atom's speed (cell i, t of its pair's tables) and the flight
+// length, nl = -ln u; Gv = d ln K / d ln s at its speed (temperature score only).
 template <int kMode>
 __device__ __forceinline__ void flight_length(const Lane& S, const Params& P, const TableView& T, const DevPair& pr,
-                                              float nl, float& inv_lam, float& ell, float& Gv)
+                                              int i, float t, float nl, float& inv_lam, float& ell, float& Gv)
 {
     // n_g <sigma g>/v (thermal) or n_g sigma(v) (gas at rest)
-    const float Kv = wtab_eval(T, pr, pr.K_off, S.speed);
+    const float Kv = wtab_at(T, pr, kTabK, i, t);
     inv_lam = P.gas_thermal ? S.ng14 * Kv / S.speed : S.ng14 * Kv;
     // diffusion shortcut: exponential steps of mean lambda_D, 1/lambda_D = n sigma_D
     if (kMode == kModeWalk && S.diff) inv_lam = S.ng14 * pr.sigma_D;
     ell = S.ng14 > 0.0f ? __fdividef(nl, inv_lam) : CUDART_INF_F;
-    if (kMode == kModeScoreT) {
-        // (this table stays in global memory: w_tab + G_off, read through L1)
-        Gv = idx_ok(P.status, (long long)pr.G_off + pr.n_w - 1, P.n_w_all)
-                 ? wtab_eval(T, pr, pr.G_off, S.speed)
-                 : 0.0f;
-    }
+    if (kMode == kModeScoreT) Gv = wtab_G(T, pr, i, t);
 }
 
 // Terms of the path scores.  Pressure: a flight of length l that ends in a collision adds
@@ -582,14 +583,23 @@ __device__ __forceinline__ float score_T_partner(const Params& P, float V2, floa
 
 // Free flight k+1 of the atom in S: its Philox block w (word 0 the free path; words 1 and 2,
 // the impact parameter and azimuth, are used by the collision; word 3 is unused), the
-// inverse mean free path and the flight length.
+// inverse mean free path, the flight length and the envelope EA + EB rho of the partner rejection
+// at its end (the speed does not change on the way).
 template <int kMode>
 __device__ void flight_begin(Lane& S, const Params& P, const TableView& T, const DevPair* pairs, StepOut& out,
-                             uint4& w, float& inv_lam, float& ell)
+                             uint4& w, float& inv_lam, float& ell, float& EA, float& EB)
 {
     S.k += 1u;
     w = philox(P, S.pid, S.strm, S.k, 0u);
-    flight_length<kMode>(S, P, T, pairs[S.pair], neg_log_fast(rn(w.x)), inv_lam, ell, out.Gv);
+    const DevPair& pr = pairs[S.pair];
+    int i;
+    float t;
+    wtab_cell(pr, S.speed, i, t);
+    flight_length<kMode>(S, P, T, pr, i, t, neg_log_fast(rn(w.x)), inv_lam, ell, out.Gv);
+    if (P.gas_thermal) {
+        EA = wtab_at(T, pr, kTabA, i, t);
+        EB = wtab_at(T, pr, kTabB, i, t);
+    }
 }
 
 // The emitting target's local index on the first flight (it is skipped then: the atom
@@ -1077,9 +1087,9 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
     out.attempts = 0;
     constexpr bool kScoreT = kMode == kModeScoreT;
     if (kScoreT) out.Gv = 0.0f;
-    float inv_lam = 0.0f, ell = 0.0f, tb = CUDART_INF_F;
+    float inv_lam = 0.0f, ell = 0.0f, EA = 0.0f, EB = 0.0f, tb = CUDART_INF_F;
     int hb = -1;
-    if (active) flight_begin<kMode>(S, P, T, pairs, out, w, inv_lam, ell);
+    if (active) flight_begin<kMode>(S, P, T, pairs, out, w, inv_lam, ell, EA, EB);
     if (kMasks) nearest_hit_masks<kMasks ? kMasks : 1>(active, S, P, T, prims, list, ell, tb, hb);
     else if (active) nearest_hit_loop(S, P, T, prims, ell, tb, hb);
     if (active) res = flight_end<kMode>(S, P, out, inv_lam, ell, tb, hb);
@@ -1090,12 +1100,6 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
     const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
     float Vx = 0.0f, Vy = 0.0f, Vz = 0.0f;
     if (P.gas_thermal) {
-        float EA = 0.0f, EB = 0.0f;
-        if (coll) {
-            const float w = w_of(pr, S.speed);
-            EA = wtab_at(T, pr, pr.A_off, w);
-            EB = wtab_at(T, pr, pr.B_off, w);
-        }
         partner_sample_warp(coll, P, T, pairs, S.pid, S.strm, S.k, S.pair, vx, vy, vz, EA, EB, Vx,
                             Vy, Vz, out.attempts);
         if (kScoreT && coll)
@@ -1704,9 +1708,11 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
             const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
             float EA = 0.0f, EB = 0.0f;
             if (P.gas_thermal) {
-                const float w = w_of(pr, S.speed);
-                EA = wtab_at(T, pr, pr.A_off, w);
-                EB = wtab_at(T, pr, pr.B_off, w);
+                int i;
+                float t;
+                wtab_cell(pr, S.speed, i, t);
+                EA = wtab_at(T, pr, kTabA, i, t);
+                EB = wtab_at(T, pr, kTabB, i, t);
             }
             const Impact h = W.hit[head + f];
             const float4 z = W.z[head + f][my_a], r = W.rho[head + f][my_a];
@@ -1764,7 +1770,12 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
 
         // ---------------------------------------------------- 3. flights
         float inv_lam = 0.0f, ell = 0.0f, Gv = 0.0f;
-        if (have) flight_length<kMode>(F, P, T, pr, nl, inv_lam, ell, Gv);
+        if (have) {
+            int i;
+            float t;
+            wtab_cell(pr, F.speed, i, t);
+            flight_length<kMode>(F, P, T, pr, i, t, nl, inv_lam, ell, Gv);
+        }
         // positions and scores before each flight: running sums over the batch, in order
         const float gain = score_gain(ell, inv_lam);
         const float aT = kScoreT ? score_T_rate(P, Gv) : 0.0f;
@@ -1909,15 +1920,20 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
     } else if (what == SPUT_PROBE_K) {
         const DevPair pr = P.pairs[idx];
         const float v = (float)x[i];
-        float val = wtab_eval(T, pr, pr.K_off, v);
+        int c;
+        float t;
+        wtab_cell(pr, v, c, t);
+        float val = wtab_at(T, pr, kTabK, c, t);
         if (!P.gas_thermal) val *= v;  // the table holds sigma(v) = K/v
         y[i] = val;
     } else if (what == SPUT_PROBE_M) {
         // rejection envelope (A, B) of the pair at speed v
         const DevPair pr = P.pairs[idx];
-        const float w = w_of(pr, (float)x[i]);
-        y[2 * i] = wtab_at(T, pr, pr.A_off, w);
-        y[2 * i + 1] = wtab_at(T, pr, pr.B_off, w);
+        int c;
+        float t;
+        wtab_cell(pr, (float)x[i], c, t);
+        y[2 * i] = wtab_at(T, pr, kTabA, c, t);
+        y[2 * i + 1] = wtab_at(T, pr, kTabB, c, t);
     } else if (what == SPUT_PROBE_LAUNCH) {
         float px, py, pz, dx, dy, dz, E;
         launch_state(P, P.rt_tab, (uint32_t)idx, (uint32_t)x[i], px, py, pz, dx, dy, dz, E);
