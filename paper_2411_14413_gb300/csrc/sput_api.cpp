@@ -296,9 +296,9 @@ static sput_status pack_instances(sput_scene* S)
         if (!C.launch_table && Em > S->pair_E_top[pair] * (1.0 + 1e-12))
             return fail(SPUT_ERR_INVALID_ARG, "E_max beyond the range of the scene's tables; recreate the scene");
         DevInstance& D = S->dinst[i];
-        D.geometry = I.geometry;
+        D.geom_pair = (uint32_t)I.geometry | (uint32_t)pair << 16;
+        D.target = C.target;
         D.cathode = I.cathode;
-        D.pair = pair;
         D.n = (uint32_t)I.n_particles;
         // n_g = p / (k_B T) in m^-3 -> mm^-3 (1e-9); sigma in A^2 -> mm^2 (1e-14)
         D.ng14 = (float)(I.pressure / kT * 1e-9 * 1e-14);
@@ -314,7 +314,7 @@ static sput_status pack_instances(sput_scene* S)
     // mean inverse free path of 1 eV atoms, for the choice of the surface test (cell_masks_pay)
     S->mean_inv_lambda = 0.0;
     for (size_t i = 0; i < S->dinst.size(); ++i) {
-        const DevPair& pr = S->dpairs[S->dinst[i].pair];
+        const DevPair& pr = S->dpairs[S->dinst[i].geom_pair >> 16];
         const double v = 1.0 / std::sqrt((double)S->dcath[S->dinst[i].cathode].E_per_v2);
         const double x = std::min(std::log(1.0 + v * pr.inv_s) * pr.w_inv_h, (double)pr.n_w);
         const int j = std::min((int)x, pr.n_w - 1);
@@ -734,7 +734,7 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     p.cell_mask = S->cell_masks.empty() ? nullptr : reinterpret_cast<const uint32_t*>(S->d_blob + S->off_cell);
     p.cell_words = S->cell_words;
     for (int a = 0; a < 3; ++a) {
-        p.cell_lo[a] = (float)S->cell_lo[a];
+        p.cell_off[a] = S->cell_h > 0.0 ? (float)(-S->cell_lo[a] / S->cell_h) : 0.0f;
         p.cell_n[a] = S->cell_n[a];
     }
     p.cell_inv_h = S->cell_h > 0.0 ? (float)(1.0 / S->cell_h) : 0.0f;

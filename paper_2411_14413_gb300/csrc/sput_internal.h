@@ -121,7 +121,8 @@ struct alignas(16) DevInstance {
     // read together at every flight (load_conditions)
     float ng14;           // n_gas (mm^-3) * 1e-14: inverse mean free path = ng14 * K / v
     uint32_t stream;      // word 1 of every Philox counter of this instance's particles
-    int geometry, pair;
+    uint32_t geom_pair;   // geometry | gas pair << 16 (both are staged in shared memory: fewer than 2^16)
+    int target;           // local index of the emitting target
     int cathode;
     uint32_t n;           // particles
     float thompson_q;     // E_max / (E_max + U_s)
@@ -151,7 +152,7 @@ struct Params {
     // that have a point within r 2^k of a point of the cell
     const uint32_t* cell_mask;
     int cell_words;
-    float cell_lo[3], cell_inv_h, cell_inv_r, cell_inv_seg;
+    float cell_off[3], cell_inv_h, cell_inv_r, cell_inv_seg;  // (cell_off = -lower corner / h)
     int cell_n[3];
     int n_prims, n_geoms, n_pairs, n_inst;
     int n_bm;

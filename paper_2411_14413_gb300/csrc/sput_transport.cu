@@ -325,6 +325,7 @@ struct Lane {
     float ng14;
     uint32_t strm;
     int geom, pair;  // geometry index (its record is read from TableView::geoms), gas pair
+    int target;      // local index of the emitting target
 };
 
 // The instance's conditions that a flight needs, 16 bytes through L1.  The transport reads them
@@ -334,8 +335,10 @@ __device__ __forceinline__ void load_conditions(Lane& S, const Params& P)
     const uint4 c = __ldg(reinterpret_cast<const uint4*>(P.inst + S.inst));
     S.ng14 = __uint_as_float(c.x);
     S.strm = c.y;
-    S.geom = idx_ok(P.status, (int)c.z, P.n_geoms) ? (int)c.z : 0;
-    S.pair = idx_ok(P.status, (int)c.w, P.n_pairs) ? (int)c.w : 0;
+    const int geom = (int)(c.z & 0xffffu), pair = (int)(c.z >> 16);
+    S.geom = idx_ok(P.status, geom, P.n_geoms) ? geom : 0;
+    S.pair = idx_ok(P.status, pair, P.n_pairs) ? pair : 0;
+    S.target = (int)c.w;
 }
 
 __device__ __forceinline__ float racetrack_r(const DevCathode& C, const float4* rt_tab, int rt_n, int n_rt_all,
@@ -441,20 +444,22 @@ __device__ void launch_state(const Params& P, const float4* rt_tab, uint32_t ins
 __device__ __forceinline__ float hit_box(const Params& P, float px, float py, float pz, float dx, float dy, float dz)
 {
     // approximate quotients (2 ulp): a hit distance needs no correctly rounded division
-    const float tx = dx > 0.0f ? __fdividef(P.box_hi[0] - px, dx)
-                               : (dx < 0.0f ? __fdividef(P.box_lo[0] - px, dx) : CUDART_INF_F);
-    const float ty = dy > 0.0f ? __fdividef(P.box_hi[1] - py, dy)
-                               : (dy < 0.0f ? __fdividef(P.box_lo[1] - py, dy) : CUDART_INF_F);
-    const float tz = dz > 0.0f ? __fdividef(P.box_hi[2] - pz, dz)
-                               : (dz < 0.0f ? __fdividef(P.box_lo[2] - pz, dz) : CUDART_INF_F);
+    const float qx = __fdividef((dx > 0.0f ? P.box_hi[0] : P.box_lo[0]) - px, dx);
+    const float qy = __fdividef((dy > 0.0f ? P.box_hi[1] : P.box_lo[1]) - py, dy);
+    const float qz = __fdividef((dz > 0.0f ? P.box_hi[2] : P.box_lo[2]) - pz, dz);
+    const float tx = fabsf(dx) > 0.0f ? qx : CUDART_INF_F;
+    const float ty = fabsf(dy) > 0.0f ? qy : CUDART_INF_F;
+    const float tz = fabsf(dz) > 0.0f ? qz : CUDART_INF_F;
     return fmaxf(fminf(tx, fminf(ty, tz)), 0.0f);
 }
 
+// kBox: the primitive may be a chamber box
+template <bool kBox>
 __device__ __forceinline__ float hit_prim(const DevPrim& Q, const Params& P, float px, float py, float pz, float dx,
                                           float dy, float dz)
 {
     float t = CUDART_INF_F;
-    if (Q.kind == SPUT_PRIM_BOX) {
+    if (kBox && Q.kind == SPUT_PRIM_BOX) {
         t = hit_box(P, px, py, pz, dx, dy, dz);
     } else if (Q.kind == SPUT_PRIM_CYLINDER) {
         const float wx = px - Q.cx, wy = py - Q.cy, wz = pz - Q.cz;
@@ -603,11 +608,8 @@ __device__ void flight_begin(Lane& S, const Params& P, const TableView& T, const
 }
 
 // The emitting target's local index on the first flight (it is skipped then: the atom
-// leaves its plane; read only then), else -1.
-__device__ __forceinline__ int excluded_prim(const Lane& S, const Params& P)
-{
-    return S.k == 1u ? P.cath[P.inst[S.inst].cathode].target : -1;
-}
+// leaves its plane), else -1.
+__device__ __forceinline__ int excluded_prim(const Lane& S) { return S.k == 1u ? S.target : -1; }
 
 // Nearest hit by a loop over the geometry's primitives, ties to the lowest index.  Every
 // primitive whose bounding sphere lies within min(ell, best t) is tested (margin covers
@@ -616,7 +618,7 @@ __device__ __forceinline__ void nearest_hit_loop(const Lane& S, const Params& P,
                                                  const DevPrim* prims, float ell, float& tb, int& hb)
 {
     const DevGeom G = T.geoms[S.geom];
-    const int excl = excluded_prim(S, P);
+    const int excl = excluded_prim(S);
     for (int li = 0; li < G.count; ++li) {
         if (li == excl) continue;
         if (!idx_ok(P.status, G.begin + li, P.n_prims)) break;
@@ -626,7 +628,7 @@ __device__ __forceinline__ void nearest_hit_loop(const Lane& S, const Params& P,
             const float reach = fminf(ell, tb) * 1.0001f + Q.br + 1e-3f;
             if (ex * ex + ey * ey + ez * ez > reach * reach) continue;
         }
-        const float t = hit_prim(Q, P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
+        const float t = hit_prim<true>(Q, P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
         if (t < tb) {
             tb = t;
             hb = li;
@@ -666,17 +668,23 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
         tb = hit_box(P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
         hb = tb < CUDART_INF_F ? box : -1;
         const float L = fminf(ell, tb);
-        int pieces = min((int)(L * P.cell_inv_seg), kCellMaxPieces - 1) + 1;
-        const float R = 0.5f * __fdividef(L, (float)pieces);
+        // 1 + floor(L / (4 h)) pieces (floor as in table_cell; at most kCellMaxPieces, also for NaN)
+        float pieces = fminf(__fadd_rd(L * P.cell_inv_seg, 8388608.0f) - 8388607.0f, (float)kCellMaxPieces);
+        const float R = 0.5f * __fdividef(L, pieces);
         // the smallest level: max(0, ceil(log2(R / r))) from the exponent bits
         const int k = max(0, (int)((__float_as_uint(R * P.cell_inv_r) + 0x7fffffu) >> 23) - 127);
-        for (float c = R; pieces > 0; --pieces, c += 2.0f * R) {
-            const float mx = (fmaf(c, S.dx, S.px) - P.cell_lo[0]) * P.cell_inv_h;
-            const float my = (fmaf(c, S.dy, S.py) - P.cell_lo[1]) * P.cell_inv_h;
-            const float mz = (fmaf(c, S.dz, S.pz) - P.cell_lo[2]) * P.cell_inv_h;
-            if (k < kCellLevels && fminf(fminf(mx, my), mz) >= 0.0f && mx < (float)P.cell_n[0] &&
-                my < (float)P.cell_n[1] && mz < (float)P.cell_n[2]) {
-                const int cell = ((int)mz * P.cell_n[1] + (int)my) * P.cell_n[0] + (int)mx;
+        // grid coordinates of the start; step of the centres
+        const float sx = fmaf(S.px, P.cell_inv_h, P.cell_off[0]), sy = fmaf(S.py, P.cell_inv_h, P.cell_off[1]),
+                    sz = fmaf(S.pz, P.cell_inv_h, P.cell_off[2]);
+        const float Rh = R * P.cell_inv_h;
+        for (float c = Rh; pieces > 0.0f; pieces -= 1.0f, c += 2.0f * Rh) {
+            // floors of the coordinates; a negative one wraps to a large unsigned number
+            const unsigned ix = __float_as_uint(__fadd_rd(fmaf(c, S.dx, sx), 8388608.0f)) - 0x4b000000u;
+            const unsigned iy = __float_as_uint(__fadd_rd(fmaf(c, S.dy, sy), 8388608.0f)) - 0x4b000000u;
+            const unsigned iz = __float_as_uint(__fadd_rd(fmaf(c, S.dz, sz), 8388608.0f)) - 0x4b000000u;
+            if (k < kCellLevels && ix < (unsigned)P.cell_n[0] && iy < (unsigned)P.cell_n[1] &&
+                iz < (unsigned)P.cell_n[2]) {
+                const int cell = (int)((iz * P.cell_n[1] + iy) * P.cell_n[0] + ix);
                 const uint32_t* m = P.cell_mask + G.cell_base + (cell * kCellLevels + k) * kWords;
                 if (kWords == 1) {
                     lo |= __ldg(m);
@@ -693,35 +701,35 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
                 if (kWords == 2 && box >= 32) hi &= ~(1u << (box - 32));
             }
         }
-        const int excl = excluded_prim(S, P);
+        const int excl = excluded_prim(S);
         if (excl >= 0 && excl < 32) lo &= ~(1u << excl);
         if (kWords == 2 && excl >= 32) hi &= ~(1u << (excl - 32));
     }
-    const int n = __popc(lo) + (kWords == 2 ? __popc(hi) : 0);
-    if (!__any_sync(kFull, n != 0)) return;
-    // pos: exclusive prefix of n over the lanes, from the ballots of its bits
     const unsigned lt = (1u << lane) - 1u;
-    int pos = 0, total = 0, bit = 0;
-    do {
-        const unsigned m = __ballot_sync(kFull, (n >> bit) & 1);
-        pos += __popc(m & lt) << bit;
-        total += __popc(m) << bit;
-        ++bit;
-    } while (__any_sync(kFull, n >> bit));
-    for (; total > 0; total -= 32, pos -= 32) {
-        // the lanes list their pairs of this round (positions 0..31)
-        const int first = pos;
-        while (pos < 32 && (kWords == 2 ? (lo | hi) : lo)) {
-            int li;
-            if (kWords == 1 || lo) {
-                li = __ffs(lo) - 1;
-                lo &= lo - 1u;
-            } else {
-                li = 31 + __ffs(hi);
-                hi &= hi - 1u;
+    for (;;) {
+        // The lanes list their candidates, one each per turn, up to 32 pairs a round.  `turn` finds the
+        // lane's place of a turn; the turns are gone through again to take the hits.
+        const unsigned lo0 = lo, hi0 = hi;
+        int total = 0;
+        for (;;) {
+            const bool any = (kWords == 2 ? lo | hi : lo) != 0u;
+            const unsigned m = __ballot_sync(kFull, any);
+            if (m == 0u || total == 32) break;
+            const int at = total + __popc(m & lt);
+            if (any && at < 32) {
+                int li;
+                if (kWords == 1 || lo) {
+                    li = __ffs(lo) - 1;
+                    lo &= lo - 1u;
+                } else {
+                    li = 31 + __ffs(hi);
+                    hi &= hi - 1u;
+                }
+                list[at].x = (uint32_t)(begin + li) << 5 | (uint32_t)lane;
             }
-            list[pos++].x = (uint32_t)(begin + li) << 5 | (uint32_t)lane;
+            total = min(32, total + __popc(m));
         }
+        if (total == 0) return;
         __syncwarp();
         const bool mine = lane < total;
         const uint32_t pr = mine ? list[lane].x : (uint32_t)lane;
@@ -732,19 +740,28 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
                     dz = __shfl_sync(kFull, S.dz, src);
         if (mine)
             list[lane].y = __float_as_uint(idx_ok(P.status, pr >> 5, P.n_prims)
-                                               ? hit_prim(prims[pr >> 5], P, px, py, pz, dx, dy, dz)
+                                               ? hit_prim<false>(prims[pr >> 5], P, px, py, pz, dx, dy, dz)
                                                : CUDART_INF_F);
         __syncwarp();
-        // and take their hits
-        for (int i = first; i < pos; ++i) {
-            const uint2 e = list[i];
-            const float t = __uint_as_float(e.y);
-            const int li = (int)(e.x >> 5) - begin;
-            if (t < tb || (t == tb && li < hb)) {
-                tb = t;
-                hb = li;
+        unsigned l0 = lo0, h0 = hi0;
+        for (int t0 = 0; t0 < total;) {
+            const bool any = (kWords == 2 ? l0 | h0 : l0) != 0u;
+            const unsigned m = __ballot_sync(kFull, any);
+            const int at = t0 + __popc(m & lt);
+            if (any && at < 32) {
+                const uint2 e = list[at];
+                const float t = __uint_as_float(e.y);
+                const int li = (int)(e.x >> 5) - begin;
+                if (t < tb || (t == tb && li < hb)) {
+                    tb = t;
+                    hb = li;
+                }
+                if (kWords == 1 || l0) l0 &= l0 - 1u;
+                else h0 &= h0 - 1u;
             }
+            t0 += __popc(m);
         }
+        if (total < 32) return;
         __syncwarp();
     }
 }
@@ -1329,6 +1346,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     S.pid = S.inst = S.k = 0u;
     S.geom = S.pair = 0;
     S.strm = 0u;
+    S.target = -1;
     S.ng14 = 0.0f;
     bool alive = false;
 
@@ -1582,6 +1600,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     S.pid = S.inst = S.k = 0u;
     S.geom = S.pair = 0;
     S.strm = 0u;
+    S.target = -1;
     S.ng14 = 0.0f;
     S.diff = false;
     bool have = false, more = true;  // more: the pool may hold further atoms (warp-uniform)
@@ -1640,6 +1659,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
                 S.inst = __shfl_sync(kFull, S.inst, src);
                 S.k = __shfl_sync(kFull, S.k, src);
                 S.geom = __shfl_sync(kFull, S.geom, src);
+                S.target = __shfl_sync(kFull, S.target, src);
                 S.pair = __shfl_sync(kFull, S.pair, src);
                 S.ng14 = __shfl_sync(kFull, S.ng14, src);
                 S.strm = __shfl_sync(kFull, S.strm, src);
@@ -1677,6 +1697,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
         F.pid = S.pid;
         F.inst = S.inst;
         F.geom = S.geom;
+        F.target = S.target;
         F.pair = S.pair;
         F.ng14 = S.ng14;
         F.k = S.k + 1u + l;
@@ -1865,6 +1886,7 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
         S.pid = S.inst = S.k = 0u;
         S.geom = S.pair = 0;
         S.strm = 0u;
+        S.target = -1;
         S.ng14 = 0.0f;
         double* o = valid ? y + (size_t)i * kTraceRows * 10 : nullptr;
         if (valid) {
