@@ -611,6 +611,18 @@ __device__ void flight_begin(Lane& S, const Params& P, const TableView& T, const
 // leaves its plane), else -1.
 __device__ __forceinline__ int excluded_prim(const Lane& S) { return S.k == 1u ? S.target : -1; }
 
+// A warp's scratch in shared memory: the pairs of the surface test, and what the partner
+// sampling hands to the lanes that try an atom's attempts.
+constexpr int kAskers = 8;
+union WarpScratch {
+    uint2 list[32];
+    struct {
+        float4 v[kAskers];   // v, EA
+        uint4 ids[kAskers];  // particle id, stream, flight, next attempt
+        uint2 p[kAskers];    // EB, pair
+    } ask;
+};
+
 // Nearest hit by a loop over the geometry's primitives, ties to the lowest index.  Every
 // primitive whose bounding sphere lies within min(ell, best t) is tested (margin covers
 // FP32 rounding): no hit beyond that can be the landing.
@@ -797,11 +809,6 @@ __device__ int flight_end(Lane& S, const Params& P, StepOut& out, float inv_lam,
     return kStepCollided;
 }
 
-// ceil(2^11 / d) for d = 1..33: floor(l / d) = (l kInv11[d]) >> 11 for l <= 32 (the excess, below
-// l / 2^11 <= 1/64, stays under the 1/33 that separates a quotient from the next integer)
-__constant__ int kInv11[34] = {0,   2048, 1024, 683, 512, 410, 342, 293, 256, 228, 205, 187, 171, 158, 147, 137, 128,
-                               121, 114,  108,  103, 98,  94,  90,  86,  82,  79,  76,  74,  71,  69,  67,  64,  63};
-
 // position of the n-th (0-based) set bit of mask; mask has more than n set bits
 __device__ __forceinline__ int nth_set_bit(unsigned mask, int n)
 {
@@ -892,14 +899,13 @@ __device__ __forceinline__ bool attempt_accept(const Attempt& d, bool weighted, 
 // (u (EA + EB E[rho]) <= EB E[rho]: rho-weighted) and, rescaled within the
 // branch, is the acceptance uniform.  Maxwellian branch: V = s (z1, z2, z3);
 // rho-weighted branch: V = s |z| (z1, z2, z3)/|(z1, z2, z3)|.  The first
-// accepted attempt is kept (attempt A-1 if none is).  Each round spreads the
-// pending particles' next attempts over all 32 lanes (consecutive attempts per
-// particle, the first 32 mod np particles one more), so the result is the
-// sequential rejection loop's result while every lane stays busy.  Must be
-// called by all 32 lanes together.
+// accepted attempt is kept (attempt A-1 if none is).  While most lanes wait for a partner, each
+// tries its own next attempt; then the pending particles' next attempts are spread over the
+// warp (2^k consecutive attempts per particle), so the result is the sequential
+// rejection loop's result while the lanes stay busy.  Must be called by all 32 lanes together.
 __device__ void partner_sample_warp(bool need, const Params& P, const TableView& T, const DevPair* pairs,
                                     uint32_t pid, uint32_t strm, uint32_t k, int pair, float vx, float vy, float vz,
-                                    float EA, float EB, float& Vx, float& Vy, float& Vz, int& attempts)
+                                    float EA, float EB, WarpScratch* ws, float& Vx, float& Vy, float& Vz, int& attempts)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -908,41 +914,46 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
     int next_a = 0;
     Vx = Vy = Vz = 0.0f;
     attempts = 0;
-    // Most lanes pending: each tries its first attempt itself, without the hand-out below.
-    bool own = __popc(pending) > 16;
     while (pending) {
+        // many lanes pending: each tries its next attempt itself; few: the whole warp tries theirs,
+        // 2^shift consecutive attempts each
+        const bool own = __popc(pending) > kAskers;
+        const bool asks = (pending >> lane) & 1u;
         uint32_t o_pid = pid, o_strm = strm, o_k = k;
-        int o_pair = pair, o_next = next_a, j = need ? 0 : A, m = 1, extra = 32, cut = 64;
-        float o_vx = vx, o_vy = vy, o_vz = vz, o_A = EA, o_B = EB;
+        int a = asks ? next_a : A, shift = 0, rank = 0;
         if (!own) {
-            // np pending particles share 32 lanes: the first `extra` get m + 1 lanes, the rest m
             const int np = __popc(pending);
-            m = (32 * kInv11[np]) >> 11;
-            extra = 32 - m * np;
-            cut = extra * (m + 1);
-            const bool more = lane < cut;
-            const int d = more ? m + 1 : m, at = more ? lane : lane - cut;
-            const int q = (at * kInv11[d]) >> 11;
-            j = at - q * d;
-            const int slot = more ? q : extra + q;
-            const int owner = nth_set_bit(pending, slot);
-            o_pid = __shfl_sync(kFull, pid, owner);
-            o_strm = __shfl_sync(kFull, strm, owner);
-            o_k = __shfl_sync(kFull, k, owner);
-            o_pair = __shfl_sync(kFull, pair, owner);
-            o_vx = __shfl_sync(kFull, vx, owner);
-            o_vy = __shfl_sync(kFull, vy, owner);
-            o_vz = __shfl_sync(kFull, vz, owner);
-            o_A = __shfl_sync(kFull, EA, owner);
-            o_B = __shfl_sync(kFull, EB, owner);
-            o_next = __shfl_sync(kFull, next_a, owner);
+            shift = __clz(np - 1) - 27;  // 5 - ceil(log2 np)
+            rank = __popc(pending & lt);
+            if (asks) {
+                ws->ask.v[rank] = make_float4(vx, vy, vz, EA);
+                ws->ask.ids[rank] = make_uint4(pid, strm, k, (uint32_t)next_a);
+                ws->ask.p[rank] = make_uint2(__float_as_uint(EB), (uint32_t)pair);
+            }
+            __syncwarp();
+            const uint4 q = ws->ask.ids[lane >> shift];
+            o_pid = q.x;
+            o_strm = q.y;
+            o_k = q.z;
+            a = lane >> shift < np ? (int)q.w + (lane & ((1 << shift) - 1)) : A;
         }
-        const int a = o_next + j;
         bool acc = false;
         float cx = 0.0f, cy = 0.0f, cz = 0.0f;
         if (a < A) {
-            const int op = idx_ok(T.status, o_pair, P.n_pairs) ? o_pair : 0;
             const Attempt d = attempt_draw(P, o_pid, o_strm, o_k, (uint32_t)a);
+            float o_vx = vx, o_vy = vy, o_vz = vz, o_A = EA, o_B = EB;
+            int op = pair;
+            if (!own) {
+                const float4 q = ws->ask.v[lane >> shift];
+                const uint2 r = ws->ask.p[lane >> shift];
+                o_vx = q.x;
+                o_vy = q.y;
+                o_vz = q.z;
+                o_A = q.w;
+                o_B = __uint_as_float(r.x);
+                op = (int)r.y;
+            }
+            if (!idx_ok(T.status, op, P.n_pairs)) op = 0;
             float ut, Bm;
             const bool weighted = attempt_weighted(d, o_A, o_B, ut, Bm);
             attempt_velocity(P, d, weighted, cx, cy, cz);
@@ -955,28 +966,23 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
                 Vx = cx;
                 Vy = cy;
                 Vz = cz;
-                attempts = 1;
+                attempts = a + 1;
             }
-            next_a = 1;
+            ++next_a;
             pending &= ~accm;
-            own = false;
             continue;
         }
-        const bool is_owner = (pending >> lane) & 1u;
         int src = lane, first = 0;
         bool done = false;
-        if (is_owner) {
-            const int my_slot = __popc(pending & lt);
-            const int my_m = my_slot < extra ? m + 1 : m;
-            const int my_lo = my_slot < extra ? my_slot * (m + 1) : cut + (my_slot - extra) * m;
-            const unsigned range = (my_m >= 32 ? kFull : ((1u << my_m) - 1u)) << my_lo;
-            const unsigned hit = accm & range;
+        if (asks) {
+            const int lanes = 1 << shift, at = rank << shift;
+            const unsigned hit = accm & ((kFull >> (32 - lanes)) << at);
             if (hit) {
                 src = __ffs(hit) - 1;
-                first = src - my_lo;
+                first = src - at;
                 done = true;
             } else {
-                next_a += my_m;
+                next_a += lanes;
             }
         }
         const float sx = __shfl_sync(kFull, cx, src);
@@ -1092,11 +1098,10 @@ __device__ __forceinline__ float energy_of(const Params& P, uint32_t inst, float
 // One flight of every active lane of the warp (flight, surface test, then for
 // the lanes that collide: warp-wide partner sampling and the scattering).
 // Must be called by all 32 lanes together; inactive lanes return kStepNone.
-// kMasks: words of the surface test's cell masks (0: the counted loop); list: the warp's
-// 32 entries of shared memory for them.
+// kMasks: words of the surface test's cell masks (0: the counted loop); ws: the warp's scratch.
 template <int kMode, int kMasks>
 __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const TableView& T, const DevPrim* prims,
-                                const DevPair* pairs, uint2* list, StepOut& out)
+                                const DevPair* pairs, WarpScratch* ws, StepOut& out)
 {
     load_conditions(S, P);
     uint4 w = make_uint4(0u, 0u, 0u, 0u);
@@ -1107,7 +1112,7 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
     float inv_lam = 0.0f, ell = 0.0f, EA = 0.0f, EB = 0.0f, tb = CUDART_INF_F;
     int hb = -1;
     if (active) flight_begin<kMode>(S, P, T, pairs, out, w, inv_lam, ell, EA, EB);
-    if (kMasks) nearest_hit_masks<kMasks ? kMasks : 1>(active, S, P, T, prims, list, ell, tb, hb);
+    if (kMasks) nearest_hit_masks<kMasks ? kMasks : 1>(active, S, P, T, prims, ws->list, ell, tb, hb);
     else if (active) nearest_hit_loop(S, P, T, prims, ell, tb, hb);
     if (active) res = flight_end<kMode>(S, P, out, inv_lam, ell, tb, hb);
     // a thermalised atom (diffusion shortcut) turns isotropically at the end of its step
@@ -1117,7 +1122,7 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
     const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
     float Vx = 0.0f, Vy = 0.0f, Vz = 0.0f;
     if (P.gas_thermal) {
-        partner_sample_warp(coll, P, T, pairs, S.pid, S.strm, S.k, S.pair, vx, vy, vz, EA, EB, Vx,
+        partner_sample_warp(coll, P, T, pairs, S.pid, S.strm, S.k, S.pair, vx, vy, vz, EA, EB, ws, Vx,
                             Vy, Vz, out.attempts);
         if (kScoreT && coll)
             S.scoreT = fmaf(score_T_partner(P, sumsq_xyz(Vx, Vy, Vz), out.Gv), P.inv_T, S.scoreT);
@@ -1247,7 +1252,7 @@ __device__ __forceinline__ void tally_timed_out(const Params& P, const Lane& S, 
 
 // ------------------------------------------------------------- kernel
 struct SmemLayout {
-    size_t prims, geoms, pairs, bm, prefix, xh, gm, pool, queue, list, counters, total;
+    size_t prims, geoms, pairs, bm, prefix, gm, pool, queue, scratch, counters, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -1266,16 +1271,14 @@ __host__ __device__ inline SmemLayout smem_layout(const Params& p)
     o = align16(o + sizeof(float4) * p.n_bm);
     L.prefix = o;
     o = align16(o + sizeof(unsigned long long) * (p.n_inst + 1));
-    L.xh = o;
-    o = align16(o + sizeof(float) * (p.n_bm + 1));
     L.gm = o;
     o = align16(o + sizeof(float4) * (kGMHalf + kGMHalfLo));
     L.pool = o;
     o = align16(o + sizeof(unsigned long long) * 4 * 8);
     L.queue = o;
     o = align16(o + sizeof(uint32_t) * kLaunchWords * 32 * 8);
-    L.list = o;
-    o = align16(o + (p.cell_mask ? sizeof(uint2) * 32 * 8 : 0));
+    L.scratch = o;
+    o = align16(o + sizeof(WarpScratch) * 8);
     L.counters = o;
     o = align16(o + (p.smem_counters ? sizeof(unsigned int) * (size_t)p.n_inst * (p.max_prims + 1) : 0));
     L.total = o;
@@ -1307,7 +1310,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     DevPair* s_pairs = reinterpret_cast<DevPair*>(smem + L.pairs);
     float4* s_bm = reinterpret_cast<float4*>(smem + L.bm);
     unsigned long long* s_prefix = reinterpret_cast<unsigned long long*>(smem + L.prefix);
-    float* s_xh = reinterpret_cast<float*>(smem + L.xh);
     float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
     unsigned long long* s_pool = reinterpret_cast<unsigned long long*>(smem + L.pool);
     uint32_t* s_queue = reinterpret_cast<uint32_t*>(smem + L.queue);
@@ -1318,7 +1320,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     copy16(s_pairs, P.pairs, sizeof(DevPair) * P.n_pairs);
     copy16(s_bm, P.bm_tab, sizeof(float4) * P.n_bm);
     copy16(s_prefix, P.prefix, sizeof(unsigned long long) * (P.n_inst + 1));
-    copy16(s_xh, P.xh_tab, sizeof(float) * (P.n_bm + 1));
     if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
     else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
     const int n_cnt = P.smem_counters ? P.n_inst * (P.max_prims + 1) : 0;
@@ -1327,7 +1328,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 
     TableView T;
     T.bm = s_bm;
-    T.xh = s_xh;
+    T.xh = P.xh_tab;  // (off the deflection table only: stays in global memory)
     T.w = P.w_tab;
     T.gm = s_gm;
     T.pairs = s_pairs;
@@ -1357,7 +1358,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     // and its queue of prepared launches: s_wpool[2] entries of kLaunchWords words
     unsigned long long* s_wpool = s_pool + 4 * (threadIdx.x >> 5);
     uint32_t* s_wqueue = s_queue + kLaunchWords * 32 * (threadIdx.x >> 5);
-    uint2* s_wlist = reinterpret_cast<uint2*>(smem + L.list) + 32 * (threadIdx.x >> 5);
+    WarpScratch* s_wscratch = reinterpret_cast<WarpScratch*>(smem + L.scratch) + (threadIdx.x >> 5);
     if (lane == 0) s_wpool[0] = s_wpool[1] = s_wpool[2] = 0ull;
     __syncwarp();
 
@@ -1454,7 +1455,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 
         // ---------------------------------------------------- one flight (all lanes together)
         StepOut so;
-        const int res = flight_step_warp<kMode, kMasks>(alive, S, P, T, s_prims, s_pairs, s_wlist, so);
+        const int res = flight_step_warp<kMode, kMasks>(alive, S, P, T, s_prims, s_pairs, s_wscratch, so);
         c_att += so.attempts;
         if (res == kStepLanded) {
             tally_landed<kMode>(P, S, s_geoms, s_prims, s_cnt, so.t, so.prim);
@@ -1526,7 +1527,7 @@ struct DrainWarp {                // by the flight's lane
 };
 
 struct DrainLayout {
-    size_t prims, geoms, pairs, bm, xh, gm, warps, total;
+    size_t prims, geoms, pairs, bm, gm, warps, total;
 };
 
 __host__ __device__ inline DrainLayout drain_layout(const Params& p)
@@ -1543,8 +1544,6 @@ __host__ __device__ inline DrainLayout drain_layout(const Params& p)
     o = align16(o + sizeof(DevPair) * p.n_pairs);
     L.bm = o;
     o = align16(o + sizeof(float4) * p.n_bm);
-    L.xh = o;
-    o = align16(o + sizeof(float) * (p.n_bm + 1));
     L.gm = o;
     o = align16(o + sizeof(float4) * (kGMHalf + kGMHalfLo));
     L.total = o;
@@ -1567,21 +1566,19 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     DevGeom* s_geoms = reinterpret_cast<DevGeom*>(smem + L.geoms);
     DevPair* s_pairs = reinterpret_cast<DevPair*>(smem + L.pairs);
     float4* s_bm = reinterpret_cast<float4*>(smem + L.bm);
-    float* s_xh = reinterpret_cast<float*>(smem + L.xh);
     float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
     DrainWarp& W = reinterpret_cast<DrainWarp*>(smem + L.warps)[threadIdx.x >> 5];
     copy16(s_prims, P.prims, sizeof(DevPrim) * P.n_prims);
     copy16(s_geoms, P.geoms, sizeof(DevGeom) * P.n_geoms);
     copy16(s_pairs, P.pairs, sizeof(DevPair) * P.n_pairs);
     copy16(s_bm, P.bm_tab, sizeof(float4) * P.n_bm);
-    copy16(s_xh, P.xh_tab, sizeof(float) * (P.n_bm + 1));
     if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
     else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
     __syncthreads();
 
     TableView T;
     T.bm = s_bm;
-    T.xh = s_xh;
+    T.xh = P.xh_tab;  // (off the deflection table only: stays in global memory)
     T.w = P.w_tab;
     T.gm = s_gm;
     T.pairs = s_pairs;
@@ -1860,6 +1857,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
 __global__ void probe_kernel(const Params P, int what, int idx, int n, const double* x, double* y)
 {
     __shared__ float4 s_gm[kGMHalf + kGMHalfLo];
+    __shared__ WarpScratch s_ws[4];  // (launched with 128 threads)
     if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
     else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
     __syncthreads();
@@ -1902,8 +1900,8 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
             StepOut so;
             // (the oracle's trace tests the counted loop; both surface tests give the same flights)
             const int status = P.E_switch > 0.0f
-                                   ? flight_step_warp<kModeWalk, 0>(running, S, P, T, P.prims, P.pairs, nullptr, so)
-                                   : flight_step_warp<kModePlain, 0>(running, S, P, T, P.prims, P.pairs, nullptr, so);
+                                   ? flight_step_warp<kModeWalk, 0>(running, S, P, T, P.prims, P.pairs, &s_ws[threadIdx.x >> 5], so)
+                                   : flight_step_warp<kModePlain, 0>(running, S, P, T, P.prims, P.pairs, &s_ws[threadIdx.x >> 5], so);
             if (running) {
                 double* q = o + (size_t)r * 10;
                 float px = S.px, py = S.py, pz = S.pz;
