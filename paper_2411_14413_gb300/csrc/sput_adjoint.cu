@@ -14,6 +14,7 @@
 //   a_j(m) = R_j(P_j) * N_j(m) / N_j(ref) * rho_j / M_j,   c_j(m) = 100 a_j(m) / sum_k a_k(m),
 // N_j(m) the arrivals of cathode j summed over measurement patch m, ref the
 // central patch, R_j linear in power through two calibration points.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -24,9 +25,18 @@
 #include "sput.h"
 #include "sput_internal.h"
 
+namespace cg = cooperative_groups;
+
 namespace {
 
 constexpr int kMaxCath = 16;
+
+// Blocks of the cluster that reduces one instance (or the composition backward): one block per
+// instance left 148 of 152 SMs idle on a four-cathode map and waited on its own loads.  The
+// partial sums meet in the first block's shared memory and are added in block order, so the
+// result does not depend on timing.
+constexpr int kCluster = 8;
+constexpr int kReduceThreads = 512;
 
 struct CompParams {
     int n_cath, n_cells, n_points, ref;
@@ -41,21 +51,41 @@ __device__ double warp_sum(double x)
     return x;
 }
 
-// grad[i] = sum_c g[i][c] * score[i][c], one block per instance
-__global__ void lr_backward_kernel(const double* g, const double* score, double* grad, long long n_cells)
+// Sum of x over the threads of the cluster, in thread 0 of its first block; part: shared memory of
+// kCluster + 32 doubles.  The last step is a cluster barrier.
+__device__ double cluster_sum(double x, double* part)
 {
-    __shared__ double part[32];
-    const long long base = (long long)blockIdx.x * n_cells;
-    double s = 0.0;
-    for (long long c = threadIdx.x; c < n_cells; c += blockDim.x) s += g[base + c] * score[base + c];
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    cg::cluster_group cl = cg::this_cluster();
+    x = warp_sum(x);
+    if ((threadIdx.x & 31) == 0) part[kCluster + (threadIdx.x >> 5)] = x;
     __syncthreads();
     if (threadIdx.x < 32) {
-        double t = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
+        double t = threadIdx.x < (blockDim.x >> 5) ? part[kCluster + threadIdx.x] : 0.0;
         t = warp_sum(t);
-        if (threadIdx.x == 0) grad[blockIdx.x] = t;
+        if (threadIdx.x == 0) cl.map_shared_rank(part, 0)[cl.block_rank()] = t;
     }
+    cl.sync();
+    double s = 0.0;
+    if (threadIdx.x == 0 && cl.block_rank() == 0)
+        for (int b = 0; b < kCluster; ++b) s += part[b];
+    return s;
+}
+
+// grad[i] = sum_c g[i][c] * score[i][c], one cluster per instance.  16 bytes per cell; at 4 x 40000
+// cells bound by latency: 31 us with one block of 256 threads per instance, 5 us so.
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kReduceThreads)
+    lr_backward_kernel(const double* g, const double* score, double* grad, long long n_cells)
+{
+    __shared__ double part[kCluster + 32];
+    const int inst = blockIdx.x / kCluster;
+    const long long base = (long long)inst * n_cells;
+    double s = 0.0;
+#pragma unroll 4
+    for (long long c = (long long)(blockIdx.x % kCluster) * blockDim.x + threadIdx.x; c < n_cells;
+         c += (long long)kCluster * blockDim.x)
+        s += g[base + c] * score[base + c];
+    s = cluster_sum(s, part);
+    if (threadIdx.x == 0 && blockIdx.x % kCluster == 0) grad[inst] = s;
 }
 
 // Derivative with respect to the Thompson cut-off.  The launch energy has the
@@ -64,7 +94,7 @@ __global__ void lr_backward_kernel(const double* g, const double* score, double*
 // end of the support adds p(E_max) E[f | E = E_max]:
 //   d E[f]/dE_max = p(E_max) (E[f | E = E_max] - E[f]),  p(E_max) = 2U / (E_max (E_max + U)).
 // With a boundary run of the same particles launched at E_max (counts_cut) and
-// dE_max/dE_i = k Lambda, one block per instance forms
+// dE_max/dE_i = k Lambda, one cluster per instance forms
 //   grad[i] = k Lambda p(E_max) sum_c g[i][c] (counts_cut[i][c] - counts[i][c]).
 // Voltage lines V_i(P) = V_a + (V_b - V_a)(P - P_a)/(P_b - P_a) (Table S1), with
 // E_i = e V for singly charged ions: dE_i/dP_i in eV/W per instance.
@@ -75,108 +105,143 @@ struct VoltParams {
 // grad_power (optional) gets grad[i] * dE_i/dP_i added: the path from the cathode
 // power through the discharge voltage to the cut-off.
 template <typename CountT>
-__global__ void emax_backward_kernel(const double* g, const CountT* counts, const CountT* counts_cut,
-                                     const sput::DevInstance* inst, double* grad, long long n_cells,
-                                     double* grad_power, VoltParams vp)
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kReduceThreads)
+    emax_backward_kernel(const double* g, const CountT* counts, const CountT* counts_cut, const sput::DevInstance* inst,
+                         double* grad, long long n_cells, double* grad_power, VoltParams vp)
 {
-    __shared__ double part[32];
-    const long long base = (long long)blockIdx.x * n_cells;
+    __shared__ double part[kCluster + 32];
+    const int i = blockIdx.x / kCluster;
+    const long long base = (long long)i * n_cells;
     double s = 0.0;
-    for (long long c = threadIdx.x; c < n_cells; c += blockDim.x)
+#pragma unroll 4
+    for (long long c = (long long)(blockIdx.x % kCluster) * blockDim.x + threadIdx.x; c < n_cells;
+         c += (long long)kCluster * blockDim.x)
         s += g[base + c] * ((double)counts_cut[base + c] - (double)counts[base + c]);
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double t = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
-        t = warp_sum(t);
-        if (threadIdx.x == 0) {
-            const sput::DevInstance I = inst[blockIdx.x];
-            const double q = I.thompson_q, U = I.U_s;
-            const double Em = U * q / (1.0 - q);
-            const double gE = (double)I.kLambda * 2.0 * U / (Em * (Em + U)) * t;
-            grad[blockIdx.x] = gE;
-            if (grad_power) grad_power[blockIdx.x] += gE * vp.dEdP[blockIdx.x];
-        }
+    const double t = cluster_sum(s, part);
+    if (threadIdx.x == 0 && blockIdx.x % kCluster == 0) {
+        const sput::DevInstance I = inst[i];
+        const double q = I.thompson_q, U = I.U_s;
+        const double Em = U * q / (1.0 - q);
+        const double gE = (double)I.kLambda * 2.0 * U / (Em * (Em + U)) * t;
+        grad[i] = gE;
+        if (grad_power) grad_power[i] += gE * vp.dEdP[i];
     }
 }
 
-// N[j][m] = sum of counts of cathode j over the cells of patch m
-__global__ void patch_sum_kernel(const long long* counts, const int32_t* patch, double* N, int n_cath, int n_cells,
-                                 int n_points)
+// N[j][m] = sum of counts of cathode j over the cells of patch m; blockIdx.y = j
+__global__ void patch_sum_kernel(const long long* counts, const int32_t* patch, double* N, int n_cells, int n_points)
 {
-    const long long total = (long long)n_cath * n_cells;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(i / n_cells), c = (int)(i % n_cells);
+    const int j = blockIdx.y;
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)n_cells; c += gridDim.x * blockDim.x) {
         const int m = patch[c];
-        if (m >= 0 && m < n_points && counts[i]) atomicAdd(N + (size_t)j * n_points + m, (double)counts[i]);
+        const long long n = counts[(size_t)j * n_cells + c];
+        if (m >= 0 && m < n_points && n) atomicAdd(N + (size_t)j * n_points + m, (double)n);
     }
 }
 
+// a_j(m) = W_j N_j(m) with W_j = R_j w_j / N_j(ref), 0 where the reference point is empty
+__device__ double arrival_weight(const double* N, const CompParams& cp, int j)
+{
+    const double nref = N[(size_t)j * cp.n_points + cp.ref];
+    return nref > 0.0 ? cp.R[j] * cp.w[j] / nref : 0.0;
+}
+
+// One thread per point, 32 to a block: FP64 runs at two FMAs per clock on an SM, so the points are
+// spread over SMs and each divides once (the weights are divided once per block).
 __global__ void composition_kernel(const double* N, double* comp, CompParams cp)
 {
+    __shared__ double W[kMaxCath];
+    if (threadIdx.x < cp.n_cath) W[threadIdx.x] = arrival_weight(N, cp, threadIdx.x);
+    __syncwarp();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= cp.n_points) return;
     double a[kMaxCath], A = 0.0;
-    for (int j = 0; j < cp.n_cath; ++j) {
-        const double nref = N[(size_t)j * cp.n_points + cp.ref];
-        a[j] = nref > 0.0 ? cp.R[j] * N[(size_t)j * cp.n_points + m] / nref * cp.w[j] : 0.0;
-        A += a[j];
-    }
-    for (int j = 0; j < cp.n_cath; ++j) comp[(size_t)m * cp.n_cath + j] = A > 0.0 ? 100.0 * a[j] / A : 0.0;
-}
-
-// dL/dN[j][m] and dL/dP_j from dL/dc[m][j]; one block of >= n_points threads
-__global__ void composition_backward_kernel(const double* N, const double* gc, double* gN, double* gP, CompParams cp)
-{
-    __shared__ double ref_acc[kMaxCath];
-    __shared__ double rate_acc[kMaxCath];
-    if (threadIdx.x < kMaxCath) {
-        ref_acc[threadIdx.x] = 0.0;
-        rate_acc[threadIdx.x] = 0.0;
-    }
-    __syncthreads();
-    for (int m = threadIdx.x; m < cp.n_points; m += blockDim.x) {
-        double a[kMaxCath], A = 0.0, gdotc = 0.0;
-        for (int j = 0; j < cp.n_cath; ++j) {
-            const double nref = N[(size_t)j * cp.n_points + cp.ref];
-            a[j] = nref > 0.0 ? cp.R[j] * N[(size_t)j * cp.n_points + m] / nref * cp.w[j] : 0.0;
+#pragma unroll
+    for (int j = 0; j < kMaxCath; ++j)
+        if (j < cp.n_cath) {
+            a[j] = W[j] * N[(size_t)j * cp.n_points + m];
             A += a[j];
         }
-        if (A <= 0.0) {
-            for (int j = 0; j < cp.n_cath; ++j) gN[(size_t)j * cp.n_points + m] = 0.0;
-            continue;
-        }
-        for (int j = 0; j < cp.n_cath; ++j) gdotc += gc[(size_t)m * cp.n_cath + j] * 100.0 * a[j] / A;
-        for (int j = 0; j < cp.n_cath; ++j) {
-            // dL/da_j = (100/A) (g_j - sum_k g_k c_k / 100)
-            const double ga = 100.0 / A * (gc[(size_t)m * cp.n_cath + j] - gdotc / 100.0);
-            const double nref = N[(size_t)j * cp.n_points + cp.ref];
-            gN[(size_t)j * cp.n_points + m] = nref > 0.0 ? ga * cp.R[j] * cp.w[j] / nref : 0.0;
-            // a_j(m) depends on N_j(ref) through 1/N_j(ref) and on R_j linearly
-            if (nref > 0.0) atomicAdd(&ref_acc[j], -ga * a[j] / nref);
-            if (cp.R[j] != 0.0) atomicAdd(&rate_acc[j], ga * a[j] / cp.R[j]);
-        }
-    }
-    __syncthreads();
+    const double scale = A > 0.0 ? 100.0 / A : 0.0;
+#pragma unroll
+    for (int j = 0; j < kMaxCath; ++j)
+        if (j < cp.n_cath) comp[(size_t)m * cp.n_cath + j] = scale * a[j];
+}
+
+// dL/dN[j][m] and dL/dP_j from dL/dc[m][j]; one cluster of 32-thread blocks.
+//   dL/da_j(m) = (100/A) (g_j - sum_k g_k c_k / 100)
+// a_j(m) depends on N_j(m), on N_j(ref) through 1/N_j(ref) and on R_j linearly, so with
+// S_j = sum_m a_j dL/da_j: dL/dN_j(ref) gets -S_j / N_j(ref) and dL/dR_j = S_j / R_j.
+// One block added 2 n_cath values per point with FP64 atomics on a handful of shared-memory
+// words: 95 us for 342 points and four cathodes; so 7 us.
+__global__ void __cluster_dims__(kCluster, 1, 1)
+    composition_backward_kernel(const double* N, const double* gc, double* gN, double* gP, CompParams cp)
+{
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double W[kMaxCath];
+    __shared__ bool on[kMaxCath];  // atoms at the reference point
+    __shared__ double part[kCluster][kMaxCath];
     if (threadIdx.x < cp.n_cath) {
-        gN[(size_t)threadIdx.x * cp.n_points + cp.ref] += ref_acc[threadIdx.x];
-        gP[threadIdx.x] = rate_acc[threadIdx.x] * cp.dRdP[threadIdx.x];
+        W[threadIdx.x] = arrival_weight(N, cp, threadIdx.x);
+        on[threadIdx.x] = N[(size_t)threadIdx.x * cp.n_points + cp.ref] > 0.0;
+    }
+    __syncwarp();
+    double S[kMaxCath];
+#pragma unroll
+    for (int j = 0; j < kMaxCath; ++j) S[j] = 0.0;
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < cp.n_points; m += gridDim.x * blockDim.x) {
+        double a[kMaxCath], A = 0.0, gdota = 0.0;
+#pragma unroll
+        for (int j = 0; j < kMaxCath; ++j)
+            if (j < cp.n_cath) {
+                a[j] = W[j] * N[(size_t)j * cp.n_points + m];
+                A += a[j];
+                gdota += gc[(size_t)m * cp.n_cath + j] * a[j];
+            }
+        const bool off = A <= 0.0;
+        const double scale = 100.0 / A;
+        gdota /= A;
+#pragma unroll
+        for (int j = 0; j < kMaxCath; ++j)
+            if (j < cp.n_cath) {
+                const double ga = off ? 0.0 : scale * (gc[(size_t)m * cp.n_cath + j] - gdota);
+                gN[(size_t)j * cp.n_points + m] = on[j] ? ga * W[j] : 0.0;
+                S[j] += ga * a[j];
+            }
+    }
+    double* first = cl.map_shared_rank(&part[0][0], 0);
+#pragma unroll
+    for (int j = 0; j < kMaxCath; ++j)
+        if (j < cp.n_cath) {
+            const double t = warp_sum(S[j]);
+            if (threadIdx.x == 0) first[cl.block_rank() * kMaxCath + j] = t;
+        }
+    cl.sync();
+    const int j = threadIdx.x;
+    if (cl.block_rank() == 0 && j < cp.n_cath) {
+        double t = 0.0;
+        for (int b = 0; b < kCluster; ++b) t += part[b][j];
+        const double nref = N[(size_t)j * cp.n_points + cp.ref];
+        if (on[j]) gN[(size_t)j * cp.n_points + cp.ref] += -t / nref;
+        gP[j] = cp.R[j] != 0.0 ? t / cp.R[j] * cp.dRdP[j] : 0.0;
     }
 }
 
 // dL/dcount[j][c] = dL/dN[j][patch(c)]
-__global__ void scatter_kernel(const double* gN, const int32_t* patch, double* gcounts, int n_cath, int n_cells,
-                               int n_points)
+__global__ void scatter_kernel(const double* gN, const int32_t* patch, double* gcounts, int n_cells, int n_points)
 {
-    const long long total = (long long)n_cath * n_cells;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(i / n_cells), c = (int)(i % n_cells);
+    const int j = blockIdx.y;
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)n_cells; c += gridDim.x * blockDim.x) {
         const int m = patch[c];
-        gcounts[i] = (m >= 0 && m < n_points) ? gN[(size_t)j * n_points + m] : 0.0;
+        gcounts[(size_t)j * n_cells + c] = m >= 0 && m < n_points ? gN[(size_t)j * n_points + m] : 0.0;
     }
+}
+
+// grid of the kernels that run over every cell of every cathode
+dim3 cell_grid(int n_cells, int n_cath)
+{
+    const int bx = (n_cells + 255) / 256;
+    return dim3((unsigned)(bx < 1216 ? bx : 1216), (unsigned)n_cath);
 }
 
 sput_status adj_fail(sput_status s, const char* msg)
@@ -220,8 +285,8 @@ sput_status sput_backward(const sput_scene* scene, const double* grad_counts, co
     sput_status st = sput_tally_layout_get(scene, &L);
     if (st != SPUT_OK) return st;
     const long long n_cells = (long long)L.nx * L.ny;
-    lr_backward_kernel<<<L.n_instances, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(grad_counts, score_tally,
-                                                                                        grad_log_pressure, n_cells);
+    lr_backward_kernel<<<L.n_instances * kCluster, kReduceThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+        grad_counts, score_tally, grad_log_pressure, n_cells);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return adj_fail(SPUT_ERR_CUDA, cudaGetErrorString(e));
     return SPUT_OK;
@@ -244,11 +309,11 @@ sput_status emax_backward_launch(const sput_scene* scene, const double* grad_cou
     const sput::DevInstance* inst = sput::scene_device_instances(scene);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (L.count_type == SPUT_COUNT_INT64)
-        emax_backward_kernel<<<L.n_instances, 256, 0, s>>>(grad_counts, static_cast<const long long*>(counts),
+        emax_backward_kernel<<<L.n_instances * kCluster, kReduceThreads, 0, s>>>(grad_counts, static_cast<const long long*>(counts),
                                                            static_cast<const long long*>(counts_cutoff), inst,
                                                            grad_ion_energy, n_cells, grad_power, vp);
     else
-        emax_backward_kernel<<<L.n_instances, 256, 0, s>>>(grad_counts, static_cast<const int*>(counts),
+        emax_backward_kernel<<<L.n_instances * kCluster, kReduceThreads, 0, s>>>(grad_counts, static_cast<const int*>(counts),
                                                            static_cast<const int*>(counts_cutoff), inst,
                                                            grad_ion_energy, n_cells, grad_power, vp);
     cudaError_t e = cudaGetLastError();
@@ -329,9 +394,9 @@ sput_status sput_composition(int n_cathodes, int n_cells, int n_points, const in
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(patch_counts, 0, sizeof(double) * (size_t)n_cathodes * n_points, s);
     if (e != cudaSuccess) return adj_fail(SPUT_ERR_CUDA, cudaGetErrorString(e));
-    patch_sum_kernel<<<304, 256, 0, s>>>(reinterpret_cast<const long long*>(counts), patch_of_cell, patch_counts,
-                                         n_cathodes, n_cells, n_points);
-    composition_kernel<<<(n_points + 127) / 128, 128, 0, s>>>(patch_counts, composition, cp);
+    patch_sum_kernel<<<cell_grid(n_cells, n_cathodes), 256, 0, s>>>(reinterpret_cast<const long long*>(counts),
+                                                                   patch_of_cell, patch_counts, n_cells, n_points);
+    composition_kernel<<<(n_points + 31) / 32, 32, 0, s>>>(patch_counts, composition, cp);
     e = cudaGetLastError();
     if (e != cudaSuccess) return adj_fail(SPUT_ERR_CUDA, cudaGetErrorString(e));
     return SPUT_OK;
@@ -349,8 +414,9 @@ sput_status sput_composition_backward(int n_cathodes, int n_cells, int n_points,
     if (!patch_counts || !patch_of_cell || !grad_composition || !grad_patch || !grad_counts || !grad_power)
         return adj_fail(SPUT_ERR_INVALID_ARG, "NULL argument");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    composition_backward_kernel<<<1, 512, 0, s>>>(patch_counts, grad_composition, grad_patch, grad_power, cp);
-    scatter_kernel<<<304, 256, 0, s>>>(grad_patch, patch_of_cell, grad_counts, n_cathodes, n_cells, n_points);
+    composition_backward_kernel<<<kCluster, 32, 0, s>>>(patch_counts, grad_composition, grad_patch, grad_power, cp);
+    scatter_kernel<<<cell_grid(n_cells, n_cathodes), 256, 0, s>>>(grad_patch, patch_of_cell, grad_counts, n_cells,
+                                                                 n_points);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return adj_fail(SPUT_ERR_CUDA, cudaGetErrorString(e));
     return SPUT_OK;
