@@ -1028,10 +1028,11 @@ __device__ __forceinline__ void deflect_off_table(const TableView& T, const DevP
 }
 
 // Binary collision in the CM frame: rotate g = v - V by (chi, psi), |g| kept; the atom's speed and
-// direction (of velocity v) become those after it.  One rare branch (off the deflection
-// table); the rest is straight-line code.
-template <int kMode>
-__device__ __forceinline__ void scatter(float& speed, float& dx, float& dy, float& dz, const Params& P,
+// direction (of velocity v) become those after it.  Straight-line code but for one rare branch
+// (off the deflection table); with kTable (the scene has a table) not even that: the
+// result is void where the return value is true, and the caller computes it without kTable.
+template <int kMode, bool kTable>
+__device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, float& dz, const Params& P,
                                         const TableView& T, const DevPair& pr, float vx, float vy, float vz, float Vx,
                                         float Vy, float Vz, const Impact& I)
 {
@@ -1045,11 +1046,11 @@ __device__ __forceinline__ void scatter(float& speed, float& dx, float& dy, floa
     const float le = logf(eps);
     float sc, cc, q = 0.0f;
     bool on_table = false;
-    if (P.chi_tab) {
+    if (kTable || P.chi_tab) {
         on_table = chi_table_q(P.chi_tab, P.status, le, max(I.j, 0), I.ty, q) && I.j >= 0;
         chi_cos_sin(q, cc, sc);
     }
-    if (!on_table && g2 > 0.0f) deflect_off_table(T, pr, eps, le, I.ub, cc, sc);
+    if (!kTable && !on_table && g2 > 0.0f) deflect_off_table(T, pr, eps, le, I.ub, cc, sc);
     const float sp = -I.nsp, cp = -I.ncp;
     float3 b1, b2;
     onb(hx, hy, hz, b1, b2);
@@ -1075,6 +1076,7 @@ __device__ __forceinline__ void scatter(float& speed, float& dx, float& dy, floa
             dz = uz * is;
         }
     }
+    return kTable && !on_table && g2 > 0.0f;
 }
 
 // Isotropic direction of the diffusion shortcut's walk from the flight block's words 1 and 2.
@@ -1128,7 +1130,7 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
             S.scoreT = fmaf(score_T_partner(P, sumsq_xyz(Vx, Vy, Vz), out.Gv), P.inv_T, S.scoreT);
     }
     if (coll) {
-        scatter<kMode>(S.speed, S.dx, S.dy, S.dz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, impact_draw(w));
+        scatter<kMode, false>(S.speed, S.dx, S.dy, S.dz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, impact_draw(w));
         if (kMode == kModeWalk && energy_of(P, S.inst, S.speed) < P.E_switch) S.diff = true;
     } else if (walk) {
         walk_direction(w, S.dx, S.dy, S.dz);
@@ -1550,6 +1552,109 @@ __host__ __device__ inline DrainLayout drain_layout(const Params& p)
     return L;
 }
 
+// The batch's collisions, one after the other (2. above): S goes through them; F, in lane f of the
+// group, keeps the velocity before flight f, and att and V2 its partner's attempts and |V|^2.
+// kFast: thermal gas and a deflection table, so that a step is one run of straight-line code in
+// which the loads and the MUFU overlap.
+template <int kMode, bool kFast>
+__device__ __forceinline__ void drain_collisions(Lane& S, Lane& F, const Params& P, const TableView& T,
+                                                 const DrainWarp& W, const DevPair& pr, bool have, int head, int l,
+                                                 int G, uint32_t& att, float& V2)
+{
+    constexpr bool kScoreT = kMode == kModeScoreT;
+    const bool thermal = kFast || P.gas_thermal;
+    const int A = P.max_attempts;
+    const int my_a = l & (kDrawn - 1);
+    const bool my_branch = (l & kDrawn) != 0;
+#pragma unroll 1
+    for (int f = 0; f < G; ++f) {
+        if (l == f) {
+            F.speed = S.speed;
+            F.dx = S.dx;
+            F.dy = S.dy;
+            F.dz = S.dz;
+            F.diff = S.diff;
+        }
+        const bool walk = kMode == kModeWalk && S.diff;
+        bool pend = have && !walk;
+        if (kMode == kModeWalk && walk) {
+            const float4 d = W.walk[head + f];
+            S.dx = d.x;
+            S.dy = d.y;
+            S.dz = d.z;
+        }
+        if (kMode == kModeWalk && !__any_sync(kFull, pend)) continue;
+        const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
+        float EA = 0.0f, EB = 0.0f;
+        if (thermal) {
+            int i;
+            float t;
+            wtab_cell(pr, S.speed, i, t);
+            EA = wtab_at(T, pr, kTabA, i, t);
+            EB = wtab_at(T, pr, kTabB, i, t);
+        }
+        const Impact h = W.hit[head + f];
+        const float4 z = W.z[head + f][my_a], r = W.rho[head + f][my_a];
+        Attempt d;
+        d.z1 = z.x;
+        d.z2 = z.y;
+        d.z3 = z.z;
+        d.u = z.w;
+        d.r3 = r.x;
+        d.rho_w = r.y;
+        d.sc_w = r.z;
+        for (int a = my_a;;) {
+            // the collision with this lane's attempt in its branch, and whether it is the one
+            float cx = 0.0f, cy = 0.0f, cz = 0.0f;
+            bool acc = true;
+            if (thermal) attempt_velocity(P, d, my_branch, cx, cy, cz);
+            float ns = S.speed, nx = S.dx, ny = S.dy, nz = S.dz;
+            const bool off = scatter<kMode, kFast>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, cx, cy, cz, h);
+            if (thermal) {
+                float ut, Bm;
+                const bool weighted = attempt_weighted(d, EA, EB, ut, Bm);
+                const float hg = attempt_h(T, pr, vx, vy, vz, cx, cy, cz);
+                const bool ok = attempt_accept(d, my_branch, ut, Bm, EA, EB, hg);
+                acc = (a < A) & (weighted == my_branch) & (ok | (a == A - 1));
+            }
+            // the first accepted attempt, in either branch
+            const unsigned m = __ballot_sync(kFull, acc) >> head;
+            const unsigned first = (m | m >> kDrawn) & ((1u << kDrawn) - 1u);
+            int src = first ? __ffs(first) - 1 : 0;
+            const uint32_t n_att = (uint32_t)(a - my_a + src) + 1u;
+            if (!((m >> src) & 1u)) src += kDrawn;
+            if (kFast && off) {  // rare
+                ns = S.speed;
+                nx = S.dx;
+                ny = S.dy;
+                nz = S.dz;
+                scatter<kMode, false>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, cx, cy, cz, h);
+            }
+            ns = __shfl_sync(kFull, ns, head + src);
+            nx = __shfl_sync(kFull, nx, head + src);
+            ny = __shfl_sync(kFull, ny, head + src);
+            nz = __shfl_sync(kFull, nz, head + src);
+            const float c2 = kScoreT ? __shfl_sync(kFull, sumsq_xyz(cx, cy, cz), head + src) : 0.0f;
+            if (pend && first) {
+                S.speed = ns;
+                S.dx = nx;
+                S.dy = ny;
+                S.dz = nz;
+                if (l == f) {
+                    att = thermal ? n_att : 0u;
+                    V2 = c2;
+                }
+                if (kMode == kModeWalk && energy_of(P, S.inst, S.speed) < P.E_switch) S.diff = true;
+                pend = false;
+            }
+            if (!__any_sync(kFull, pend)) break;
+            // rare: none of the drawn attempts; the group draws four more
+            a += kDrawn;
+            d = attempt_draw(P, S.pid, S.strm, S.k + 1u + f, (uint32_t)a);
+        }
+    }
+}
+
 template <int kMode, int kMasks>
 __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
 {
@@ -1591,7 +1696,6 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     T.status = P.status;
 
     const int lane = threadIdx.x & 31;
-    const int A = P.max_attempts;
     Lane S;  // the group's atom, the same in its lanes
     S.px = S.py = S.pz = S.dx = S.dy = S.dz = S.speed = S.score = S.scoreT = 0.0f;
     S.pid = S.inst = S.k = 0u;
@@ -1703,88 +1807,8 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
         uint32_t att = 0u;
         float V2 = 0.0f;
         const DevPair& pr = s_pairs[S.pair];
-        const int my_a = l & (kDrawn - 1);
-        const bool my_branch = (l & kDrawn) != 0;
-#pragma unroll 1
-        for (int f = 0; f < G; ++f) {
-            if (l == f) {
-                F.speed = S.speed;
-                F.dx = S.dx;
-                F.dy = S.dy;
-                F.dz = S.dz;
-                F.diff = S.diff;
-            }
-            const bool walk = kMode == kModeWalk && S.diff;
-            bool pend = have && !walk;
-            if (kMode == kModeWalk && walk) {
-                const float4 d = W.walk[head + f];
-                S.dx = d.x;
-                S.dy = d.y;
-                S.dz = d.z;
-            }
-            if (kMode == kModeWalk && !__any_sync(kFull, pend)) continue;
-            const float vx = __fmul_rn(S.speed, S.dx), vy = __fmul_rn(S.speed, S.dy), vz = __fmul_rn(S.speed, S.dz);
-            float EA = 0.0f, EB = 0.0f;
-            if (P.gas_thermal) {
-                int i;
-                float t;
-                wtab_cell(pr, S.speed, i, t);
-                EA = wtab_at(T, pr, kTabA, i, t);
-                EB = wtab_at(T, pr, kTabB, i, t);
-            }
-            const Impact h = W.hit[head + f];
-            const float4 z = W.z[head + f][my_a], r = W.rho[head + f][my_a];
-            Attempt d;
-            d.z1 = z.x;
-            d.z2 = z.y;
-            d.z3 = z.z;
-            d.u = z.w;
-            d.r3 = r.x;
-            d.rho_w = r.y;
-            d.sc_w = r.z;
-            for (int a = my_a;;) {
-                // the collision with this lane's attempt in its branch, and whether it is the one
-                float cx = 0.0f, cy = 0.0f, cz = 0.0f;
-                bool acc = true;
-                if (P.gas_thermal) {
-                    float ut, Bm;
-                    const bool weighted = attempt_weighted(d, EA, EB, ut, Bm);
-                    attempt_velocity(P, d, my_branch, cx, cy, cz);
-                    const float hg = attempt_h(T, pr, vx, vy, vz, cx, cy, cz);
-                    acc = a < A && weighted == my_branch &&
-                          (attempt_accept(d, my_branch, ut, Bm, EA, EB, hg) || a == A - 1);
-                }
-                float ns = S.speed, nx = S.dx, ny = S.dy, nz = S.dz;
-                scatter<kMode>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, cx, cy, cz, h);
-                // the first accepted attempt, in either branch
-                const unsigned m = __ballot_sync(kFull, acc) >> head;
-                const unsigned first = (m | m >> kDrawn) & ((1u << kDrawn) - 1u);
-                int src = first ? __ffs(first) - 1 : 0;
-                const uint32_t n_att = (uint32_t)(a - my_a + src) + 1u;
-                if (!((m >> src) & 1u)) src += kDrawn;
-                ns = __shfl_sync(kFull, ns, head + src);
-                nx = __shfl_sync(kFull, nx, head + src);
-                ny = __shfl_sync(kFull, ny, head + src);
-                nz = __shfl_sync(kFull, nz, head + src);
-                const float c2 = kScoreT ? __shfl_sync(kFull, sumsq_xyz(cx, cy, cz), head + src) : 0.0f;
-                if (pend && first) {
-                    S.speed = ns;
-                    S.dx = nx;
-                    S.dy = ny;
-                    S.dz = nz;
-                    if (l == f) {
-                        att = P.gas_thermal ? n_att : 0u;
-                        V2 = c2;
-                    }
-                    if (kMode == kModeWalk && energy_of(P, S.inst, S.speed) < P.E_switch) S.diff = true;
-                    pend = false;
-                }
-                if (!__any_sync(kFull, pend)) break;
-                // rare: none of the drawn attempts; the group draws four more
-                a += kDrawn;
-                d = attempt_draw(P, S.pid, S.strm, S.k + 1u + f, (uint32_t)a);
-            }
-        }
+        if (P.gas_thermal && P.chi_tab) drain_collisions<kMode, true>(S, F, P, T, W, pr, have, head, l, G, att, V2);
+        else drain_collisions<kMode, false>(S, F, P, T, W, pr, have, head, l, G, att, V2);
 
         // ---------------------------------------------------- 3. flights
         float inv_lam = 0.0f, ell = 0.0f, Gv = 0.0f;
