@@ -147,10 +147,12 @@ __device__ __forceinline__ float wtab_G(const TableView& T, const DevPair& pr, i
 }
 
 // sigma(g) g in A^2 km/s
+// (kMoliere: known not to be hard spheres)
+template <bool kMoliere>
 __device__ __forceinline__ float h_of_g(const TableView& T, const DevPair& pr, float g, float g2)
 {
     const float b = bmax_eval(T, __logf(pr.kappa * g2));
-    return pr.hard_sphere ? pr.sigma_scale * g : pr.sigma_scale * b * b * g;
+    return !kMoliere && pr.hard_sphere ? pr.sigma_scale * g : pr.sigma_scale * b * b * g;
 }
 
 // 1 - exp(-y) without cancellation for small y
@@ -872,11 +874,12 @@ __device__ __forceinline__ void attempt_velocity(const Params& P, const Attempt&
 }
 
 // h(g) = sigma(g) g between the atom's velocity v and the gas velocity c
+template <bool kMoliere>
 __device__ __forceinline__ float attempt_h(const TableView& T, const DevPair& pr, float vx, float vy, float vz, float cx,
                                            float cy, float cz)
 {
     const float g2 = sumsq_yxz(__fsub_rn(vx, cx), __fsub_rn(vy, cy), __fsub_rn(vz, cz));
-    return h_of_g(T, pr, sqrt_fast(g2), g2);
+    return h_of_g<kMoliere>(T, pr, sqrt_fast(g2), g2);
 }
 
 // Acceptance: the branch's own uniform, rescaled to (0, 1], times the envelope against h.
@@ -957,7 +960,7 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
             float ut, Bm;
             const bool weighted = attempt_weighted(d, o_A, o_B, ut, Bm);
             attempt_velocity(P, d, weighted, cx, cy, cz);
-            const float hg = attempt_h(T, pairs[op], o_vx, o_vy, o_vz, cx, cy, cz);
+            const float hg = attempt_h<false>(T, pairs[op], o_vx, o_vy, o_vz, cx, cy, cz);
             acc = attempt_accept(d, weighted, ut, Bm, o_A, o_B, hg) || a == A - 1;
         }
         const unsigned accm = __ballot_sync(kFull, acc);
@@ -1001,8 +1004,8 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
 // The draws of a collision, from its flight's Philox block.
 struct Impact {
     float ub;        // uniform of the impact parameter b = b_max sqrt(ub)
-    int j;           // column of ln(ub)/2 in the deflection table, -1 below it
-    float ty;
+    int j;           // column of ln(ub)/2 in the deflection table and position in it; below the
+    float ty;        // table 0 and -1
     float nsp, ncp;  // negated sine and cosine of the azimuth
 };
 
@@ -1010,7 +1013,10 @@ __device__ __forceinline__ Impact impact_draw(const uint4& w)
 {
     Impact I;
     I.ub = rn(w.y);
-    if (!chi_table_column(0.5f * logf(I.ub), I.j, I.ty)) I.j = -1;
+    if (!chi_table_column(0.5f * logf(I.ub), I.j, I.ty)) {
+        I.j = 0;
+        I.ty = -1.0f;
+    }
     neg_sincos_2pi_fast(rn(w.z), &I.nsp, &I.ncp);
     return I;
 }
@@ -1028,10 +1034,11 @@ __device__ __forceinline__ void deflect_off_table(const TableView& T, const DevP
 }
 
 // Binary collision in the CM frame: rotate g = v - V by (chi, psi), |g| kept; the atom's speed and
-// direction (of velocity v) become those after it.  Straight-line code but for one rare branch
-// (off the deflection table); with kTable (the scene has a table) not even that: the
-// result is void where the return value is true, and the caller computes it without kTable.
-template <int kMode, bool kTable>
+// direction (of velocity v) become those after it.  kUsual (the scene has a deflection table):
+// straight-line code for what nearly every collision is, on the table, with a relative speed
+// and a speed afterwards whose squares do not underflow; otherwise it returns false, with the
+// result void, and the caller computes the collision without kUsual.
+template <int kMode, bool kUsual>
 __device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, float& dz, const Params& P,
                                         const TableView& T, const DevPair& pr, float vx, float vy, float vz, float Vx,
                                         float Vy, float Vz, const Impact& I)
@@ -1046,11 +1053,11 @@ __device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, floa
     const float le = logf(eps);
     float sc, cc, q = 0.0f;
     bool on_table = false;
-    if (kTable || P.chi_tab) {
-        on_table = chi_table_q(P.chi_tab, P.status, le, max(I.j, 0), I.ty, q) && I.j >= 0;
+    if (kUsual || P.chi_tab) {
+        on_table = chi_table_q(P.chi_tab, P.status, le, I.j, I.ty, q);
         chi_cos_sin(q, cc, sc);
     }
-    if (!kTable && !on_table && g2 > 0.0f) deflect_off_table(T, pr, eps, le, I.ub, cc, sc);
+    if (!kUsual && g2 > 0.0f && !(on_table && I.ty >= 0.0f)) deflect_off_table(T, pr, eps, le, I.ub, cc, sc);
     const float sp = -I.nsp, cp = -I.ncp;
     float3 b1, b2;
     onb(hx, hy, hz, b1, b2);
@@ -1060,6 +1067,17 @@ __device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, floa
     const float nvx = fmaf(pr.m2M, gpx, dot2(pr.m1M, vx, pr.m2M, Vx));
     const float nvy = fmaf(pr.m2M, gpy, dot2(pr.m1M, vy, pr.m2M, Vy));
     const float nvz = fmaf(pr.m2M, gpz, dot2(pr.m1M, vz, pr.m2M, Vz));
+    if (kUsual) {
+        const float sp2 = sumsq_yxz(nvx, nvy, nvz);
+        const float is = rsqrtf(sp2);
+        speed = sp2 * is;
+        dx = nvx * is;
+        dy = nvy * is;
+        dz = nvz * is;
+        // (2e-30: above the limit of the scaling below, however the sums round; the NaN of g2 = 0
+        // fails it too)
+        return on_table && I.ty >= 0.0f && sp2 > 2e-30f;
+    }
     // an atom slowed to ~1e-15 km/s or below (gas at rest) would underflow the
     // squares: scale by the exact power of two 2^60 first
     const float up = sumsq_xyz(nvx, nvy, nvz) < 1e-30f ? 0x1p60f : 1.0f;
@@ -1076,7 +1094,7 @@ __device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, floa
             dz = uz * is;
         }
     }
-    return kTable && !on_table && g2 > 0.0f;
+    return true;
 }
 
 // Isotropic direction of the diffusion shortcut's walk from the flight block's words 1 and 2.
@@ -1130,7 +1148,18 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
             S.scoreT = fmaf(score_T_partner(P, sumsq_xyz(Vx, Vy, Vz), out.Gv), P.inv_T, S.scoreT);
     }
     if (coll) {
-        scatter<kMode, false>(S.speed, S.dx, S.dy, S.dz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, impact_draw(w));
+        const Impact I = impact_draw(w);
+        float ns = 0.0f, nx = 0.0f, ny = 0.0f, nz = 0.0f;
+        bool usual = false;
+        if (P.chi_tab) usual = scatter<kMode, true>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, I);
+        if (usual) {
+            S.speed = ns;
+            S.dx = nx;
+            S.dy = ny;
+            S.dz = nz;
+        } else {
+            scatter<kMode, false>(S.speed, S.dx, S.dy, S.dz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, I);
+        }
         if (kMode == kModeWalk && energy_of(P, S.inst, S.speed) < P.E_switch) S.diff = true;
     } else if (walk) {
         walk_direction(w, S.dx, S.dy, S.dz);
@@ -1609,11 +1638,11 @@ __device__ __forceinline__ void drain_collisions(Lane& S, Lane& F, const Params&
             bool acc = true;
             if (thermal) attempt_velocity(P, d, my_branch, cx, cy, cz);
             float ns = S.speed, nx = S.dx, ny = S.dy, nz = S.dz;
-            const bool off = scatter<kMode, kFast>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, cx, cy, cz, h);
+            const bool usual = scatter<kMode, kFast>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, cx, cy, cz, h);
             if (thermal) {
                 float ut, Bm;
                 const bool weighted = attempt_weighted(d, EA, EB, ut, Bm);
-                const float hg = attempt_h(T, pr, vx, vy, vz, cx, cy, cz);
+                const float hg = attempt_h<kFast>(T, pr, vx, vy, vz, cx, cy, cz);
                 const bool ok = attempt_accept(d, my_branch, ut, Bm, EA, EB, hg);
                 acc = (a < A) & (weighted == my_branch) & (ok | (a == A - 1));
             }
@@ -1623,7 +1652,7 @@ __device__ __forceinline__ void drain_collisions(Lane& S, Lane& F, const Params&
             int src = first ? __ffs(first) - 1 : 0;
             const uint32_t n_att = (uint32_t)(a - my_a + src) + 1u;
             if (!((m >> src) & 1u)) src += kDrawn;
-            if (kFast && off) {  // rare
+            if (kFast && !usual) {  // rare
                 ns = S.speed;
                 nx = S.dx;
                 ny = S.dy;
