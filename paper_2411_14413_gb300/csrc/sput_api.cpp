@@ -138,7 +138,8 @@ struct sput_scene {
     size_t stage_bytes = 0;
     cudaStream_t own_stream = nullptr;
     Params base{};
-    int smem_counters_fit = 0;  // per-primitive counters fit in shared memory
+    int smem_counters_fit = 0;   // per-primitive counters fit in shared memory
+    int smem_counters_free = 0;  // and leave as many blocks per SM as without
     // launch shape for opts fields left 0 (set by sput_autotune)
     int def_threads = 256, def_bps = 0, def_chunk = 32, def_flags = 0;
 };
@@ -799,6 +800,13 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
         }
     }
     S->smem_counters_fit = p.smem_counters;
+    if (p.smem_counters) {
+        // 512 instances of 16 primitives take 35 KB of them: two blocks per SM instead of four
+        Params q = p;
+        q.smem_counters = 0;
+        S->smem_counters_free = transport_max_blocks_per_sm(256, transport_smem_bytes(p)) ==
+                                transport_max_blocks_per_sm(256, transport_smem_bytes(q));
+    }
     if (drain_smem_bytes(p) <= S->smem_optin) S->drain_bps = drain_max_blocks_per_sm(drain_smem_bytes(p));
     *out = S;
     return SPUT_OK;
@@ -927,7 +935,10 @@ sput_status run_impl(sput_scene* S, const sput_run_opts* opts, cudaStream_t stre
     p.ticket_counter = scratch;
     p.stats = scratch + 1;
     p.status = reinterpret_cast<unsigned int*>(scratch + 1 + kNumStats);
-    p.smem_counters = (flags & SPUT_RUN_NO_SMEM_COUNTERS) ? 0 : S->smem_counters_fit;
+    // counters in shared memory: where they fit and, unless asked for, cost no resident block
+    p.smem_counters = flags & SPUT_RUN_NO_SMEM_COUNTERS ? 0
+                      : flags & SPUT_RUN_SMEM_COUNTERS  ? S->smem_counters_fit
+                                                        : S->smem_counters_free;
     p.launch_at_cutoff = cutoff ? 1 : 0;
     p.inject_nonfinite = (opts->flags & SPUT_RUN_INJECT_NONFINITE) ? 1 : 0;
     const bool masks =
