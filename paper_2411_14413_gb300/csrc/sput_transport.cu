@@ -108,7 +108,7 @@ __device__ __forceinline__ float bmax_eval(const TableView& T, float ln_eps)
     int i;
     float t;
     table_cell(fminf(fmaxf((ln_eps - T.bm_lo) * T.bm_inv_h, 0.0f), T.bm_n), T.bm_top, i, t);
-    return cubic(T.bm[i], t);
+    return cubic(__ldg(T.bm + i), t);
 }
 
 __device__ __forceinline__ float xh_eval(const TableView& T, float ln_eps)
@@ -1283,7 +1283,7 @@ __device__ __forceinline__ void tally_timed_out(const Params& P, const Lane& S, 
 
 // ------------------------------------------------------------- kernel
 struct SmemLayout {
-    size_t prims, geoms, pairs, bm, prefix, gm, pool, queue, scratch, counters, total;
+    size_t prims, geoms, pairs, prefix, gm, pool, queue, scratch, counters, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -1298,8 +1298,6 @@ __host__ __device__ inline SmemLayout smem_layout(const Params& p)
     o = align16(o + sizeof(DevGeom) * p.n_geoms);
     L.pairs = o;
     o = align16(o + sizeof(DevPair) * p.n_pairs);
-    L.bm = o;
-    o = align16(o + sizeof(float4) * p.n_bm);
     L.prefix = o;
     o = align16(o + sizeof(unsigned long long) * (p.n_inst + 1));
     L.gm = o;
@@ -1339,7 +1337,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     DevPrim* s_prims = reinterpret_cast<DevPrim*>(smem + L.prims);
     DevGeom* s_geoms = reinterpret_cast<DevGeom*>(smem + L.geoms);
     DevPair* s_pairs = reinterpret_cast<DevPair*>(smem + L.pairs);
-    float4* s_bm = reinterpret_cast<float4*>(smem + L.bm);
     unsigned long long* s_prefix = reinterpret_cast<unsigned long long*>(smem + L.prefix);
     float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
     unsigned long long* s_pool = reinterpret_cast<unsigned long long*>(smem + L.pool);
@@ -1349,7 +1346,6 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     copy16(s_prims, P.prims, sizeof(DevPrim) * P.n_prims);
     copy16(s_geoms, P.geoms, sizeof(DevGeom) * P.n_geoms);
     copy16(s_pairs, P.pairs, sizeof(DevPair) * P.n_pairs);
-    copy16(s_bm, P.bm_tab, sizeof(float4) * P.n_bm);
     copy16(s_prefix, P.prefix, sizeof(unsigned long long) * (P.n_inst + 1));
     if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
     else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
@@ -1358,7 +1354,7 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
     __syncthreads();
 
     TableView T;
-    T.bm = s_bm;
+    T.bm = P.bm_tab;
     T.xh = P.xh_tab;  // (off the deflection table only: stays in global memory)
     T.w = P.w_tab;
     T.gm = s_gm;
@@ -1558,7 +1554,7 @@ struct DrainWarp {                // by the flight's lane
 };
 
 struct DrainLayout {
-    size_t prims, geoms, pairs, bm, gm, warps, total;
+    size_t prims, geoms, pairs, gm, warps, total;
 };
 
 __host__ __device__ inline DrainLayout drain_layout(const Params& p)
@@ -1573,8 +1569,6 @@ __host__ __device__ inline DrainLayout drain_layout(const Params& p)
     o = align16(o + sizeof(DevGeom) * p.n_geoms);
     L.pairs = o;
     o = align16(o + sizeof(DevPair) * p.n_pairs);
-    L.bm = o;
-    o = align16(o + sizeof(float4) * p.n_bm);
     L.gm = o;
     o = align16(o + sizeof(float4) * (kGMHalf + kGMHalfLo));
     L.total = o;
@@ -1699,19 +1693,17 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     DevPrim* s_prims = reinterpret_cast<DevPrim*>(smem + L.prims);
     DevGeom* s_geoms = reinterpret_cast<DevGeom*>(smem + L.geoms);
     DevPair* s_pairs = reinterpret_cast<DevPair*>(smem + L.pairs);
-    float4* s_bm = reinterpret_cast<float4*>(smem + L.bm);
     float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
     DrainWarp& W = reinterpret_cast<DrainWarp*>(smem + L.warps)[threadIdx.x >> 5];
     copy16(s_prims, P.prims, sizeof(DevPrim) * P.n_prims);
     copy16(s_geoms, P.geoms, sizeof(DevGeom) * P.n_geoms);
     copy16(s_pairs, P.pairs, sizeof(DevPair) * P.n_pairs);
-    copy16(s_bm, P.bm_tab, sizeof(float4) * P.n_bm);
     if (threadIdx.x < kGMHalf) s_gm[threadIdx.x] = P.gm[threadIdx.x];
     else if (threadIdx.x < kGMHalf + kGMHalfLo) s_gm[threadIdx.x] = P.gm_lo[threadIdx.x - kGMHalf];
     __syncthreads();
 
     TableView T;
-    T.bm = s_bm;
+    T.bm = P.bm_tab;
     T.xh = P.xh_tab;  // (off the deflection table only: stays in global memory)
     T.w = P.w_tab;
     T.gm = s_gm;
