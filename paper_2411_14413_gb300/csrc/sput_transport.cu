@@ -76,6 +76,37 @@ __device__ __forceinline__ bool idx_ok(unsigned int* status, long long i, long l
 #endif
 }
 
+// ------------------------------------------------------------- MUFU functions
+// Approximate functions for arguments that are no denormals: the forms that flush them spare the
+// scaling around the MUFU (a comparison and two or three instructions each, some 25 in a flight
+// and its collision) and give the same result for all others.
+__device__ __forceinline__ float fast_lg2(float x)
+{
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fast_ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fast_rsqrt(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fast_div(float a, float b)
+{
+    float y;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+__device__ __forceinline__ float fast_ln(float x) { return fast_lg2(x) * 0.69314718056f; }
+__device__ __forceinline__ float fast_exp(float x) { return fast_ex2(x * 1.44269504089f); }
+
 // ------------------------------------------------------------- tables
 // Cell and position of a table coordinate x in [0, n], top = 2^23 + n - 1: i = min(floor(x), n - 1),
 // t = x - i.  The sum with 2^23, rounded down, holds floor(x) in its mantissa; a conversion to
@@ -121,7 +152,7 @@ __device__ __forceinline__ float xh_eval(const TableView& T, float ln_eps)
 
 // The rate tables' coordinate w = ln(1 + v/s), from the MUFU logarithm: its error
 // (about 4e-7 absolute) moves K, A and B far less than their interpolation error.
-__device__ __forceinline__ float w_of(const DevPair& pr, float v) { return __logf(1.0f + v * pr.inv_s); }
+__device__ __forceinline__ float w_of(const DevPair& pr, float v) { return fast_ln(1.0f + v * pr.inv_s); }
 
 // K(v), A(v), B(v) and G(v) of a pair: cubic pieces in w = ln(1 + v/s).  K, A and B lie beside one
 // another (three float4 per piece), so one cell lookup serves all three.  The tables are read
@@ -151,7 +182,7 @@ __device__ __forceinline__ float wtab_G(const TableView& T, const DevPair& pr, i
 template <bool kMoliere>
 __device__ __forceinline__ float h_of_g(const TableView& T, const DevPair& pr, float g, float g2)
 {
-    const float b = bmax_eval(T, __logf(pr.kappa * g2));
+    const float b = bmax_eval(T, fast_ln(pr.kappa * g2));
     return !kMoliere && pr.hard_sphere ? pr.sigma_scale * g : pr.sigma_scale * b * b * g;
 }
 
@@ -264,9 +295,9 @@ __device__ __forceinline__ bool chi_table_q(const float4* tab, unsigned int* sta
 // cos chi = (1 - T^2)/(1 + T^2), sin chi = 2T/(1 + T^2)
 __device__ __forceinline__ void chi_cos_sin(float q, float& cc, float& sc)
 {
-    const float Tq = __expf(fminf(q, 40.0f));
+    const float Tq = fast_exp(fminf(q, 40.0f));
     const float T2 = Tq * Tq;
-    const float inv = __fdividef(1.0f, 1.0f + T2);
+    const float inv = fast_div(1.0f, 1.0f + T2);
     cc = (1.0f - T2) * inv;
     sc = 2.0f * Tq * inv;
 }
@@ -288,16 +319,16 @@ __device__ __forceinline__ void sincos_2pi_fast(float u, float* s, float* c)
 
 // -ln u for u in (0, 1] from the MUFU logarithm (absolute error about 2^-21.4 near 1,
 // 3 ulp elsewhere), clamped at 0 where the approximation rounds above zero
-__device__ __forceinline__ float neg_log_fast(float u) { return fmaxf(-__logf(u), 0.0f); }
+__device__ __forceinline__ float neg_log_fast(float u) { return fmaxf(-fast_ln(u), 0.0f); }
 
 // sqrt(x) for x >= 0 as x / sqrt(x) from the MUFU reciprocal square root (about 2 ulp); 0 at 0
-__device__ __forceinline__ float sqrt_fast(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
+__device__ __forceinline__ float sqrt_fast(float x) { return x > 0.0f ? x * fast_rsqrt(x) : 0.0f; }
 
 // orthonormal pair perpendicular to unit n (Duff et al., JCGT 6(1), 2017)
 __device__ __forceinline__ void onb(float nx, float ny, float nz, float3& b1, float3& b2)
 {
     float sgn = copysignf(1.0f, nz);
-    float a = __fdividef(-1.0f, sgn + nz);
+    float a = fast_div(-1.0f, sgn + nz);
     float b = nx * ny * a;
     b1 = make_float3(1.0f + sgn * nx * nx * a, sgn * b, -sgn * nx);
     b2 = make_float3(b, sgn + ny * ny * a, -ny);
@@ -446,9 +477,9 @@ __device__ void launch_state(const Params& P, const float4* rt_tab, uint32_t ins
 __device__ __forceinline__ float hit_box(const Params& P, float px, float py, float pz, float dx, float dy, float dz)
 {
     // approximate quotients (2 ulp): a hit distance needs no correctly rounded division
-    const float qx = __fdividef((dx > 0.0f ? P.box_hi[0] : P.box_lo[0]) - px, dx);
-    const float qy = __fdividef((dy > 0.0f ? P.box_hi[1] : P.box_lo[1]) - py, dy);
-    const float qz = __fdividef((dz > 0.0f ? P.box_hi[2] : P.box_lo[2]) - pz, dz);
+    const float qx = fast_div((dx > 0.0f ? P.box_hi[0] : P.box_lo[0]) - px, dx);
+    const float qy = fast_div((dy > 0.0f ? P.box_hi[1] : P.box_lo[1]) - py, dy);
+    const float qz = fast_div((dz > 0.0f ? P.box_hi[2] : P.box_lo[2]) - pz, dz);
     const float tx = fabsf(dx) > 0.0f ? qx : CUDART_INF_F;
     const float ty = fabsf(dy) > 0.0f ? qy : CUDART_INF_F;
     const float tz = fabsf(dz) > 0.0f ? qz : CUDART_INF_F;
@@ -476,7 +507,7 @@ __device__ __forceinline__ float hit_prim(const DevPrim& Q, const Params& P, flo
         if (A > 0.0f && disc >= 0.0f) {
             const float sq = sqrtf(disc);
             const float q = -0.5f * (B + copysignf(sq, B));
-            float r1 = __fdividef(q, A), r2 = q != 0.0f ? __fdividef(Cc, q) : r1;
+            float r1 = fast_div(q, A), r2 = q != 0.0f ? fast_div(Cc, q) : r1;
             const float tlo = fminf(r1, r2), thi = fmaxf(r1, r2);
             if (tlo > 0.0f && fabsf(fmaf(tlo, da, wa)) <= Q.p1) t = tlo;
             else if (thi > 0.0f && fabsf(fmaf(thi, da, wa)) <= Q.p1) t = thi;
@@ -485,7 +516,7 @@ __device__ __forceinline__ float hit_prim(const DevPrim& Q, const Params& P, flo
         const float den = dx * Q.nx + dy * Q.ny + dz * Q.nz;
         if (den != 0.0f) {
             const float num = (Q.cx - px) * Q.nx + (Q.cy - py) * Q.ny + (Q.cz - pz) * Q.nz;
-            const float tt = __fdividef(num, den);
+            const float tt = fast_div(num, den);
             if (tt > 0.0f) {
                 const float qx = fmaf(tt, dx, px) - Q.cx, qy = fmaf(tt, dy, py) - Q.cy, qz = fmaf(tt, dz, pz) - Q.cz;
                 const float a1 = qx * Q.ux + qy * Q.uy + qz * Q.uz;
@@ -572,7 +603,7 @@ __device__ __forceinline__ void flight_length(const Lane& S, const Params& P, co
     inv_lam = P.gas_thermal ? S.ng14 * Kv / S.speed : S.ng14 * Kv;
     // diffusion shortcut: exponential steps of mean lambda_D, 1/lambda_D = n sigma_D
     if (kMode == kModeWalk && S.diff) inv_lam = S.ng14 * pr.sigma_D;
-    ell = S.ng14 > 0.0f ? __fdividef(nl, inv_lam) : CUDART_INF_F;
+    ell = S.ng14 > 0.0f ? fast_div(nl, inv_lam) : CUDART_INF_F;
     if (kMode == kModeScoreT) Gv = wtab_G(T, pr, i, t);
 }
 
@@ -684,7 +715,7 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
         const float L = fminf(ell, tb);
         // 1 + floor(L / (4 h)) pieces (floor as in table_cell; at most kCellMaxPieces, also for NaN)
         float pieces = fminf(__fadd_rd(L * P.cell_inv_seg, 8388608.0f) - 8388607.0f, (float)kCellMaxPieces);
-        const float R = 0.5f * __fdividef(L, pieces);
+        const float R = 0.5f * fast_div(L, pieces);
         // the smallest level: max(0, ceil(log2(R / r))) from the exponent bits
         const int k = max(0, (int)((__float_as_uint(R * P.cell_inv_r) + 0x7fffffu) >> 23) - 127);
         // grid coordinates of the start; step of the centres
@@ -848,7 +879,7 @@ __device__ __forceinline__ Attempt attempt_draw(const Params& P, uint32_t pid, u
     const uint32_t lowb = ((wn.x & 0xffu) << 24) | ((wn.y & 0xffu) << 16) | ((wn.z & 0xffu) << 8);
     d.u = rn(lowb);
     const float r32 = sumsq_xyz(d.z1, d.z2, d.z3);
-    const float ir3 = r32 > 0.0f ? rsqrtf(r32) : 0.0f;
+    const float ir3 = r32 > 0.0f ? fast_rsqrt(r32) : 0.0f;
     d.r3 = r32 * ir3;
     d.rho_w = sqrt_fast(r32 + z4 * z4);
     d.sc_w = P.s_gas * (d.rho_w * ir3);
@@ -1046,7 +1077,7 @@ __device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, floa
     const float gx = __fsub_rn(vx, Vx), gy = __fsub_rn(vy, Vy), gz = __fsub_rn(vz, Vz);
     // (the temperature-score instance rounds this sum in the other order, as its results always were)
     const float g2 = kMode == kModeScoreT ? sumsq_yxz(gx, gy, gz) : sumsq_xyz(gx, gy, gz);
-    const float ig = rsqrtf(g2);
+    const float ig = kUsual ? fast_rsqrt(g2) : rsqrtf(g2);
     const float g = g2 * ig;
     const float hx = gx * ig, hy = gy * ig, hz = gz * ig;
     const float eps = pr.kappa * g2;
@@ -1069,7 +1100,7 @@ __device__ __forceinline__ bool scatter(float& speed, float& dx, float& dy, floa
     const float nvz = fmaf(pr.m2M, gpz, dot2(pr.m1M, vz, pr.m2M, Vz));
     if (kUsual) {
         const float sp2 = sumsq_yxz(nvx, nvy, nvz);
-        const float is = rsqrtf(sp2);
+        const float is = fast_rsqrt(sp2);
         speed = sp2 * is;
         dx = nvx * is;
         dy = nvy * is;
