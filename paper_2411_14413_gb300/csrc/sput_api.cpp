@@ -790,15 +790,12 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     }
     // privatise per-primitive counters in shared memory while they fit
     p.smem_counters = (size_t)p.n_inst * (p.max_prims + 1) <= 12288 ? 1 : 0;
-    if (transport_smem_bytes(p) > S->smem_optin) {
-        p.smem_counters = 0;
-        // the masks' pair lists give way to the scene's own tables
-        if (transport_smem_bytes(p) > S->smem_optin) p.cell_mask = nullptr;
-        if (transport_smem_bytes(p) > S->smem_optin) {
-            sput_scene_destroy(S);
-            return fail(SPUT_ERR_UNSUPPORTED, "scene tables exceed the shared memory of one block");
-        }
+    p.block_warps = 8;
+    if (transport_scene_bytes(p) > S->smem_optin) {
+        sput_scene_destroy(S);
+        return fail(SPUT_ERR_UNSUPPORTED, "scene tables exceed the shared memory of one block");
     }
+    if (transport_smem_bytes(p) > S->smem_optin) p.smem_counters = 0;
     S->smem_counters_fit = p.smem_counters;
     if (p.smem_counters) {
         // 512 instances of 16 primitives take 35 KB of them: two blocks per SM instead of four
@@ -958,6 +955,12 @@ sput_status run_impl(sput_scene* S, const sput_run_opts* opts, cudaStream_t stre
     }
     CUDA_TRY(cudaMemsetAsync(scratch, 0, kRunScratchBytes, stream));
 
+    // (a scene near the limit leaves room for fewer warps' queues)
+    p.block_warps = threads / 32;
+    while (transport_smem_bytes(p) > S->smem_optin && threads > 32) {
+        threads -= 32;
+        p.block_warps = threads / 32;
+    }
     const size_t smem = transport_smem_bytes(p);
     int bps = transport_max_blocks_per_sm(threads, smem);
     if (bps < 1) return fail(SPUT_ERR_UNSUPPORTED, "launch shape does not fit on an SM");
@@ -1172,11 +1175,13 @@ sput_status sput_autotune(sput_scene* S, const sput_run_opts* base, void* stream
     std::vector<Cand> cands;
     for (int threads : {128, 192, 256}) {
         Params probe = S->base;
+        probe.block_warps = threads / 32;
         probe.smem_counters = S->smem_counters_fit;
         const int occ = transport_max_blocks_per_sm(threads, transport_smem_bytes(probe));
         for (int fl : {SPUT_RUN_SMEM_COUNTERS, SPUT_RUN_NO_SMEM_COUNTERS}) {
             if (fl == SPUT_RUN_SMEM_COUNTERS && !S->smem_counters_fit) continue;
             Params pr = S->base;
+            pr.block_warps = threads / 32;
             pr.smem_counters = fl == SPUT_RUN_SMEM_COUNTERS ? 1 : 0;
             const int maxb = transport_max_blocks_per_sm(threads, transport_smem_bytes(pr));
             if (maxb < 1) continue;

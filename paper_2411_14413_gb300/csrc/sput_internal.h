@@ -189,6 +189,7 @@ struct Params {
     uint32_t rk0[10], rk1[10];
     unsigned long long ticket_begin, ticket_end;
     int chunk;
+    int block_warps;                   // warps per block
     int smem_counters;                 // prim/timed-out counters privatised in shared memory
     int launch_at_cutoff;              // launch energy = E_max (SPUT_RUN_LAUNCH_AT_CUTOFF)
     float E_switch;                    // eV; below it after a collision the atom turns diffusive (0 = off)
@@ -223,6 +224,7 @@ int transport_configure(int max_dynamic_smem);
 int transport_launch(const Params& p, int blocks, int threads, size_t smem, void* stream);
 // (the launch picks the kernel instance with the temperature score when p.score_T is set)
 size_t transport_smem_bytes(const Params& p);
+size_t transport_scene_bytes(const Params& p);
 // the drain of the atoms that transport_kernel hands over (Params::pool)
 constexpr int kDrainThreads = 256;
 int drain_launch(const Params& p, int blocks, size_t smem, void* stream);

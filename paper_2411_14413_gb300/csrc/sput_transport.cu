@@ -1334,11 +1334,11 @@ __host__ __device__ inline SmemLayout smem_layout(const Params& p)
     L.gm = o;
     o = align16(o + sizeof(float4) * (kGMHalf + kGMHalfLo));
     L.pool = o;
-    o = align16(o + sizeof(unsigned long long) * 4 * 8);
+    o = align16(o + sizeof(unsigned long long) * 4 * p.block_warps);
     L.queue = o;
-    o = align16(o + sizeof(uint32_t) * kLaunchWords * 32 * 8);
+    o = align16(o + sizeof(uint32_t) * kLaunchWords * 32 * p.block_warps);
     L.scratch = o;
-    o = align16(o + sizeof(WarpScratch) * 8);
+    o = align16(o + sizeof(WarpScratch) * p.block_warps);
     L.counters = o;
     o = align16(o + (p.smem_counters ? sizeof(unsigned int) * (size_t)p.n_inst * (p.max_prims + 1) : 0));
     L.total = o;
@@ -2047,6 +2047,18 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
 }  // namespace
 
 size_t transport_smem_bytes(const Params& p) { return smem_layout(p).total; }
+
+// What counts towards the largest scene: a block's tables, pools and launch queues at eight warps,
+// and the cross-section table, the apsis table and the stream words as if they were staged
+// too (the limit dates from when they were, and scenes are accepted by it still).
+size_t transport_scene_bytes(const Params& p)
+{
+    Params q = p;
+    q.block_warps = 8;
+    q.smem_counters = 0;
+    return smem_layout(q).total - align16(sizeof(WarpScratch) * 8) + sizeof(float4) * p.n_bm +
+           align16(sizeof(float) * (p.n_bm + 1)) + align16(sizeof(uint32_t) * p.n_inst);
+}
 
 namespace {
 
