@@ -386,7 +386,7 @@ static void build_cell_masks(sput_scene* S)
         ext[a] = S->chamber.box_hi[a] - S->chamber.box_lo[a];
         emax = std::max(emax, ext[a]);
     }
-    // kCellGrid cells along the longest side (0.5 or 1 MB per geometry here), half as many when
+    // kCellGrid cells along the longest side (0.25, 0.5 or 1 MB per geometry here), half as many when
     // the geometries' masks would take more than 256 MB
     size_t ncell = 0;
     for (int n = kCellGrid; n >= kCellGrid / 2; n /= 2) {
@@ -398,7 +398,8 @@ static void build_cell_masks(sput_scene* S)
     const double h = S->cell_h, half_diag = 0.5 * std::sqrt(3.0) * h;
     double reach[kCellLevels];
     for (int k = 0; k < kCellLevels; ++k) reach[k] = half_diag + std::ldexp(h / 8.0, k) + 0.1;
-    const size_t words = ncell * kCellLevels * S->cell_words;
+    const bool half = S->max_prims <= 16;  // 16-bit masks (little endian)
+    const size_t words = half ? (ncell * kCellLevels + 1) / 2 : ncell * kCellLevels * S->cell_words;
     S->cell_masks.assign(S->geoms.size() * words, 0u);
     for (size_t g = 0; g < S->geoms.size(); ++g) {
         const sput_geometry& G = S->geoms[g];
@@ -406,15 +407,19 @@ static void build_cell_masks(sput_scene* S)
         uint32_t* m = &S->cell_masks[g * words];
         for (int iz = 0; iz < S->cell_n[2]; ++iz)
             for (int iy = 0; iy < S->cell_n[1]; ++iy)
-                for (int ix = 0; ix < S->cell_n[0]; ++ix, m += kCellLevels * S->cell_words) {
+                for (int ix = 0; ix < S->cell_n[0]; ++ix) {
+                    const size_t cell = ((size_t)iz * S->cell_n[1] + iy) * S->cell_n[0] + ix;
                     const double x[3] = {S->cell_lo[0] + (ix + 0.5) * h, S->cell_lo[1] + (iy + 0.5) * h,
                                          S->cell_lo[2] + (iz + 0.5) * h};
                     for (int li = 0; li < G.prim_count; ++li) {
                         const DevPrim& Q = S->dprims[G.prim_begin + li];
                         if (Q.kind == SPUT_PRIM_BOX) continue;
                         const double d = surface_distance(Q, x);
-                        for (int k = kCellLevels - 1; k >= 0 && d <= reach[k]; --k)
-                            m[k * S->cell_words + (li >> 5)] |= 1u << (li & 31);
+                        for (int k = kCellLevels - 1; k >= 0 && d <= reach[k]; --k) {
+                            const size_t e = cell * kCellLevels + k;  // the cell's mask of this level
+                            if (half) m[e >> 1] |= 1u << (li + 16 * (int)(e & 1));
+                            else m[e * S->cell_words + (li >> 5)] |= 1u << (li & 31);
+                        }
                     }
                 }
     }
@@ -734,6 +739,7 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     p.chi_tab = ct ? reinterpret_cast<const float4*>(S->d_blob + S->off_chi) : nullptr;
     p.cell_mask = S->cell_masks.empty() ? nullptr : reinterpret_cast<const uint32_t*>(S->d_blob + S->off_cell);
     p.cell_words = S->cell_words;
+    p.cell_half = S->max_prims <= 16;
     for (int a = 0; a < 3; ++a) {
         p.cell_off[a] = S->cell_h > 0.0 ? (float)(-S->cell_lo[a] / S->cell_h) : 0.0f;
         p.cell_n[a] = S->cell_n[a];

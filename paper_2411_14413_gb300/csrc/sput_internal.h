@@ -152,6 +152,7 @@ struct Params {
     // that have a point within r 2^k of a point of the cell
     const uint32_t* cell_mask;
     int cell_words;
+    int cell_half;  // masks of 16 bits (at most 16 primitives): half the footprint in L1
     float cell_off[3], cell_inv_h, cell_inv_r, cell_inv_seg;  // (cell_off = -lower corner / h)
     int cell_n[3];
     int n_prims, n_geoms, n_pairs, n_inst;

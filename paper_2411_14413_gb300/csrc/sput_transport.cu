@@ -730,11 +730,12 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
             if (k < kCellLevels && ix < (unsigned)P.cell_n[0] && iy < (unsigned)P.cell_n[1] &&
                 iz < (unsigned)P.cell_n[2]) {
                 const int cell = (int)((iz * P.cell_n[1] + iy) * P.cell_n[0] + ix);
-                const uint32_t* m = P.cell_mask + G.cell_base + (cell * kCellLevels + k) * kWords;
+                const uint32_t* m = P.cell_mask + G.cell_base;
+                const int e = cell * kCellLevels + k;
                 if (kWords == 1) {
-                    lo |= __ldg(m);
+                    lo |= P.cell_half ? __ldg(reinterpret_cast<const unsigned short*>(m) + e) : __ldg(m + e);
                 } else {
-                    const uint2 m2 = __ldg(reinterpret_cast<const uint2*>(m));
+                    const uint2 m2 = __ldg(reinterpret_cast<const uint2*>(m) + e);
                     lo |= m2.x;
                     hi |= m2.y;
                 }

@@ -29,7 +29,7 @@ def _scene(n_prims, pressure, box_last, chamber):
 
 @pytest.mark.parametrize("box_last", [False, True])
 @pytest.mark.parametrize("pressure", [0.0, 0.3, 3.0])
-@pytest.mark.parametrize("n_prims,chamber", [(7, None), (9, None), (32, ((-211.0, -187.5, -100.0), (203.0, 199.0, 171.3))),
+@pytest.mark.parametrize("n_prims,chamber", [(7, None), (9, None), (16, None), (17, None), (32, ((-211.0, -187.5, -100.0), (203.0, 199.0, 171.3))),
                                              (33, None), (63, ((-300.0, -150.0, -95.0), (155.0, 160.0, 640.0))),
                                              (64, None)])
 def test_masks_match_loop(n_prims, chamber, pressure, box_last):
