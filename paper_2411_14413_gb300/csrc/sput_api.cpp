@@ -331,11 +331,11 @@ static sput_status pack_instances(sput_scene* S)
 // geometry's primitives by a mask lookup per piece of a flight and a round of (lane,
 // primitive) pairs, so it needs several primitives and flights that are short against the
 // chamber (edge / lambda, primitives).  Measured on a GB300, loop -> masks in ms:
-//   16 primitives, 4e6 atoms:   0 Pa 0.28 -> 0.34, 0.05 Pa 0.77 -> 0.82, 0.1 Pa (edge/lambda 6)
-//                               1.32 -> 1.31, 0.2 Pa 2.44 -> 2.18, 0.5 Pa 9.0 -> 7.8
-//   64 primitives, 4e6 atoms:   0 Pa 0.73 -> 0.78, 0.05 Pa (edge/lambda 3) 1.51 -> 1.13,
-//                               0.5 Pa 12.9 -> 5.9
-//   7 primitives, 4e6 atoms:    0.2 Pa 2.25 -> 2.43, 0.5 Pa 10.6 -> 10.9, 1 Pa 44.4 -> 44.4
+//   16 primitives, 4e6 atoms:   0 Pa 0.28 -> 0.31, 0.05 Pa 0.80 -> 0.84, 0.1 Pa (edge/lambda 6)
+//                               1.17 -> 1.16, 0.2 Pa 2.03 -> 1.84
+//   64 primitives, 4e6 atoms:   0 Pa 0.73 -> 0.75, 0.05 Pa (edge/lambda 3) 1.52 -> 1.19
+//   7 primitives, 4e6 atoms:    0.2 Pa 1.78 -> 2.01, 0.5 Pa 8.49 -> 8.63; 1.2e6 atoms: 1 Pa
+//                               14.05 -> 13.97, 2 Pa 48.9 -> 48.1
 static bool cell_masks_pay(const sput_scene* S)
 {
     double edge = 0.0;

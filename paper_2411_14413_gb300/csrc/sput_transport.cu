@@ -4,9 +4,10 @@
 // lanes from a warp-private pool of tickets that it takes in chunks from one
 // global counter, so every lane runs exactly one free flight per loop
 // iteration (Sec. "The SIMTRA model": launch, free flight, surface test,
-// binary collision, repeated until the atom lands).  The geometry and the small
-// interaction tables are staged in shared memory; the rate tables, the
-// deflection table and the cell masks are read through L1/L2.  The scattering
+// binary collision, repeated until the atom lands).  A run's last atoms, and
+// small runs, go to drain_kernel, which carries one atom with several lanes.
+// The geometry is staged in shared memory; the rate, cross-section and
+// deflection tables and the cell masks are read through L1/L2.  The scattering
 // angle comes from a bicubic table of ln tan(chi/2) built from the classical
 // deflection integral, and from Gauss-Mehler quadrature in FP32 outside the
 // table's range.  Counts are integer atomics (bit-exact, order independent);
@@ -696,9 +697,9 @@ __device__ __forceinline__ void nearest_hit_loop(const Lane& S, const Params& P,
 // The transport is bound by instruction issue, and the loop took 43 % (16 primitives, 0.5 Pa)
 // to 67 % (64 primitives, 3 Pa) of the kernel: a warp ran 9.2 of 16 primitives' tests per
 // step although 0.12 per atom cross the primitive at all.  Masks of the midpoint leave 13
-// pairs per warp and step (0.5 Pa), so one round does.  Measured loop -> masks (GB300):
-// quaternary 4e7 atoms 67.2 -> 58.8 ms, 64 primitives at 3 Pa 1e6 atoms 118 -> 59 ms, with the
-// diffusion shortcut 4e6 atoms 61.3 -> 24.7 ms.
+// pairs per warp and step (0.5 Pa), so one round does.  Measured loop -> masks (GB300, before
+// what followed): quaternary 4e7 atoms 67.2 -> 58.8 ms, 64 primitives at 3 Pa 1e6 atoms
+// 118 -> 59 ms, with the diffusion shortcut 4e6 atoms 61.3 -> 24.7 ms.
 template <int kWords>
 __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, const Params& P, const TableView& T,
                                                   const DevPrim* prims, uint2* list, float ell, float& tb, int& hb)
@@ -1358,9 +1359,11 @@ __device__ __forceinline__ void copy16(void* dst, const void* src, size_t bytes)
 
 // Persistent warp pool.  Four blocks of 256 threads per SM (32 warps, 64 registers a
 // thread): the issue-bound loop gains more from the extra warps than it loses to the
-// few spills at 64 registers; the lane state is kept small for it (a geometry index
-// instead of the geometry's fields, the ticket recomputed from (instance, id), the
-// warp's ticket pool in shared memory).
+// few spills at 64 registers (five blocks at 48 registers: quaternary 48.7 against 46.8 ms); the
+// lane state is kept small for it (the instance's conditions read at each flight, the ticket
+// recomputed from (instance, id), the warp's ticket pool in shared memory).  Bound by
+// instruction issue: 50 warp instructions per collision on the quaternary scene, issue slots
+// 80 % busy.
 template <int kMode, int kMasks>
 __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 {
@@ -1568,12 +1571,12 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 // A warp starts with as many lanes per atom as the pool's size allows, and once the pool is
 // empty the lanes of finished atoms join the others'.  Every number is computed as in the
 // single-lane step, so the results are bit-identical.
-// Bound by the latency of the chain (320 instructions and 1650 cycles per step, 0.82 us, of which
-// 370 wait for the deflection table in L1 or L2).  Measured on a GB300 without and with the
-// drain: single Ni 3e3 atoms 1.8 -> 0.53 ms, 1e5 2.4 -> 1.26 ms, quaternary 4e5 3.0 -> 1.8 ms,
-// 64 primitives at 3 Pa 1e5 atoms 31 -> 14.5 ms, 1e6 59 -> 47 ms.  Runs of 3e4 single-Ni atoms
-// take 0.74 ms when they go to it at once, 0.95 ms when only the last atoms of each warp do;
-// from 1.5e5 atoms on (one per lane of the GPU) the two meet.
+// Bound by the latency of the chain, 1200 cycles (0.6 us) per step, a third of it waiting for the
+// deflection table in L1 or L2.  Measured on a GB300 without and with the drain when it came:
+// single Ni 3e3 atoms 1.8 -> 0.53 ms (now 0.34), 1e5 2.4 -> 1.26 ms (0.90), quaternary 4e5
+// 3.0 -> 1.8 ms (1.4), 64 primitives at 3 Pa 1e6 atoms 59 -> 47 ms (38).  Runs of 3e4 single-Ni
+// atoms took 0.74 ms when they went to it at once, 0.95 ms when only the last atoms of each
+// warp did; from 1.5e5 atoms on (one per lane of the GPU) the two met.
 constexpr int kDrawn = 4;
 constexpr int kMinGroupLog2 = 3;
 
