@@ -85,15 +85,16 @@ OPS_PER_COLLISION = 78
 OPS_PER_PARTICLE = 2 * PHILOX_BLOCK_OPS + 80
 WORK_MODEL = {"philox_block": PHILOX_BLOCK_OPS, "flight": OPS_PER_FLIGHT, "prim_test": OPS_PER_PRIM_TEST,
               "partner_attempt": OPS_PER_ATTEMPT, "collision": OPS_PER_COLLISION, "particle": OPS_PER_PARTICLE}
-# Executed active-lane instructions per collision of the current transport
-# kernel (ncu smsp__thread_inst_executed.sum / collisions of one launch, small
+# Executed active-lane instructions per collision of the current transport and
+# drain kernels (ncu smsp__thread_inst_executed.sum / collisions of one run, small
 # case of the workload); the issue share is reported beside the algorithmic
 # fraction.  None = no capture of the current build.
-EXEC_LANE_INSTR_PER_COLLISION = {"quaternary": 1814.0, "large": 2667.0}
-# DRAM bytes (read + write) of one launch of the quaternary workload, from the
-# one-pass capture of the current kernel (mean of 5 launches: 4.10 MB read,
-# 0.23 MB written); None whenever the kernel changed after the capture.
-TRAFFIC_PER_LAUNCH = 4.33e6
+EXEC_LANE_INSTR_PER_COLLISION = {"quaternary": 1316.0, "large": 1312.0}
+# DRAM bytes (read + write) of one run of the quaternary workload, from the
+# one-pass capture of the current kernels (transport 4.15 MB read and 0.23 MB
+# written, drain 4.88 MB read, mean of 3 runs); None whenever a kernel changed
+# after the capture.
+TRAFFIC_PER_LAUNCH = 9.26e6
 
 
 def log(*a):
@@ -438,7 +439,7 @@ def run_ours(args, rank, world, local_rank):
         "peaks": peaks,
         "e2e": {"value": (e2e_coll_all / e2e_t_all) if e2e_t_all > 0 else None, "unit": UNIT,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        "gpu_launches": args.steps,
+        "gpu_launches": 2 * args.steps,  # the transport and the drain of its last atoms
         "autotune": None if tune is None else {"block_threads": tune.block_threads, "blocks_per_sm": tune.blocks_per_sm,
                                                "ticket_chunk": tune.ticket_chunk, "flags": tune.flags,
                                                "candidates": tune.n_candidates},

@@ -367,8 +367,8 @@ static double surface_distance(const DevPrim& Q, const double* x)
 // Cell masks of the surface test (nearest_hit_masks).  A uniform grid of cubic cells
 // covers the chamber box.  For every geometry, cell c and level k, a mask holds the local
 // primitives whose surface lies within r 2^k of a point of c: distance to the cell's centre
-// at most half its diagonal + r 2^k, grown by 0.1 mm, far above the FP32 rounding of
-// positions, midpoints and hit distances (1e-4 mm at these sizes).  Chamber boxes are left
+// at most half its diagonal + r 2^k, grown by 0.1 mm + h/1000 (in a chamber of any size far
+// above the FP32 rounding of positions, midpoints and hit distances: 1e-4 mm in one of 400 mm).  Chamber boxes are left
 // out: the flight tests the walls by themselves.  A geometry of more than 64 primitives, or
 // without chamber walls, leaves the masks out (every flight tests every primitive).
 static void build_cell_masks(sput_scene* S)
@@ -397,7 +397,7 @@ static void build_cell_masks(sput_scene* S)
     }
     const double h = S->cell_h, half_diag = 0.5 * std::sqrt(3.0) * h;
     double reach[kCellLevels];
-    for (int k = 0; k < kCellLevels; ++k) reach[k] = half_diag + std::ldexp(h / 8.0, k) + 0.1;
+    for (int k = 0; k < kCellLevels; ++k) reach[k] = half_diag + std::ldexp(h / 8.0, k) + 0.1 + 1e-3 * h;
     const bool half = S->max_prims <= 16;  // 16-bit masks (little endian)
     const size_t words = half ? (ncell * kCellLevels + 1) / 2 : ncell * kCellLevels * S->cell_words;
     S->cell_masks.assign(S->geoms.size() * words, 0u);
