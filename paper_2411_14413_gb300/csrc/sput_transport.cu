@@ -1730,6 +1730,9 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
     DevPair* s_pairs = reinterpret_cast<DevPair*>(smem + L.pairs);
     float4* s_gm = reinterpret_cast<float4*>(smem + L.gm);
     DrainWarp& W = reinterpret_cast<DrainWarp*>(smem + L.warps)[threadIdx.x >> 5];
+    // the lanes of a group without an atom go through the collisions with the others: what they read
+    // has to be a table column from the start (shared memory begins with anything)
+    W.hit[threadIdx.x & 31] = Impact{1.0f, 0, 0.0f, 0.0f, 0.0f};
     copy16(s_prims, P.prims, sizeof(DevPrim) * P.n_prims);
     copy16(s_geoms, P.geoms, sizeof(DevGeom) * P.n_geoms);
     copy16(s_pairs, P.pairs, sizeof(DevPair) * P.n_pairs);

@@ -98,3 +98,36 @@ def test_flags_and_range():
     table = copy.deepcopy(workloads.scene_single_ni_table(n=3000, pressure=1.0))
     got, _ = _both(table)
     assert int(np.asarray(got["timed_out"].sum().cpu())) == 0
+
+
+@pytest.mark.parametrize("n", [1, 5, 33, 5491])
+@pytest.mark.parametrize("physics", [{}, {"gas_motion": "stationary", "max_collisions": 100}])
+def test_idle_groups_stay_in_bounds(n, physics):
+    """Groups without an atom go through a warp's collisions too.  The bounds-checked library must
+    report no index outside its table for them, whatever the shared memory held before: here what
+    a transport with large tables left in it."""
+    import ctypes as C
+
+    import torch
+
+    import paper_2411_14413_gb300 as pkg
+    from paper_2411_14413_gb300 import _native as N
+    from paper_2411_14413_gb300 import api
+
+    lib = N.load(path=N.CHECKED_LIB_PATH)
+    dirty = pkg.Transport(workloads.scene_tilt_pressure_sweep(n_range=(300, 1000)))
+    sc = workloads.scene_large_shielded(n=n, pressure=0.8, nx=31, ny=17, physics=physics)
+    d, keep = api.scene_desc(sc)
+    h = C.c_void_p()
+    assert lib.sput_scene_create(C.byref(d), 0, C.byref(h)) == 0
+    counts = torch.zeros((1, 17, 31), dtype=torch.int64, device="cuda")
+    tal = N.sput_tallies()
+    tal.counts = counts.data_ptr()
+    for seed in range(3):
+        dirty.run(seed=seed, want_stats=False, flags=N.SPUT_RUN_SMEM_COUNTERS)
+        st = N.sput_run_stats()
+        rc = lib.sput_run(h, C.byref(api.run_opts(seed=seed)), C.c_void_p(torch.cuda.current_stream().cuda_stream),
+                          C.byref(tal), C.byref(st))
+        assert rc == 0 and st.device_status == 0 and st.particles == n
+    lib.sput_scene_destroy(h)
+    dirty.close()
