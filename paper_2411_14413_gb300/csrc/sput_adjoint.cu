@@ -51,14 +51,21 @@ __device__ double warp_sum(double x)
     return x;
 }
 
+// Another block's shared memory may be touched only once that block has started: every thread
+// arrives at the cluster's barrier when its kernel starts, and waits there for the others just
+// before the stores to the first block, behind the kernel's own loads.
+__device__ void cluster_started() { cg::cluster_group::barrier_arrive(); }
+__device__ void cluster_wait() { cg::cluster_group::barrier_wait(); }
+
 // Sum of x over the threads of the cluster, in thread 0 of its first block; part: shared memory of
-// kCluster + 32 doubles.  The last step is a cluster barrier.
+// kCluster + 32 doubles; the kernel called cluster_started() first.  The last step is a cluster barrier: no block ends before the stores to it.
 __device__ double cluster_sum(double x, double* part)
 {
     cg::cluster_group cl = cg::this_cluster();
     x = warp_sum(x);
     if ((threadIdx.x & 31) == 0) part[kCluster + (threadIdx.x >> 5)] = x;
     __syncthreads();
+    cluster_wait();
     if (threadIdx.x < 32) {
         double t = threadIdx.x < (blockDim.x >> 5) ? part[kCluster + threadIdx.x] : 0.0;
         t = warp_sum(t);
@@ -77,6 +84,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kReduceThread
     lr_backward_kernel(const double* g, const double* score, double* grad, long long n_cells)
 {
     __shared__ double part[kCluster + 32];
+    cluster_started();
     const int inst = blockIdx.x / kCluster;
     const long long base = (long long)inst * n_cells;
     double s = 0.0;
@@ -110,6 +118,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kReduceThread
                          double* grad, long long n_cells, double* grad_power, VoltParams vp)
 {
     __shared__ double part[kCluster + 32];
+    cluster_started();
     const int i = blockIdx.x / kCluster;
     const long long base = (long long)i * n_cells;
     double s = 0.0;
@@ -181,6 +190,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1)
     __shared__ double W[kMaxCath];
     __shared__ bool on[kMaxCath];  // atoms at the reference point
     __shared__ double part[kCluster][kMaxCath];
+    cluster_started();
     if (threadIdx.x < cp.n_cath) {
         W[threadIdx.x] = arrival_weight(N, cp, threadIdx.x);
         on[threadIdx.x] = N[(size_t)threadIdx.x * cp.n_points + cp.ref] > 0.0;
@@ -209,6 +219,8 @@ __global__ void __cluster_dims__(kCluster, 1, 1)
                 S[j] += ga * a[j];
             }
     }
+    __syncwarp();
+    cluster_wait();
     double* first = cl.map_shared_rank(&part[0][0], 0);
 #pragma unroll
     for (int j = 0; j < kMaxCath; ++j)
