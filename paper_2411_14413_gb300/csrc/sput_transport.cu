@@ -808,8 +808,8 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
             }
             t0 += __popc(m);
         }
+        __syncwarp();  // (what writes the scratch next does so after these reads)
         if (total < 32) return;
-        __syncwarp();
     }
 }
 
@@ -997,6 +997,7 @@ __device__ void partner_sample_warp(bool need, const Params& P, const TableView&
             acc = attempt_accept(d, weighted, ut, Bm, o_A, o_B, hg) || a == A - 1;
         }
         const unsigned accm = __ballot_sync(kFull, acc);
+        if (!own) __syncwarp();  // (a vote does not order memory: the scratch is written again after these reads)
         if (own) {
             if (acc) {
                 Vx = cx;

@@ -37,3 +37,17 @@ def test_clusters_have_started_before_remote_stores():
         b = bodies[name]
         head = b[b.index("{"):b.index("cluster_started()")] if "cluster_started()" in b else None
         assert head is not None and not re.search(r"\b(if|for|while|return)\b", head), name
+
+
+def test_warp_scratch_is_ordered_between_its_uses():
+    """A warp's scratch in shared memory serves the surface test and the partner sampling in turn.
+    Votes and shuffles do not order memory: after the last reads of each use there is a __syncwarp."""
+    bodies = dict(_bodies(_source("sput_transport.cu")))
+    surface = bodies["nearest_hit_masks"]
+    reads = surface.rindex("list[at]")
+    leave = surface.index("if (total < 32) return;")
+    assert reads < surface.index("__syncwarp()", reads) < leave
+    partner = bodies["partner_sample_warp"]
+    reads = partner.rindex("ws->ask")
+    again = partner.index("if (own)", reads)
+    assert "if (!own) __syncwarp();" in partner[reads:again]
