@@ -263,7 +263,7 @@ typedef struct sput_run_opts {
 #define SPUT_RUN_NO_CELL_MASKS 16   /* surface test over every primitive, by a counted loop */
 #define SPUT_RUN_CELL_MASKS 32      /* surface test restricted by the cell masks: a flight tests the primitives that
                                        have a point near enough to its midpoint's cell (geometries of at most 64
-                                       primitives with chamber walls).  Default: on when the largest geometry
+                                       primitives, with chamber walls or all inside the chamber box).  Default: on when the largest geometry
                                        has more than 8 primitives and flights are short against the chamber.
                                        Results are identical either way; only the speed differs */
 #define SPUT_RUN_INJECT_NONFINITE 8 /* failure-path test aid: particle 0 of every instance starts with a NaN
@@ -299,8 +299,9 @@ const char* sput_last_error(void);
  * before any CUDA call, e.g. an instance whose Thompson cut-off
  * E_max = k Lambda E_i - U_s is not positive), CUDA, NO_MEMORY, and UNSUPPORTED
  * when the primitives and small tables a block stages do not fit its shared
- * memory (about 2800 primitives).  Geometries of more than 64 primitives run the
- * surface test without cell masks. */
+ * memory (about 2800 primitives).  Geometries of more than 64 primitives, and those without
+ * chamber walls of which one lies outside the chamber box, run the surface test without
+ * cell masks. */
 sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scene** out);
 
 /* Replace the instance table (pressures, ion energies, k, particle counts).

@@ -336,6 +336,8 @@ static sput_status pack_instances(sput_scene* S)
 //   64 primitives, 4e6 atoms:   0 Pa 0.73 -> 0.75, 0.05 Pa (edge/lambda 3) 1.52 -> 1.19
 //   7 primitives, 4e6 atoms:    0.2 Pa 1.78 -> 2.01, 0.5 Pa 8.49 -> 8.63; 1.2e6 atoms: 1 Pa
 //                               14.05 -> 13.97, 2 Pa 48.9 -> 48.1
+//   63 primitives, no walls, 1e6 atoms (at most 2000 collisions): 0.3 Pa 33.4 -> 17.1, 0.5 Pa
+//                               38.5 -> 20.0; 1e5 atoms: 3 Pa 16.4 -> 8.8
 static bool cell_masks_pay(const sput_scene* S)
 {
     double edge = 0.0;
@@ -364,20 +366,39 @@ static double surface_distance(const DevPrim& Q, const double* x)
     return std::sqrt(z * z + dr * dr);
 }
 
+// Whether a geometry's primitives all lie inside the chamber box (to half of the masks' margin).
+static bool inside_chamber(const sput_scene* S, const sput_geometry& G)
+{
+    for (int li = 0; li < G.prim_count; ++li) {
+        const sput_primitive& P = S->prims[G.prim_begin + li];
+        if (P.kind == SPUT_PRIM_BOX) continue;
+        for (int a = 0; a < 3; ++a) {
+            const double r = P.kind == SPUT_PRIM_CYLINDER
+                                 ? P.p0 * std::sqrt(std::max(0.0, 1.0 - P.u[a] * P.u[a])) + P.p1 * std::fabs(P.u[a])
+                             : P.kind == SPUT_PRIM_RECT ? P.p0 * std::fabs(P.u[a]) + P.p1 * std::fabs(P.v[a])
+                                                        : P.p1 * std::hypot(P.u[a], P.v[a]);
+            if (P.center[a] - r < S->chamber.box_lo[a] - 0.05 || P.center[a] + r > S->chamber.box_hi[a] + 0.05) return false;
+        }
+    }
+    return true;
+}
+
 // Cell masks of the surface test (nearest_hit_masks).  A uniform grid of cubic cells
 // covers the chamber box.  For every geometry, cell c and level k, a mask holds the local
 // primitives whose surface lies within r 2^k of a point of c: distance to the cell's centre
 // at most half its diagonal + r 2^k, grown by 0.1 mm + h/1000 (in a chamber of any size far
 // above the FP32 rounding of positions, midpoints and hit distances: 1e-4 mm in one of 400 mm).  Chamber boxes are left
-// out: the flight tests the walls by themselves.  A geometry of more than 64 primitives, or
-// without chamber walls, leaves the masks out (every flight tests every primitive).
+// out: the flight tests the walls by themselves.  Without walls a flight may leave the grid; it
+// then takes the nearest cell's mask, which needs every primitive inside the chamber box.  A
+// geometry of more than 64 primitives, or without walls and with a primitive that sticks out,
+// leaves the masks out (every flight tests every primitive).
 static void build_cell_masks(sput_scene* S)
 {
     S->cell_masks.clear();
     S->cell_h = 0.0;
     S->cell_words = 1;
     for (size_t g = 0; g < S->geoms.size(); ++g) {
-        if (S->geoms[g].prim_count > 64 || S->dgeoms[g].box() < 0) return;
+        if (S->geoms[g].prim_count > 64 || (S->dgeoms[g].box() < 0 && !inside_chamber(S, S->geoms[g]))) return;
         if (S->geoms[g].prim_count > 32) S->cell_words = 2;
     }
     double ext[3], emax = 0.0;

@@ -682,9 +682,15 @@ __device__ __forceinline__ void nearest_hit_loop(const Lane& S, const Params& P,
     }
 }
 
+// grid coordinate x's cell, the nearest one of n when x lies outside (0 for NaN)
+__device__ __forceinline__ unsigned grid_clamp(float x, int n)
+{
+    return (unsigned)fminf(fmaxf(x, 0.0f), (float)(n - 1));
+}
+
 // Nearest hit of every active lane by the cell masks, the whole warp together.
-//   * The chamber walls are tested first, so the flight is a segment of length
-//     L = min(ell, wall) inside the box.
+//   * The chamber walls, if the geometry has them, are tested first, so the flight is a segment
+//     of length L = min(ell, wall) inside the box.
 //   * It is cut into pieces of at most 4 cell edges (most flights are one piece).  All of a
 //     piece lies within R, half its length, of its centre: the mask of the centre's cell at
 //     the smallest level r 2^k >= R holds every primitive it can reach (usually none: most
@@ -710,8 +716,9 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
     if (active) {
         const DevGeom G = T.geoms[S.geom];
         begin = G.begin;
-        const int box = G.box();  // a geometry with masks has one
+        const int box = G.box();
         tb = hit_box(P, S.px, S.py, S.pz, S.dx, S.dy, S.dz);
+        tb = box >= 0 ? tb : CUDART_INF_F;
         hb = tb < CUDART_INF_F ? box : -1;
         const float L = fminf(ell, tb);
         // 1 + floor(L / (4 h)) pieces (floor as in table_cell; at most kCellMaxPieces, also for NaN)
@@ -725,11 +732,21 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
         const float Rh = R * P.cell_inv_h;
         for (float c = Rh; pieces > 0.0f; pieces -= 1.0f, c += 2.0f * Rh) {
             // floors of the coordinates; a negative one wraps to a large unsigned number
-            const unsigned ix = __float_as_uint(__fadd_rd(fmaf(c, S.dx, sx), 8388608.0f)) - 0x4b000000u;
-            const unsigned iy = __float_as_uint(__fadd_rd(fmaf(c, S.dy, sy), 8388608.0f)) - 0x4b000000u;
-            const unsigned iz = __float_as_uint(__fadd_rd(fmaf(c, S.dz, sz), 8388608.0f)) - 0x4b000000u;
-            if (k < kCellLevels && ix < (unsigned)P.cell_n[0] && iy < (unsigned)P.cell_n[1] &&
-                iz < (unsigned)P.cell_n[2]) {
+            unsigned ix = __float_as_uint(__fadd_rd(fmaf(c, S.dx, sx), 8388608.0f)) - 0x4b000000u;
+            unsigned iy = __float_as_uint(__fadd_rd(fmaf(c, S.dy, sy), 8388608.0f)) - 0x4b000000u;
+            unsigned iz = __float_as_uint(__fadd_rd(fmaf(c, S.dz, sz), 8388608.0f)) - 0x4b000000u;
+            bool in = k < kCellLevels && ix < (unsigned)P.cell_n[0] && iy < (unsigned)P.cell_n[1] &&
+                      iz < (unsigned)P.cell_n[2];
+            if (!in) {
+                // A centre outside the grid (without walls, or by rounding at one) takes the cell
+                // nearest to it: the chamber is convex and what the flight may hit lies in it, so
+                // that cell is no farther from any of it than the centre.
+                ix = grid_clamp(fmaf(c, S.dx, sx), P.cell_n[0]);
+                iy = grid_clamp(fmaf(c, S.dy, sy), P.cell_n[1]);
+                iz = grid_clamp(fmaf(c, S.dz, sz), P.cell_n[2]);
+                in = k < kCellLevels;
+            }
+            if (in) {
                 const int cell = (int)((iz * P.cell_n[1] + iy) * P.cell_n[0] + ix);
                 const uint32_t* m = P.cell_mask + G.cell_base;
                 const int e = cell * kCellLevels + k;
@@ -741,10 +758,10 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
                     hi |= m2.y;
                 }
             } else {
-                // a centre outside the grid (FP32 rounding at a wall), or a flight that starts outside
+                // longer than kCellMaxPieces pieces: no walls stop it
                 lo = G.count >= 32 ? ~0u : (1u << G.count) - 1u;
                 if (kWords == 2) hi = G.count >= 64 ? ~0u : G.count > 32 ? (1u << (G.count - 32)) - 1u : 0u;
-                if (box < 32) lo &= ~(1u << box);
+                if (box >= 0 && box < 32) lo &= ~(1u << box);
                 if (kWords == 2 && box >= 32) hi &= ~(1u << (box - 32));
             }
         }
@@ -2098,6 +2115,13 @@ int instance_mode(const Params& p) { return p.score_T ? kModeScoreT : (p.E_switc
 
 }  // namespace
 
+#ifdef SPUT_CHECKED
+// For the tests of the checked library: which surface test the last run enqueued by this thread
+// took (words of its cell masks, 0: the counted loop).
+thread_local int t_mask_words = -1;
+extern "C" int sput_checked_mask_words() { return t_mask_words; }
+#endif
+
 size_t drain_smem_bytes(const Params& p) { return drain_layout(p).total; }
 
 int transport_max_blocks_per_sm(int threads, size_t smem) { return min_blocks_per_sm(kTransport, threads, smem); }
@@ -2118,6 +2142,9 @@ int transport_configure(int max_dynamic_smem)
 
 int transport_launch(const Params& p, int blocks, int threads, size_t smem, void* stream)
 {
+#ifdef SPUT_CHECKED
+    t_mask_words = p.cell_mask ? p.cell_words : 0;
+#endif
     kTransport[instance_mode(p)][p.cell_mask ? p.cell_words : 0]<<<blocks, threads, smem,
                                                                    reinterpret_cast<cudaStream_t>(stream)>>>(p);
     return (int)cudaGetLastError();
