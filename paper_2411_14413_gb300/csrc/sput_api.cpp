@@ -312,10 +312,11 @@ static sput_status pack_instances(sput_scene* S)
         S->prefix[i + 1] = S->prefix[i] + I.n_particles;
     }
     S->n_tickets = S->prefix.back();
-    // mean inverse free path of 1 eV atoms, for the choice of the surface test (cell_masks_pay)
+    // mean inverse free path of 1 eV atoms, for the choice of the surface test (cell_masks_pay); by the
+    // pair itself: a scene whose indices do not fit geom_pair gets here and is refused later
     S->mean_inv_lambda = 0.0;
     for (size_t i = 0; i < S->dinst.size(); ++i) {
-        const DevPair& pr = S->dpairs[S->dinst[i].geom_pair >> 16];
+        const DevPair& pr = S->dpairs[S->dcath[S->dinst[i].cathode].pair];
         const double v = 1.0 / std::sqrt((double)S->dcath[S->dinst[i].cathode].E_per_v2);
         const double x = std::min(std::log(1.0 + v * pr.inv_s) * pr.w_inv_h, (double)pr.n_w);
         const int j = std::min((int)x, pr.n_w - 1);
