@@ -105,7 +105,8 @@ struct sput_scene {
     // cell masks of the surface test (empty: a geometry has more than 64 primitives)
     std::vector<uint32_t> cell_masks;
     int cell_words = 1;
-    double mean_inv_lambda = 0.0;  // 1/mm, of 1 eV atoms, mean over the instances' particles
+    // 1/mm, of 1 eV atoms: mean over the instances' particles, and of the instance with most
+    double mean_inv_lambda = 0.0, max_inv_lambda = 0.0;
     double cell_lo[3] = {0, 0, 0}, cell_h = 0.0;
     int cell_n[3] = {0, 0, 0};
     std::vector<DevCathode> dcath;
@@ -312,9 +313,10 @@ static sput_status pack_instances(sput_scene* S)
         S->prefix[i + 1] = S->prefix[i] + I.n_particles;
     }
     S->n_tickets = S->prefix.back();
-    // mean inverse free path of 1 eV atoms, for the choice of the surface test (cell_masks_pay); by the
-    // pair itself: a scene whose indices do not fit geom_pair gets here and is refused later
-    S->mean_inv_lambda = 0.0;
+    // inverse free path of 1 eV atoms, for the choice of the surface test (cell_masks_pay) and of the atoms
+    // for the drain (hand_over); by the pair itself: a scene whose indices do not fit geom_pair gets
+    // here and is refused later
+    S->mean_inv_lambda = S->max_inv_lambda = 0.0;
     for (size_t i = 0; i < S->dinst.size(); ++i) {
         const DevPair& pr = S->dpairs[S->dcath[S->dinst[i].cathode].pair];
         const double v = 1.0 / std::sqrt((double)S->dcath[S->dinst[i].cathode].E_per_v2);
@@ -324,8 +326,17 @@ static sput_status pack_instances(sput_scene* S)
         const double t = x - j, K = c.x + t * (c.y + t * (c.z + t * c.w));
         const double inv_lambda = S->dinst[i].ng14 * (S->physics.gas_motion == SPUT_GAS_THERMAL ? K / v : K);
         S->mean_inv_lambda += inv_lambda * ((double)S->dinst[i].n / (double)std::max(1ull, S->n_tickets));
+        if (S->dinst[i].n) S->max_inv_lambda = std::max(S->max_inv_lambda, inv_lambda);
     }
     return SPUT_OK;
+}
+
+// the chamber's longest side, mm
+static double chamber_edge(const sput_scene* S)
+{
+    double edge = 0.0;
+    for (int a = 0; a < 3; ++a) edge = std::max(edge, S->chamber.box_hi[a] - S->chamber.box_lo[a]);
+    return edge;
 }
 
 // Whether the surface test by cell masks is the faster one.  It replaces the loop over the
@@ -341,9 +352,7 @@ static sput_status pack_instances(sput_scene* S)
 //                               38.5 -> 20.0; 1e5 atoms: 3 Pa 16.4 -> 8.8
 static bool cell_masks_pay(const sput_scene* S)
 {
-    double edge = 0.0;
-    for (int a = 0; a < 3; ++a) edge = std::max(edge, S->chamber.box_hi[a] - S->chamber.box_lo[a]);
-    return S->max_prims > 8 && S->max_prims * edge * S->mean_inv_lambda > 96.0;
+    return S->max_prims > 8 && S->max_prims * chamber_edge(S) * S->mean_inv_lambda > 96.0;
 }
 
 // Distance from a point to a primitive's surface (not to a chamber box's).
@@ -889,6 +898,42 @@ namespace {
 // atoms 1.86 / 1.85 / 1.81 / 1.81 ms, 64 primitives at 3 Pa 1e6 atoms 48.5 / 47.2 / 47.0 / 47.7 ms.
 constexpr int kDrainLive = 12;
 
+// Which atoms of a run of n go from transport_kernel to drain_kernel (Params::drain_live): none (0),
+// each warp's last ones (kDrainLive), or every one as soon as it is launched (32: the run fits the
+// pool).  The drain shortens the run's longest trajectory, whose steps number with the chamber's
+// side in free paths, x, and grow with ln n.  It costs a launch and a batch of flights drawn for
+// nothing per atom (30 us at least; 230 us for 1.5e5 atoms that land on their first flight), so it
+// needs long trajectories (in some instance), and all atoms only while they are few for its
+// groups of lanes against their trajectories (in the mean).
+// Measured on a GB300, none / last / all in us, single Ni:
+//             3000 atoms            3e4                  1e5                   1.5e5              4e5
+//   x = 0      37 /   42 /   62      39 /   43 /   90     47 /   49 /  169      53 /   56 /  228    60 /   66
+//   x = 3      86 /   80 /   73      91 /   91 /  107    115 /  128 /  189     127 /  150 /  250   160 /  184
+//   x = 6     141 /  107 /   84     186 /  124 /  124    202 /  155 /  212     223 /  189 /  271   293 /  226
+//   x = 18    587 /  239 /  194     714 /  314 /  290    872 /  424 /  468     987 /  492 /  576  1197 /  729
+//   x = 61   4232 / 1918 / 1067    5639 / 2867 / 1934   6934 / 3796 / 3534    8186 / 4701 / 4696  9615 / 6735
+// The lines below follow these, four targets with 16 primitives and one with 64 (x from 0 to 61,
+// 1 to 1e6 atoms): 1.01 times the fastest of the three on average, where the drain always, all
+// at once up to the pool's size, took 1.27 times it and up to 5.5 times it in vacuum.  The
+// diffusion shortcut shortens what is left of a trajectory (x counts 0.45; there 1e5 atoms take
+// 160 / 159 / 223 us at x = 12, 1036 / 500 / 697 us at x = 61).  With a gas at rest the drain has no
+// straight-line step (x counts 0.4), and slow atoms leave the deflection table for the scattering
+// integral, which the drain computes for every attempt: beyond x = 20 only few atoms gain (3e4
+// atoms at x = 12 561 / 351 / 344 us, x = 60 828 / 1134 / 1194 us).
+int hand_over(const sput_scene* S, unsigned long long n)
+{
+    const bool rest = S->physics.gas_motion != SPUT_GAS_THERMAL;
+    const bool integral = rest && S->physics.interaction == SPUT_INTERACTION_MOLIERE;
+    const double count = rest ? 0.4 : S->physics.thermal_switch_eV > 0.0 ? 0.45 : 1.0;
+    const double x = chamber_edge(S) * S->max_inv_lambda, y = count * x;
+    if (y * std::log1p((double)n) < 20.0) return 0;
+    if (n <= pool_atoms(S) && (double)n <= 3700.0 * count * chamber_edge(S) * S->mean_inv_lambda &&
+        !(integral && n > 20000))
+        return 32;
+    if (integral) return x >= 5.0 && x <= 20.0 ? kDrainLive : 0;
+    return y >= 4.0 ? kDrainLive : 0;
+}
+
 struct TallySizes {
     size_t counts, energy, score, prim_counts, timed_out, hist_E, hist_A, score_T;
 };
@@ -1000,14 +1045,13 @@ sput_status run_impl(sput_scene* S, const sput_run_opts* opts, cudaStream_t stre
     if (threads_out) *threads_out = threads;
     // the drain of the last atoms (drain_kernel); its pool belongs to the scene and is serialised
     // with the scene's scratch, so runs on another scratch do without
-    const bool drain = S->drain_bps > 0 && scratch == S->d_scratch;
+    const int drain_live = S->drain_bps > 0 && scratch == S->d_scratch ? hand_over(S, te - tb) : 0;
+    const bool drain = drain_live > 0;
     if (drain) {
         p.pool = S->d_pool;
         p.pool_count = reinterpret_cast<unsigned int*>(scratch + 2 + kNumStats);
         p.pool_next = p.pool_count + 8;
-        // a run that fits the pool goes to the drain as soon as its atoms are launched; of a larger
-        // one a warp hands over what it has left once its tickets are used up and few are alive
-        p.drain_live = te - tb <= pool_atoms(S) ? 32 : kDrainLive;
+        p.drain_live = drain_live;
     }
     CUDA_TRY(cudaEventRecord(S->ev0, stream));
     int le = transport_launch(p, blocks, threads, smem, stream);

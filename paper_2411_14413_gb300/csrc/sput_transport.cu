@@ -2117,9 +2117,11 @@ int instance_mode(const Params& p) { return p.score_T ? kModeScoreT : (p.E_switc
 
 #ifdef SPUT_CHECKED
 // For the tests of the checked library: which surface test the last run enqueued by this thread
-// took (words of its cell masks, 0: the counted loop).
-thread_local int t_mask_words = -1;
+// took (words of its cell masks, 0: the counted loop), and which atoms it handed to the drain
+// (Params::drain_live, 0: none).
+thread_local int t_mask_words = -1, t_drain_live = -1;
 extern "C" int sput_checked_mask_words() { return t_mask_words; }
+extern "C" int sput_checked_drain_live() { return t_drain_live; }
 #endif
 
 size_t drain_smem_bytes(const Params& p) { return drain_layout(p).total; }
@@ -2144,6 +2146,7 @@ int transport_launch(const Params& p, int blocks, int threads, size_t smem, void
 {
 #ifdef SPUT_CHECKED
     t_mask_words = p.cell_mask ? p.cell_words : 0;
+    t_drain_live = p.pool ? p.drain_live : 0;
 #endif
     kTransport[instance_mode(p)][p.cell_mask ? p.cell_words : 0]<<<blocks, threads, smem,
                                                                    reinterpret_cast<cudaStream_t>(stream)>>>(p);
