@@ -147,6 +147,7 @@ struct Params {
     const float4* rt_tab;              // racetrack inverse-CDF pieces (2 rt_n per cathode)
     const float* lt_tab;               // joint launch-table CDFs (see DevCathode::lt_off)
     const float4* chi_tab;             // deflection table: kChiCells cells of 4 float4 (null: hard spheres)
+    int usual;                         // collisions try the straight-line form first: a deflection table and a thermal gas
     // cell masks of the surface test (null: off): per geometry, cell of a uniform grid over the
     // chamber and level k, cell_words words with the local primitives (chamber boxes left out)
     // that have a point within r 2^k of a point of the cell

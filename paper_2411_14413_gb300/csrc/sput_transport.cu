@@ -1202,7 +1202,9 @@ __device__ int flight_step_warp(bool active, Lane& S, const Params& P, const Tab
         const Impact I = impact_draw(w);
         float ns = 0.0f, nx = 0.0f, ny = 0.0f, nz = 0.0f;
         bool usual = false;
-        if (P.chi_tab) usual = scatter<kMode, true>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, I);
+        // (in a gas at rest atoms slow down below the table and most collisions would be computed
+        // twice: 1e6 single-Ni atoms 3.08 ms without the first form, 3.33 with it)
+        if (P.usual) usual = scatter<kMode, true>(ns, nx, ny, nz, P, T, pr, vx, vy, vz, Vx, Vy, Vz, I);
         if (usual) {
             S.speed = ns;
             S.dx = nx;
@@ -1884,7 +1886,7 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
         uint32_t att = 0u;
         float V2 = 0.0f;
         const DevPair& pr = s_pairs[S.pair];
-        if (P.gas_thermal && P.chi_tab) drain_collisions<kMode, true>(S, F, P, T, W, pr, have, head, l, G, att, V2);
+        if (P.usual) drain_collisions<kMode, true>(S, F, P, T, W, pr, have, head, l, G, att, V2);
         else drain_collisions<kMode, false>(S, F, P, T, W, pr, have, head, l, G, att, V2);
 
         // ---------------------------------------------------- 3. flights
