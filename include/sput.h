@@ -317,7 +317,10 @@ sput_status sput_tally_layout_get(const sput_scene* scene, sput_tally_layout* ou
  * host synchronisation).  With stats != NULL it waits for the kernel (at most
  * opts->timeout_ms when > 0, else SPUT_ERR_TIMEOUT without touching the
  * device) and fills the counters.  Concurrent runs of one scene on different
- * streams race on the scene's scratch counters: serialise them. */
+ * streams race on the scene's scratch counters and its pool of handed-over
+ * atoms: serialise them.  (Overlapping runs give void results; an atom that
+ * finds no slot in the pool, or a slot that holds no atom of the run, is left out
+ * and sets bit 2 of device_status.) */
 sput_status sput_run(sput_scene* scene, const sput_run_opts* opts, void* stream, const sput_tallies* tallies,
                      sput_run_stats* stats);
 

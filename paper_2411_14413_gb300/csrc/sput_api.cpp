@@ -1050,6 +1050,7 @@ sput_status run_impl(sput_scene* S, const sput_run_opts* opts, cudaStream_t stre
     const bool drain = drain_live > 0;
     if (drain) {
         p.pool = S->d_pool;
+        p.pool_slots = (unsigned)pool_atoms(S);
         p.pool_count = reinterpret_cast<unsigned int*>(scratch + 2 + kNumStats);
         p.pool_next = p.pool_count + 8;
         p.drain_live = drain_live;

@@ -54,6 +54,7 @@ constexpr double kEnvM = 1.5957691216057308;
 enum : uint32_t {
     kStatusNonFinite = 1u << 0,   // a particle state became NaN/Inf; the particle was retired as timed out
     kStatusBadIndex = 1u << 1,    // a tally or table index fell outside its buffer; the write was skipped
+    kStatusHandOver = 1u << 2,    // the pool was full, or held other than this run's atoms (overlapping runs of a scene)
 };
 
 // One primitive, 80 bytes; n = u x v precomputed; (bx, by, bz, br) bounds it.
@@ -202,6 +203,7 @@ struct Params {
     unsigned int* status;
     // atoms handed over from transport_kernel to drain_kernel (null: none), 4 float4 each
     float4* pool;
+    unsigned int pool_slots;           // atoms that the pool holds
     unsigned int* pool_count;          // atoms in the pool (zeroed before the run)
     unsigned int* pool_next;           // next atom to take (zeroed before the run)
     int drain_live;                    // a warp without tickets hands its atoms over from this many on (32: at once)
