@@ -770,6 +770,7 @@ sput_status sput_scene_create(const sput_scene_desc* desc, int device, sput_scen
     p.chi_tab = ct ? reinterpret_cast<const float4*>(S->d_blob + S->off_chi) : nullptr;
     p.usual = ct && thermal;
     p.cell_mask = S->cell_masks.empty() ? nullptr : reinterpret_cast<const uint32_t*>(S->d_blob + S->off_cell);
+    p.n_cell_words = (long long)S->cell_masks.size();
     p.cell_words = S->cell_words;
     p.cell_half = S->max_prims <= 16;
     for (int a = 0; a < 3; ++a) {

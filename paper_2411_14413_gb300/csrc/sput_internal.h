@@ -153,6 +153,7 @@ struct Params {
     // chamber and level k, cell_words words with the local primitives (chamber boxes left out)
     // that have a point within r 2^k of a point of the cell
     const uint32_t* cell_mask;
+    long long n_cell_words;            // entries of cell_mask (bound of the checked build)
     int cell_words;
     int cell_half;  // masks of 16 bits (at most 16 primitives): half the footprint in L1
     float cell_off[3], cell_inv_h, cell_inv_r, cell_inv_seg;  // (cell_off = -lower corner / h)

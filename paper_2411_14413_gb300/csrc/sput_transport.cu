@@ -750,7 +750,10 @@ __device__ __forceinline__ void nearest_hit_masks(bool active, const Lane& S, co
                 const int cell = (int)((iz * P.cell_n[1] + iy) * P.cell_n[0] + ix);
                 const uint32_t* m = P.cell_mask + G.cell_base;
                 const int e = cell * kCellLevels + k;
-                if (kWords == 1) {
+                if (!idx_ok(P.status, G.cell_base + (P.cell_half ? (long long)e / 2 : (long long)kWords * e + kWords - 1),
+                            P.n_cell_words)) {
+                    // (the checked build reports it)
+                } else if (kWords == 1) {
                     lo |= P.cell_half ? __ldg(reinterpret_cast<const unsigned short*>(m) + e) : __ldg(m + e);
                 } else {
                     const uint2 m2 = __ldg(reinterpret_cast<const uint2*>(m) + e);
@@ -2156,8 +2159,12 @@ extern "C" void sput_checked_overlap(unsigned taken, unsigned room, int byte)
     t_pool_room = room;
     t_pool_byte = byte;
 }
-static Params overlapped(Params p)
+// and how many words of its cell masks the runs of this thread may read (-1: all)
+thread_local long long t_mask_limit = -1;
+extern "C" void sput_checked_mask_limit(long long words) { t_mask_limit = words; }
+static Params for_test(Params p)
 {
+    if (t_mask_limit >= 0 && t_mask_limit < p.n_cell_words) p.n_cell_words = t_mask_limit;
     if (t_pool_room && p.pool && t_pool_taken + t_pool_room <= p.pool_slots) p.pool_slots = t_pool_taken + t_pool_room;
     return p;
 }
@@ -2185,7 +2192,7 @@ int transport_launch(const Params& run, int blocks, int threads, size_t smem, vo
 {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
 #ifdef SPUT_CHECKED
-    const Params p = overlapped(run);
+    const Params p = for_test(run);
     t_mask_words = p.cell_mask ? p.cell_words : 0;
     t_drain_live = p.pool ? p.drain_live : 0;
     if (p.pool && p.pool_slots != run.pool_slots) {
@@ -2202,7 +2209,7 @@ int transport_launch(const Params& run, int blocks, int threads, size_t smem, vo
 int drain_launch(const Params& run, int blocks, size_t smem, void* stream)
 {
 #ifdef SPUT_CHECKED
-    const Params p = overlapped(run);
+    const Params p = for_test(run);
     t_pool_room = 0;
 #else
     const Params& p = run;

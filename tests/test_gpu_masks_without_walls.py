@@ -78,3 +78,19 @@ def test_default():
     last = out.prims[-1]
     out.box_hi = tuple(float(x) for x in out.box_hi[:2]) + (float(last["center"][2]),)
     assert _checked_run(out) == (0, 0)
+
+
+@pytest.mark.parametrize("n_prims", [16, 32, 63])
+def test_mask_reads_are_checked(n_prims):
+    """The bounds-checked library reports a mask index behind the masks' end."""
+    from paper_2411_14413_gb300 import _native as N
+
+    lib = N.load(path=N.CHECKED_LIB_PATH)
+    lib.sput_checked_mask_limit.argtypes = [C.c_longlong]
+    sc = _scene(n_prims, 0.3, n=2000)
+    try:
+        lib.sput_checked_mask_limit(1000)
+        assert _checked_run(sc, N.SPUT_RUN_CELL_MASKS)[0] == 2
+    finally:
+        lib.sput_checked_mask_limit(-1)
+    assert _checked_run(sc, N.SPUT_RUN_CELL_MASKS)[0] == 0
