@@ -280,7 +280,7 @@ typedef struct sput_run_stats {
     uint32_t device_status;      /* bit mask of device checks, 0 = clean */
     uint32_t grid_blocks;        /* launch shape that ran */
     uint32_t block_threads;
-    float kernel_ms;             /* device time of the transport kernel (CUDA events) */
+    float kernel_ms;             /* device time of the transport and the drain (CUDA events) */
 } sput_run_stats;
 
 /* Library version (SPUT_ABI_VERSION) and status text. */
@@ -365,12 +365,14 @@ sput_status sput_run_noalloc(sput_scene* scene, const sput_run_opts* opts, void*
  * ticket chunk, shared-memory counters) on `sample_tickets` tickets taken as
  * four equal ranges spread over the scene's ticket space, and keep the fastest
  * (most collisions per second of kernel time) as the scene default for runs
- * whose opts leave those fields 0.  Uses `tallies` as scratch output (their
- * contents are overwritten).  Synchronous.  The results of every candidate are
- * reported in *out. */
+ * whose opts leave those fields 0.  The shapes are those of the transport kernel, and
+ * its time is what is compared: the drain of the last atoms, whose shape is fixed, is
+ * left out of it, and a sample small enough to go to the drain as a whole is
+ * transported.  Uses `tallies` as scratch output (their contents are overwritten).
+ * Synchronous.  The results of every candidate are reported in *out. */
 typedef struct sput_tune_result {
     int block_threads, blocks_per_sm, ticket_chunk, flags; /* the chosen shape */
-    float best_rate;             /* collisions per second of kernel time on the sample */
+    float best_rate;             /* the sample's collisions per second of the transport kernel's time */
     int n_candidates;
     int reserved;
     int cand_threads[32], cand_bps[32], cand_chunk[32], cand_flags[32];
@@ -381,9 +383,9 @@ sput_status sput_autotune(sput_scene* scene, const sput_run_opts* base, void* st
                           uint64_t sample_tickets, sput_tune_result* out);
 
 /* CUDA graph of one run (tally clearing when opts->accumulate == 0, scratch
- * clearing and the transport kernel), captured on `stream` and instantiated.
- * sput_graph_launch replays it on `stream` with a new seed (the kernel node's
- * parameters are updated in the executable graph).  The graph keeps the
+ * clearing, the transport kernel and, where the run has one, the drain of its last
+ * atoms), captured on `stream` and instantiated.  sput_graph_launch replays it on
+ * `stream` with a new seed (the kernel nodes' parameters are updated in the executable graph).  The graph keeps the
  * tally pointers and ticket range it was made with.  The scene must outlive
  * the graph; a run or launch of the scene must not overlap another. */
 typedef struct sput_graph sput_graph;
