@@ -1982,6 +1982,14 @@ __global__ void __launch_bounds__(kDrainThreads, 2) drain_kernel(const Params P)
 }
 
 // ------------------------------------------------------------- probes
+template <int kMode>
+__device__ int trace_step(int words, bool active, Lane& S, const Params& P, const TableView& T, WarpScratch* ws, StepOut& out)
+{
+    return words == 0   ? flight_step_warp<kMode, 0>(active, S, P, T, P.prims, P.pairs, ws, out)
+           : words == 1 ? flight_step_warp<kMode, 1>(active, S, P, T, P.prims, P.pairs, ws, out)
+                        : flight_step_warp<kMode, 2>(active, S, P, T, P.prims, P.pairs, ws, out);
+}
+
 __global__ void probe_kernel(const Params P, int what, int idx, int n, const double* x, double* y)
 {
     __shared__ float4 s_gm[kGMHalf + kGMHalfLo];
@@ -2026,10 +2034,11 @@ __global__ void probe_kernel(const Params P, int what, int idx, int n, const dou
         for (int r = 1; r < kTraceRows; ++r) {
             if (!__any_sync(kFull, running)) break;
             StepOut so;
-            // (the oracle's trace tests the counted loop; both surface tests give the same flights)
-            const int status = P.E_switch > 0.0f
-                                   ? flight_step_warp<kModeWalk, 0>(running, S, P, T, P.prims, P.pairs, &s_ws[threadIdx.x >> 5], so)
-                                   : flight_step_warp<kModePlain, 0>(running, S, P, T, P.prims, P.pairs, &s_ws[threadIdx.x >> 5], so);
+            // (the surface test of the scene's masks where it has them, whatever a run would choose)
+            WarpScratch* ws = &s_ws[threadIdx.x >> 5];
+            const int words = P.cell_mask ? P.cell_words : 0;
+            const int status = P.E_switch > 0.0f ? trace_step<kModeWalk>(words, running, S, P, T, ws, so)
+                                                 : trace_step<kModePlain>(words, running, S, P, T, ws, so);
             if (running) {
                 double* q = o + (size_t)r * 10;
                 float px = S.px, py = S.py, pz = S.pz;

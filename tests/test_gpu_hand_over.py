@@ -74,3 +74,35 @@ def test_same_results(pressure, n):
     for f in ("particles", "landed", "timed_out", "flights", "collisions", "attempts"):
         assert getattr(st_a, f) == getattr(st_b, f), f
     tr.close()
+
+
+@pytest.mark.parametrize("mode", ["plain", "score_T", "walk"])
+@pytest.mark.parametrize("name", ["single_ni", "quaternary", "large"])
+def test_atoms_on_their_way(name, mode):
+    """More atoms than the pool holds: what a warp hands over has flights, scores and, with the
+    diffusion shortcut, the walk behind it.  Seven primitives (the loop), 16 and 64 (masks of one and
+    two words)."""
+    import torch
+
+    import paper_2411_14413_gb300 as pkg
+    from paper_2411_14413_gb300 import api
+
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 1024 + 1
+    kw = {"n_per_cathode": n // 4 + 1} if name == "quaternary" else {"n": n}
+    kw["physics"] = {"thermal_switch_eV": 0.1} if mode == "walk" else {}
+    sc = workloads.scene_by_name(name, pressure=0.6, **kw)
+    assert _choice(sc) == LAST
+    tr = pkg.Transport(sc, records=True, energy=True, score=True, score_T=mode == "score_T")
+    stream = torch.cuda.current_stream().cuda_stream
+    st_a = api.sput_run_noalloc(tr.h, api.run_opts(seed=29), stream, tr._tal)
+    want = {k: v.clone() for k, v in tr.t.items()}
+    tr.t["records"].fill_(7)
+    st_b = api.sput_run(tr.h, api.run_opts(seed=29), stream, tr._tal)
+    for k, v in tr.t.items():
+        if v.dtype == torch.float64:
+            assert torch.allclose(want[k], v, rtol=1e-12, atol=1e-12 * float(want[k].abs().max() + 1e-300)), k
+        else:
+            assert torch.equal(want[k], v), k
+    for f in ("particles", "landed", "timed_out", "flights", "collisions", "attempts"):
+        assert getattr(st_a, f) == getattr(st_b, f), f
+    tr.close()
