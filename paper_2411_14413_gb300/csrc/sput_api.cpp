@@ -1041,7 +1041,7 @@ sput_status run_impl(sput_scene* S, const sput_run_opts* opts, cudaStream_t stre
         p.block_warps = threads / 32;
     }
     const size_t smem = transport_smem_bytes(p);
-    int bps = transport_max_blocks_per_sm(threads, smem);
+    int bps = transport_blocks_per_sm(p, threads, smem);
     if (bps < 1) return fail(SPUT_ERR_UNSUPPORTED, "launch shape does not fit on an SM");
     if (bps_req > 0) bps = std::min(bps, bps_req);
     unsigned long long need = (te - tb + threads - 1) / threads;

@@ -235,7 +235,9 @@ constexpr int kDrainThreads = 256;
 int drain_launch(const Params& p, int blocks, size_t smem, void* stream);
 size_t drain_smem_bytes(const Params& p);
 int drain_max_blocks_per_sm(size_t smem);
+// resident blocks per SM: the fewest of all instances, and of the one that p launches
 int transport_max_blocks_per_sm(int threads, size_t smem);
+int transport_blocks_per_sm(const Params& p, int threads, size_t smem);
 int probe_launch(const Params& p, int what, int idx, int n, const double* x_dev, double* y_dev, void* stream);
 
 // Device copy of the scene's instance table (for the adjoint kernels).

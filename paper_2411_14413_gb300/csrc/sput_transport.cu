@@ -2183,6 +2183,14 @@ size_t drain_smem_bytes(const Params& p) { return drain_layout(p).total; }
 
 int transport_max_blocks_per_sm(int threads, size_t smem) { return min_blocks_per_sm(kTransport, threads, smem); }
 
+int transport_blocks_per_sm(const Params& p, int threads, size_t smem)
+{
+    int nb = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &nb, kTransport[instance_mode(p)][p.cell_mask ? p.cell_words : 0], threads, smem);
+    return e == cudaSuccess ? nb : 0;
+}
+
 int drain_max_blocks_per_sm(size_t smem) { return min_blocks_per_sm(kDrain, kDrainThreads, smem); }
 
 int transport_configure(int max_dynamic_smem)
