@@ -303,7 +303,10 @@ static sput_status pack_instances(sput_scene* S)
         D.cathode = I.cathode;
         D.n = (uint32_t)I.n_particles;
         // n_g = p / (k_B T) in m^-3 -> mm^-3 (1e-9); sigma in A^2 -> mm^2 (1e-14)
+        // (below 1e-37, 4e-35 Pa, no gas: the inverse mean free path would be a denormal number, by
+        // which the kernel does not divide)
         D.ng14 = (float)(I.pressure / kT * 1e-9 * 1e-14);
+        if (D.ng14 < 1e-37f) D.ng14 = 0.0f;
         D.thompson_q = (float)(Em / (Em + C.U_s));
         D.U_s = (float)C.U_s;
         D.kLambda = (float)(I.k * 4.0 * S->chamber.gas_mass * C.mass /
