@@ -89,12 +89,17 @@ WORK_MODEL = {"philox_block": PHILOX_BLOCK_OPS, "flight": OPS_PER_FLIGHT, "prim_
 # drain kernels (ncu smsp__thread_inst_executed.sum / collisions of one run, small
 # case of the workload); the issue share is reported beside the algorithmic
 # fraction.  None = no capture of the current build.
-EXEC_LANE_INSTR_PER_COLLISION = {"quaternary": 1316.0, "large": 1312.0}
+EXEC_LANE_INSTR_PER_COLLISION = {"quaternary": 1312.0, "large": 1308.0}
 # DRAM bytes (read + write) of one run of the quaternary workload, from the
-# one-pass capture of the current kernels (transport 4.15 MB read and 0.23 MB
-# written, drain 4.88 MB read, mean of 3 runs); None whenever a kernel changed
-# after the capture.
-TRAFFIC_PER_LAUNCH = 9.26e6
+# one-pass capture of the current kernels (transport 4.32 MB, drain 4.93 MB, all
+# of it read, mean of 3 runs); None whenever a kernel changed after the capture.
+TRAFFIC_PER_LAUNCH = 9.25e6
+# Surface tests per flight that the cell masks leave (the chamber walls, and the
+# primitives within reach of the flight, counted once on a small case): the work
+# model charges one per primitive of the geometry, as the method without masks
+# needs, so its fraction counts work that the kernel does not do.  Beside it the
+# line gives the fraction with these tests only (the mask lookup not counted).
+TESTS_PER_FLIGHT = {"quaternary": 1.31, "sweep": 1.14, "large": 1.21}
 
 
 def log(*a):
@@ -272,7 +277,7 @@ def measure_peaks(torch, api, dev, n_slots):
     return out
 
 
-def roofline_entry(stats_list, kernel_ms, prims, peaks, exec_per_coll=None, traffic=None):
+def roofline_entry(stats_list, kernel_ms, prims, peaks, exec_per_coll=None, traffic=None, tests=None):
     """Algorithmic lane-op roofline of the transport kernel over a list of runs."""
     ops = statistics.mean(algorithmic_lane_ops(s, prims) for s in stats_list)
     coll = statistics.mean(s["collisions"] for s in stats_list)
@@ -284,6 +289,10 @@ def roofline_entry(stats_list, kernel_ms, prims, peaks, exec_per_coll=None, traf
          "peak_basis": "measured FP32 FMA lane-op rate of this GPU in this run (sput_microbench ffma)",
          "algorithmic_lane_ops_per_launch": ops, "algorithmic_lane_ops_per_collision": ops / max(1.0, coll),
          "prims_per_flight": prims, "work_model": WORK_MODEL}
+    if tests is not None:
+        left = statistics.mean(algorithmic_lane_ops(s, tests) for s in stats_list)
+        e["tests_per_flight"] = tests
+        e["frac_with_tests_made"] = left / t / peaks["ffma"]
     if exec_per_coll is not None:
         e["executed_lane_instr_per_collision"] = exec_per_coll
         e["issue_frac"] = exec_per_coll * coll / t / peaks["ffma"]
@@ -412,7 +421,8 @@ def run_ours(args, rank, world, local_rank):
     value = coll_all / (total_ms_all / 1e3)
     prims = mean_prims(sc)
     traffic = TRAFFIC_PER_LAUNCH if (args.workload == "quaternary" and args.particles == 10_000_000) else None
-    roof = roofline_entry(stats, kernel_ms, prims, peaks, EXEC_LANE_INSTR_PER_COLLISION.get(args.workload), traffic)
+    roof = roofline_entry(stats, kernel_ms, prims, peaks, EXEC_LANE_INSTR_PER_COLLISION.get(args.workload), traffic,
+                          TESTS_PER_FLIGHT.get(args.workload))
     # landing tally: per substrate-grid landing one int64 count and one fp64 energy reduction
     t_kernel = statistics.mean(kernel_ms) / 1e3
     red_i = grid_landings
@@ -580,7 +590,7 @@ def sub_sweep(args, torch, pkg, api, workloads, dev, peaks):
     ms = e0.elapsed_time(e1)
     plain = plain_per_instance(torch, tr, sc, 7, stream, flush, st["collisions"], batched=tr.t["counts"].clone())
     tr.close()
-    roof = roofline_entry([st], [st["kernel_ms"]], mean_prims(sc), peaks)
+    roof = roofline_entry([st], [st["kernel_ms"]], mean_prims(sc), peaks, tests=TESTS_PER_FLIGHT["sweep"])
     return {"workload": WORKLOADS["sweep"], "particle_scale": scale, "particles": sc.total_particles,
             "value": st["collisions"] / (ms / 1e3), "unit": UNIT, "landed_per_s": st["landed"] / (ms / 1e3),
             "ms": ms, "plain_per_instance": plain, "batched_over_plain": plain["ms"] / ms,
@@ -603,7 +613,8 @@ def sub_large(args, torch, pkg, api, workloads, dev, peaks):
     torch.cuda.synchronize(dev)
     ms = e0.elapsed_time(e1)
     tr.close()
-    roof = roofline_entry([st], [st["kernel_ms"]], mean_prims(sc), peaks, EXEC_LANE_INSTR_PER_COLLISION.get("large"))
+    roof = roofline_entry([st], [st["kernel_ms"]], mean_prims(sc), peaks, EXEC_LANE_INSTR_PER_COLLISION.get("large"),
+                          tests=TESTS_PER_FLIGHT["large"])
     return {"workload": WORKLOADS["large"], "particles": n, "particle_scale": n / 1e9,
             "value": st["collisions"] / (ms / 1e3), "unit": UNIT, "landed_per_s": st["landed"] / (ms / 1e3),
             "ms": ms, "collisions_per_particle": st["collisions"] / n,
