@@ -79,7 +79,7 @@ __device__ double cluster_sum(double x, double* part)
 }
 
 // grad[i] = sum_c g[i][c] * score[i][c], one cluster per instance.  16 bytes per cell; at 4 x 40000
-// cells bound by latency: 31 us with one block of 256 threads per instance, 5 us so.
+// cells bound by latency: 31 us with one block of 256 threads per instance, 7.5 us so (under ncu).
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kReduceThreads)
     lr_backward_kernel(const double* g, const double* score, double* grad, long long n_cells)
 {
@@ -182,7 +182,7 @@ __global__ void composition_kernel(const double* N, double* comp, CompParams cp)
 // a_j(m) depends on N_j(m), on N_j(ref) through 1/N_j(ref) and on R_j linearly, so with
 // S_j = sum_m a_j dL/da_j: dL/dN_j(ref) gets -S_j / N_j(ref) and dL/dR_j = S_j / R_j.
 // One block added 2 n_cath values per point with FP64 atomics on a handful of shared-memory
-// words: 95 us for 342 points and four cathodes; so 7 us.
+// words: 95 us for 342 points and four cathodes; so 15 us (under ncu).
 __global__ void __cluster_dims__(kCluster, 1, 1)
     composition_backward_kernel(const double* N, const double* gc, double* gN, double* gP, CompParams cp)
 {

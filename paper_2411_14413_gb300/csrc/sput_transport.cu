@@ -702,7 +702,7 @@ __device__ __forceinline__ unsigned grid_clamp(float x, int n)
 // (lowest index) are those of the loop above.  kWords: 32-bit words of a mask.
 // The transport is bound by instruction issue, and the loop took 43 % (16 primitives, 0.5 Pa)
 // to 67 % (64 primitives, 3 Pa) of the kernel: a warp ran 9.2 of 16 primitives' tests per
-// step although 0.12 per atom cross the primitive at all.  Masks of the midpoint leave 13
+// step although 0.12 per atom cross the primitive at all.  Masks of the midpoint leave 8
 // pairs per warp and step (0.5 Pa), so one round does.  Measured loop -> masks (GB300, before
 // what followed): quaternary 4e7 atoms 67.2 -> 58.8 ms, 64 primitives at 3 Pa 1e6 atoms
 // 118 -> 59 ms, with the diffusion shortcut 4e6 atoms 61.3 -> 24.7 ms.
@@ -1615,10 +1615,9 @@ __global__ void __launch_bounds__(256, 4) transport_kernel(const Params P)
 // single-lane step, so the results are bit-identical.
 // Bound by the latency of the chain, 1200 cycles (0.6 us) per step, a third of it waiting for the
 // deflection table in L1 or L2.  Measured on a GB300 without and with the drain when it came:
-// single Ni 3e3 atoms 1.8 -> 0.53 ms (now 0.34), 1e5 2.4 -> 1.26 ms (0.90), quaternary 4e5
-// 3.0 -> 1.8 ms (1.4), 64 primitives at 3 Pa 1e6 atoms 59 -> 47 ms (38).  Runs of 3e4 single-Ni
-// atoms took 0.74 ms when they went to it at once, 0.95 ms when only the last atoms of each
-// warp did; from 1.5e5 atoms on (one per lane of the GPU) the two met.
+// single Ni 3e3 atoms 1.8 -> 0.53 ms (now 0.35), 1e5 2.4 -> 1.26 ms (0.91), quaternary 4e5
+// 3.0 -> 1.8 ms (1.3), 64 primitives at 3 Pa 1e6 atoms 59 -> 47 ms (38).  Which atoms of a run
+// come here: hand_over in sput_api.cpp.
 constexpr int kDrawn = 4;
 constexpr int kMinGroupLog2 = 3;
 
